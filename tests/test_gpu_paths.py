@@ -1,0 +1,55 @@
+"""GPU tests of the kernels' variants at the sizes where they can go wrong, against the CPU oracle
+or a plain 64-bit reference."""
+import numpy as np
+import pytest
+
+from paper_1504_01883_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def B():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1504_01883_gb300 import _build, binding
+    _build.build()
+    return binding
+
+
+@pytest.fixture(scope="module")
+def ctx(B):
+    c = B.Context(0)
+    yield c
+    c.close()
+
+
+from gpu_util import dev_f32, dev_u16, dev_u8, host_u16, rbf_error_scale, rel_score_error  # noqa: E402,F401
+
+
+@pytest.mark.parametrize("shape", [(37, 45), (64, 31), (480, 640)])
+@pytest.mark.parametrize("colour_w", [640, 20000])
+@pytest.mark.parametrize("density", [0.0, 0.002, 0.9])
+def test_face_roi_scan_from_the_edges(B, ctx, orc, shape, colour_w, density):
+    """The region scan reads a window from its edges inwards: frames that are empty, nearly empty
+    (few pixels, anywhere) and dense, windows of less than one strip of rows or columns, depths at
+    both ends of the valid range, and colour images too wide for 32-bit coordinates."""
+    H, W = shape
+    rng = synth.rng_for(H + colour_w + int(1000 * density))
+    depth = rng.choice(np.array([399, 400, 401, 1000, 3000, 7999, 8000, 8001, 65535], np.uint16), (3, H, W))
+    depth[rng.random((3, H, W)) >= density] = 0
+    boxes = np.zeros(60, orc.RECT_DTYPE)
+    boxes["frame"] = rng.integers(0, 3, 60)
+    boxes["x"], boxes["y"] = rng.integers(-20, W + 40, 60), rng.integers(-20, H + 10, 60)
+    boxes["w"], boxes["h"] = rng.integers(1, W + 20, 60), rng.integers(1, H + 20, 60)
+    cal = synth.calibration(rng, colour_w, H)
+    for flip in (1, -1):  # a mirrored mapping too
+        cal["a"][0] *= flip
+        cal["a"][2] = 0 if flip > 0 else 65536 * W
+        want = orc.face_roi(depth, cal, boxes)
+        got = B.rgbd_face_roi(ctx, dev_u16(depth), B.Calib.from_record(cal), B.rects_tensor(boxes)).cpu().numpy()
+        for i, f in enumerate(["frame", "x", "y", "w", "h"]):
+            assert (got[:, i] == want[f]).all(), (flip, f)
+    ctx.status(clear=True)
