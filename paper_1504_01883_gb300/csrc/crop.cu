@@ -1,0 +1,219 @@
+// crop.cu -- A1 alone (rgbd_crop_affine; Section 2.1, Eq. 1): face rects resampled into crops that
+// are written out, for callers that want the faces themselves.
+#include <algorithm>
+
+#include "internal.h"
+#include "resample.cuh"
+
+namespace rgbd {
+namespace {
+
+constexpr int kCropThreads = 256;
+
+struct CropArgs {
+    const uint8_t* grey;
+    const uint16_t* depth;
+    int n_frames, H, W;
+    const rgbd_rect* rects;
+    const int32_t* affine;
+    int n, oh, ow;
+    int ow4;        // groups of 4 columns
+    int rows;       // crop rows per CTA
+    int lanes_log2; // lanes of a warp on one row
+    int wide;       // 4-byte grey and 8-byte depth stores are aligned
+    uint8_t* og;
+    uint16_t* od;
+    uint32_t* status;
+};
+
+__device__ __forceinline__ void store_group(const CropArgs& a, size_t o, int u, uint32_t gw, uint32_t d01,
+                                            uint32_t d23) {
+    if (a.wide) {
+        *reinterpret_cast<uint32_t*>(a.og + o) = gw;
+        *reinterpret_cast<uint2*>(a.od + o) = make_uint2(d01, d23);
+        return;
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        if (u + e < a.ow) {
+            a.og[o + e] = (uint8_t)(gw >> (8 * e));
+            a.od[o + e] = (uint16_t)((e < 2 ? d01 : d23) >> (16 * (e & 1)));
+        }
+}
+
+// One CTA per (strip of crop rows, rect).  The taps of every column and of the strip's rows are
+// computed once into shared memory (a 64-bit division each: one per pixel and axis is what bound
+// this step before), and a thread makes 4 neighbouring pixels and stores them in two words.  For
+// rects at most twice as wide as the crop the four grey taps of a column pair lie in one aligned
+// 8-byte window of a source row, so a pair costs two 32-bit loads per row and each horizontal
+// interpolation is a byte permute and a 4-way byte dot product.  Bound by the gathers through L1,
+// with HBM behind (frames in once, crops out once).  4096 rects of side 48..256 over 256 frames
+// of 640x480 -> 128x128: 570 us with a thread and two divisions per pixel, 120 us now.
+__global__ void __launch_bounds__(kCropThreads) crop_rect_kernel(const CropArgs a) {
+    extern __shared__ __align__(16) unsigned char crop_smem[];
+    uint4* cm = reinterpret_cast<uint4*>(crop_smem);                  // [2][ow4]: taps of a column pair
+    uint32_t* nn = reinterpret_cast<uint32_t*>(cm + 2 * a.ow4);       // [2][ow4]: its nearest columns
+    uint2* rm = reinterpret_cast<uint2*>(nn + 2 * a.ow4);             // [rows]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int v0 = blockIdx.x * a.rows, v1 = min(a.oh, v0 + a.rows);
+    const int lpr = 1 << a.lanes_log2, rpw = 32 >> a.lanes_log2;      // lanes per row, rows per warp
+    const int ql = lane & (lpr - 1), vl = v0 + warp * rpw + (lane >> a.lanes_log2);
+    const int vstep = (kCropThreads / 32) * rpw;
+    for (int k = blockIdx.y; k < a.n; k += gridDim.y) {
+        const rgbd_rect r = a.rects[k];
+        const size_t crop0 = (size_t)k * a.oh * a.ow;
+        const bool ok = r.frame >= 0 && r.frame < a.n_frames && r.w > 0 && r.h > 0;
+        if (!ok) {
+            for (int v = vl; v < v1; v += vstep)
+                for (int q = ql; q < a.ow4; q += lpr)
+                    store_group(a, crop0 + (size_t)v * a.ow + 4 * q, 4 * q, 0u, 0u, 0u);
+            if (blockIdx.x == 0 && tid == 0) atomicOr(a.status, RGBD_STATUS_BAD_RECT);
+            continue;
+        }
+        const uint8_t* gsrc = a.grey + (size_t)r.frame * a.H * a.W;
+        const uint16_t* dsrc = a.depth + (size_t)r.frame * a.H * a.W;
+        const bool pair_win = r.w <= 2 * a.ow && (a.W & 3) == 0 && a.W >= 8 &&
+                              (reinterpret_cast<size_t>(a.grey) & 3) == 0;
+        __syncthreads();  // the taps of the rect before are no longer read
+        for (int i = tid; i < 2 * a.ow4 + (v1 - v0); i += kCropThreads) {
+            if (i < 2 * a.ow4) {  // columns 2i, 2i + 1 (past the crop's edge: its last column again)
+                const uint2 t0 = make_tap(rect_coord_q16(r.x, r.w, a.ow, min(2 * i, a.ow - 1)), a.W);
+                const uint2 t1 = make_tap(rect_coord_q16(r.x, r.w, a.ow, min(2 * i + 1, a.ow - 1)), a.W);
+                uint4 c = make_uint4(t0.x, 0u, t1.x, 0u);
+                if (pair_win) {
+                    // .x / .z = byte selector (o, o + dx, o) of each column in the window that starts at
+                    // byte wb (kept above .x's selector), .y / .w = byte weights (255 - fx, fx, 1, 0):
+                    // a permute and a dot product give 256 p(o) + fx (p(o + dx) - p(o)).  Neighbouring
+                    // taps are at most 2 apart, so every offset is at most 7.
+                    const uint32_t wb = min(t0.x & 0xFFFCu, (uint32_t)a.W - 8u);
+                    auto sel = [&](uint32_t t) {
+                        const uint32_t o = (t & 0xFFFFu) - wb, od = o + ((t >> 16) & 1u);
+                        return o | (od << 4) | (o << 8);
+                    };
+                    auto wts = [](uint32_t t) { return (255u - (t >> 24)) | ((t >> 24) << 8) | (1u << 16); };
+                    c = make_uint4(sel(t0.x) | (wb << 16), wts(t0.x), sel(t1.x), wts(t1.x));
+                }
+                const int at = (i & 1) * a.ow4 + (i >> 1);
+                cm[at] = c;
+                nn[at] = t0.y | (t1.y << 16);
+            } else {
+                const int v = i - 2 * a.ow4;
+                rm[v] = make_tap(rect_coord_q16(r.y, r.h, a.oh, v0 + v), a.H);
+            }
+        }
+        __syncthreads();
+        for (int v = vl; v < v1; v += vstep) {
+            const uint2 ry = rm[v - v0];
+            const uint32_t fy = ry.x >> 24;
+            const uint8_t* g0 = gsrc + (size_t)(ry.x & 0xFFFFu) * a.W;
+            const uint8_t* g1 = g0 + (size_t)((ry.x >> 16) & 1u) * a.W;
+            const uint16_t* drow = dsrc + (size_t)ry.y * a.W;
+            for (int q = ql; q < a.ow4; q += lpr) {
+                uint32_t acc[4], dv[4];  // acc: the grey value in byte 2
+#pragma unroll
+                for (int e2 = 0; e2 < 2; ++e2) {
+                    const uint4 c = cm[e2 * a.ow4 + q];
+                    const uint32_t cols = nn[e2 * a.ow4 + q];
+                    if (pair_win) {
+                        const uint32_t* w0 = reinterpret_cast<const uint32_t*>(g0 + (c.x >> 16));
+                        const uint32_t* w1 = reinterpret_cast<const uint32_t*>(g1 + (c.x >> 16));
+                        const uint32_t a0 = __ldg(w0), a1 = __ldg(w0 + 1), b0 = __ldg(w1), b1 = __ldg(w1 + 1);
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            const uint32_t h0 = __dp4a(__byte_perm(a0, a1, j ? c.z : c.x), j ? c.w : c.y, 0u);
+                            const uint32_t h1 = __dp4a(__byte_perm(b0, b1, j ? c.z : c.x), j ? c.w : c.y, 0u);
+                            acc[2 * e2 + j] = h0 * (256u - fy) + (h1 * fy + 32768u);
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            const uint32_t t = j ? c.z : c.x;
+                            const uint32_t xa = t & 0xFFFFu, dx = (t >> 16) & 1u, fx = t >> 24;
+                            const uint32_t h0 = (256u - fx) * __ldg(g0 + xa) + fx * __ldg(g0 + xa + dx);
+                            const uint32_t h1 = (256u - fx) * __ldg(g1 + xa) + fx * __ldg(g1 + xa + dx);
+                            acc[2 * e2 + j] = h0 * (256u - fy) + (h1 * fy + 32768u);
+                        }
+                    }
+                    dv[2 * e2] = __ldg(drow + (cols & 0xFFFFu));
+                    dv[2 * e2 + 1] = __ldg(drow + (cols >> 16));
+                }
+                const uint32_t gw = __byte_perm(__byte_perm(acc[0], acc[1], 0x0062u),
+                                                __byte_perm(acc[2], acc[3], 0x0062u), 0x5410u);
+                store_group(a, crop0 + (size_t)v * a.ow + 4 * q, 4 * q, gw, dv[0] | (dv[1] << 16),
+                            dv[2] | (dv[3] << 16));
+            }
+        }
+    }
+}
+
+// The same split of the work for a general affine map: source points by 64-bit products per pixel.
+__global__ void __launch_bounds__(kCropThreads) crop_affine_kernel(const CropArgs a) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int v0 = blockIdx.x * a.rows, v1 = min(a.oh, v0 + a.rows);
+    const int lpr = 1 << a.lanes_log2, rpw = 32 >> a.lanes_log2;
+    const int ql = lane & (lpr - 1), vl = v0 + warp * rpw + (lane >> a.lanes_log2);
+    for (int k = blockIdx.y; k < a.n; k += gridDim.y) {
+        const rgbd_rect r = a.rects[k];
+        const bool ok = r.frame >= 0 && r.frame < a.n_frames && r.w > 0 && r.h > 0;
+        if (!ok && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.status, RGBD_STATUS_BAD_RECT);
+        int64_t m[6] = {0, 0, 0, 0, 0, 0};
+        if (ok)
+            for (int i = 0; i < 6; ++i) m[i] = __ldg(a.affine + 6 * (size_t)k + i);
+        const uint8_t* gsrc = a.grey + (ok ? (size_t)r.frame * a.H * a.W : 0);
+        const uint16_t* dsrc = a.depth + (ok ? (size_t)r.frame * a.H * a.W : 0);
+        for (int v = vl; v < v1; v += (kCropThreads / 32) * rpw)
+            for (int q = ql; q < a.ow4; q += lpr) {
+                uint32_t gw = 0, d[2] = {0, 0};
+                if (ok) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int u = 4 * q + e;
+                        const uint2 tx = make_tap(m[0] * u + m[1] * v + m[2], a.W);
+                        const uint2 ty = make_tap(m[3] * u + m[4] * v + m[5], a.H);
+                        gw |= bilerp(gsrc, a.W, tx.x, ty.x) << (8 * e);
+                        d[e >> 1] |= (uint32_t)__ldg(dsrc + (size_t)ty.y * a.W + tx.y) << (16 * (e & 1));
+                    }
+                }
+                store_group(a, ((size_t)k * a.oh + v) * a.ow + 4 * q, 4 * q, gw, d[0], d[1]);
+            }
+    }
+}
+
+}  // namespace
+
+int launch_crop_affine(rgbd_ctx* ctx, const uint8_t* grey, const uint16_t* depth, int n_frames, int H, int W,
+                       const rgbd_rect* rects, const int32_t* affine, int n, int out_h, int out_w, uint8_t* og,
+                       uint16_t* od, cudaStream_t s) {
+    CropArgs a;
+    a.grey = grey, a.depth = depth, a.n_frames = n_frames, a.H = H, a.W = W, a.rects = rects, a.affine = affine;
+    a.n = n, a.oh = out_h, a.ow = out_w, a.og = og, a.od = od, a.status = ctx->d_status;
+    a.ow4 = (out_w + 3) / 4;
+    a.lanes_log2 = 0;
+    while (a.lanes_log2 < 5 && (1 << a.lanes_log2) < a.ow4) ++a.lanes_log2;
+    a.wide = out_w % 4 == 0 && (reinterpret_cast<uintptr_t>(og) & 3) == 0 && (reinterpret_cast<uintptr_t>(od) & 7) == 0;
+    // Rows per CTA: a strip pays for the column taps (two divisions per 4 columns), so strips are as
+    // tall as they can be while the grid still has some CTAs for every SM; at least one pass of the
+    // CTA's warps over the strip.
+    const int pass = (kCropThreads / 32) * (32 >> a.lanes_log2);
+    const long long want = 6LL * ctx->props.sm_count;
+    const long long strips = std::max(1LL, std::min((want + n - 1) / n, (long long)(out_h + pass - 1) / pass));
+    a.rows = (int)((out_h + strips - 1) / strips);
+    const dim3 grid((unsigned)((out_h + a.rows - 1) / a.rows), (unsigned)std::min(n, 65535));
+    const size_t smem = (sizeof(uint4) + sizeof(uint32_t)) * 2 * (size_t)a.ow4 + sizeof(uint2) * (size_t)a.rows;
+    if (affine) {
+        crop_affine_kernel<<<grid, kCropThreads, 0, s>>>(a);
+    } else {
+        // crops up to 4096 columns and rows: 41 KB of column taps and 33 KB of row taps at most
+        if (smem > 48 * 1024) {
+            const cudaError_t e =
+                cudaFuncSetAttribute(crop_rect_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return cuda_error(e, "rgbd_crop_affine: smem attribute");
+        }
+        crop_rect_kernel<<<grid, kCropThreads, smem, s>>>(a);
+    }
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_error(e, "rgbd_crop_affine: launch");
+    return RGBD_OK;
+}
+
+}  // namespace rgbd

@@ -34,34 +34,12 @@
 #include <algorithm>
 
 #include "internal.h"
+#include "resample.cuh"
 
 namespace rgbd {
 namespace {
 
 constexpr unsigned FULL = 0xFFFFFFFFu;
-
-// ---------------------------------------------------------------------------------------
-// A1 helpers: Q16.16 source coordinates, pixel centre to pixel centre.
-// ---------------------------------------------------------------------------------------
-
-// origin + (i + 1/2) * len / out_len - 1/2 in Q16.16 (len > 0, so the quotient is >= 0).
-__device__ __forceinline__ int64_t rect_coord_q16(int origin, int len, int out_len, int i) {
-    uint64_t num = (uint64_t)(2 * i + 1) * (uint64_t)len * 65536ull;
-    return (int64_t)origin * 65536 + (int64_t)(num / (2ull * (uint64_t)out_len)) - 32768;
-}
-
-// Packs the taps of one coordinate: .x = a | (b - a) << 16 | frac << 24 (bilinear: clamped
-// taps a = floor, b = floor + 1, Q8 fraction), .y = the clamped nearest index.
-__device__ __forceinline__ uint2 make_tap(int64_t q, int lim) {
-    const int64_t f0 = q >> 16;  // floor (arithmetic shift)
-    const int frac = (int)((q >> 8) & 255);
-    const int64_t nn = (q + 32768) >> 16;
-    const int64_t hi = (int64_t)lim - 1;
-    const int a = (int)(f0 < 0 ? 0 : (f0 > hi ? hi : f0));
-    const int b = (int)(f0 + 1 < 0 ? 0 : (f0 + 1 > hi ? hi : f0 + 1));
-    const int n = (int)(nn < 0 ? 0 : (nn > hi ? hi : nn));
-    return make_uint2((uint32_t)a | ((uint32_t)(b - a) << 16) | ((uint32_t)frac << 24), (uint32_t)n);
-}
 
 // Asks L2 for the source rows of a face rect (grey and depth, each row's span widened by one
 // pixel for the bilinear taps and clamped to the frame): one prefetch per 128 bytes, every
@@ -85,18 +63,6 @@ __device__ __forceinline__ void prefetch_rect_rows(const uint8_t* grey, const ui
             if (pp >= last - 127) break;
         }
     }
-}
-
-// Bilinear grey sample with Q8 weights (they sum to 2^16), rounded half up.
-__device__ __forceinline__ uint32_t bilerp(const uint8_t* img, int W, uint32_t cx, uint32_t ry) {
-    const uint32_t xa = cx & 0xFFFFu, dx = (cx >> 16) & 1u, fx = cx >> 24;
-    const uint32_t ya = ry & 0xFFFFu, dy = (ry >> 16) & 1u, fy = ry >> 24;
-    const uint8_t* r0 = img + (size_t)ya * W + xa;
-    const uint8_t* r1 = r0 + (size_t)dy * W;
-    const uint32_t p00 = __ldg(r0), p01 = __ldg(r0 + dx);
-    const uint32_t p10 = __ldg(r1), p11 = __ldg(r1 + dx);
-    const uint32_t acc = (256u - fy) * ((256u - fx) * p00 + fx * p01) + fy * ((256u - fx) * p10 + fx * p11);
-    return (acc + 32768u) >> 16;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1068,42 +1034,6 @@ size_t face256_smem(int S) {
 }
 
 // ---------------------------------------------------------------------------------------
-// Plain crop (rgbd_crop_affine): one thread per crop pixel.
-// ---------------------------------------------------------------------------------------
-__global__ void crop_affine_kernel(const uint8_t* __restrict__ grey, const uint16_t* __restrict__ depth,
-                                   int n_frames, int H, int W, const rgbd_rect* __restrict__ rects,
-                                   const int32_t* __restrict__ affine, int n, int oh, int ow,
-                                   uint8_t* __restrict__ og, uint16_t* __restrict__ od,
-                                   uint32_t* status) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= oh * ow) return;
-    const int v = p / ow, u = p - v * ow;
-    for (int k = blockIdx.y; k < n; k += gridDim.y) {
-        const rgbd_rect r = rects[k];
-        const size_t o = (size_t)k * oh * ow + p;
-        if (!(r.frame >= 0 && r.frame < n_frames && r.w > 0 && r.h > 0)) {
-            og[o] = 0;
-            od[o] = 0;
-            if (p == 0) atomicOr(status, RGBD_STATUS_BAD_RECT);
-            continue;
-        }
-        int64_t xq, yq;
-        if (affine) {
-            const int32_t* m = affine + 6 * (size_t)k;
-            xq = (int64_t)m[0] * u + (int64_t)m[1] * v + m[2];
-            yq = (int64_t)m[3] * u + (int64_t)m[4] * v + m[5];
-        } else {
-            xq = rect_coord_q16(r.x, r.w, ow, u);
-            yq = rect_coord_q16(r.y, r.h, oh, v);
-        }
-        const uint2 tx = make_tap(xq, W), ty = make_tap(yq, H);
-        const size_t base = (size_t)r.frame * H * W;
-        og[o] = (uint8_t)bilerp(grey + base, W, tx.x, ty.x);
-        od[o] = __ldg(depth + base + (size_t)ty.y * W + tx.y);
-    }
-}
-
-// ---------------------------------------------------------------------------------------
 // A5 alone: per-cell normalisation of count rows; one CTA per row.
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ float store_x(void* out, int dtype, size_t idx, float x, float scale,
@@ -1293,18 +1223,6 @@ int launch_lbp_fused(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
         default:
             return set_error(RGBD_ERR_UNSUPPORTED, "lbp_fused_features: crop %d (32, 64, 96 or 128)", a.crop);
     }
-}
-
-int launch_crop_affine(rgbd_ctx* ctx, const uint8_t* grey, const uint16_t* depth, int n_frames,
-                       int H, int W, const rgbd_rect* rects, const int32_t* affine, int n,
-                       int out_h, int out_w, uint8_t* og, uint16_t* od, cudaStream_t s) {
-    const int px = out_h * out_w;
-    dim3 grid((px + 255) / 256, std::min(n, 65535));
-    crop_affine_kernel<<<grid, 256, 0, s>>>(grey, depth, n_frames, H, W, rects, affine, n, out_h,
-                                            out_w, og, od, ctx->d_status);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_error(e, "rgbd_crop_affine: launch");
-    return RGBD_OK;
 }
 
 int launch_normalize(const uint16_t* feats, int n, int dim, int nbins, int x_dtype, void* x_out,

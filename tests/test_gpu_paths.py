@@ -53,3 +53,38 @@ def test_face_roi_scan_from_the_edges(B, ctx, orc, shape, colour_w, density):
         for i, f in enumerate(["frame", "x", "y", "w", "h"]):
             assert (got[:, i] == want[f]).all(), (flip, f)
     ctx.status(clear=True)
+
+
+@pytest.mark.parametrize("out_h,out_w", [(1, 1), (7, 5), (33, 64), (64, 100), (130, 257), (3, 1300)])
+@pytest.mark.parametrize("W", [8, 101, 320])
+def test_crop_affine_sizes(B, ctx, orc, out_h, out_w, W):
+    """Crops of widths that are and are not whole groups of 4 columns, strips of rows with a
+    remainder, frames of odd width (byte gathers) and of the narrowest width with 8-byte windows,
+    rects narrower and wider than twice the crop, partly outside the frame, and bad ones; by rect
+    and by affine map."""
+    rng = synth.rng_for(out_h * 1000 + out_w + W)
+    H = 60
+    g = rng.integers(0, 256, (2, H, W)).astype(np.uint8)
+    d = rng.integers(0, 65536, (2, H, W)).astype(np.uint16)
+    r = np.zeros(9, orc.RECT_DTYPE)
+    r["frame"] = rng.integers(0, 2, 9)
+    r["x"], r["y"] = rng.integers(-W, W, 9), rng.integers(-H, H, 9)
+    r["w"] = [1, 2 * out_w, 2 * out_w + 1, out_w, 5 * out_w, max(1, out_w // 3), 40, 0, 9]
+    r["h"] = [1, 2 * out_h, 3, out_h, 5 * out_h, 11, 40, 5, 9]
+    r[8]["frame"] = 2
+    gd, dd, rd = dev_u8(g), dev_u16(d), B.rects_tensor(r)
+    og, od = B.rgbd_crop_affine(ctx, gd, dd, rd, out_h, out_w)
+    og, od = og.cpu().numpy(), host_u16(od)
+    for k in range(7):
+        wg, wd = orc.crop(g[r[k]["frame"]], d[r[k]["frame"]], tuple(r[k][f] for f in ("x", "y", "w", "h")), out_h, out_w)
+        assert (og[k] == wg).all() and (od[k] == wd).all(), k
+    assert not og[7:].any() and not od[7:].any()
+    assert ctx.status(clear=True) & B.STATUS_BAD_RECT
+    aff = rng.integers(-70000, 70000, (9, 6)).astype(np.int32)
+    aff[:, [2, 5]] *= 30
+    og, od = B.rgbd_crop_affine(ctx, gd, dd, rd, out_h, out_w, affine=torch.from_numpy(aff).cuda())
+    og, od = og.cpu().numpy(), host_u16(od)
+    for k in range(7):
+        wg, wd = orc.crop(g[r[k]["frame"]], d[r[k]["frame"]], (0, 0, 1, 1), out_h, out_w, affine=aff[k])
+        assert (og[k] == wg).all() and (od[k] == wd).all(), k
+    ctx.status(clear=True)
