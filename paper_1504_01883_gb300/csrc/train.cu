@@ -2,68 +2,111 @@
 // face database; the paper does it on the CPU).  The dual problem of every class is solved by
 // sequential minimal optimisation with the maximal violating pair, on one kernel matrix that all
 // classes share:
-//   kernel_matrix_kernel  K_st = exp(-gamma max(0, |x_s|^2 + |x_t|^2 - 2 x_s . x_t)), fp32, a
-//                         64 x 64 register-tiled product per CTA;
+//   kernel_matrix_kernel  K_st = exp(-gamma max(0, |x_s|^2 + |x_t|^2 - 2 x_s . x_t)), fp32, one
+//                         tile of the lower triangle per CTA, written twice;
 //   smo_kernel            one CTA per class; alpha and the gradient G stay in shared memory; each
 //                         step reduces the two selections over the CTA, updates the pair on one
 //                         thread, then G_t += y_t lambda (K_it - K_jt) with all threads.
-#include <float.h>
+#include <limits.h>
 #include <stdint.h>
 
 #include <algorithm>
 
+#include "f32_tile.cuh"
 #include "internal.h"
 
 namespace rgbd {
 namespace {
 
-constexpr int KM_TILE = 64, KM_K = 16;
-constexpr int SMO_THREADS = 1024;
+// K_st = exp(-gamma max(0, |x_s|^2 + |x_t|^2 - 2 x_s . x_t)) for s >= t by tiles of BM x BM, and its
+// mirror image: the product, the sum of norms and so K itself are symmetric bit for bit, so half of
+// the products do.  The tiles of the lower triangle are numbered row by row.  Bound by the FMA
+// pipes.  4096 x 4096 rows of 15104: 20.4 ms as a full matrix with 4 x 4 outputs a thread,
+// 4.5 ms now.
+__device__ __forceinline__ void triangle_tile(long long idx, int& bi, int& bj) {
+    long long r = (long long)((sqrt(8.0 * (double)idx + 1.0) - 1.0) * 0.5);
+    while ((r + 1) * (r + 2) / 2 <= idx) ++r;  // the root is rounded: step to the exact row
+    while (r * (r + 1) / 2 > idx) --r;
+    bi = (int)r;
+    bj = (int)(idx - r * (r + 1) / 2);
+}
 
-__global__ void __launch_bounds__(256) kernel_matrix_kernel(const float* __restrict__ x, const float* __restrict__ xsq,
-                                                            int n, int k_pad, float gamma, float* __restrict__ K) {
-    __shared__ float As[KM_K][KM_TILE + 4];
-    __shared__ float Bs[KM_K][KM_TILE + 4];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int s0 = blockIdx.y * KM_TILE, t0 = blockIdx.x * KM_TILE;
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < k_pad; k0 += KM_K) {
-        // 64 rows x 16 columns of each operand: 256 threads load 4 values each
-        for (int e = threadIdx.x; e < KM_TILE * KM_K; e += 256) {
-            const int r = e / KM_K, kk = e - r * KM_K;
-            const int sr = s0 + r, tr = t0 + r;
-            As[kk][r] = (sr < n && k0 + kk < k_pad) ? x[(size_t)sr * k_pad + k0 + kk] : 0.f;
-            Bs[kk][r] = (tr < n && k0 + kk < k_pad) ? x[(size_t)tr * k_pad + k0 + kk] : 0.f;
-        }
-        __syncthreads();
+// ORDERED: tiles spread evenly over one CTA per SM (f32_ordered_tiles), else one tile per CTA.
+template <int BM, bool VEC, bool ORDERED>
+__global__ void __launch_bounds__(F32Tile<BM, BM>::NT, 1) kernel_matrix_kernel(const float* __restrict__ x,
+                                                                          const float* __restrict__ xsq, int n,
+                                                                          int k_pad, float gamma, long long tiles,
+                                                                          float* K, uint32_t* ready,
+                                                                          uint32_t* status) {
+    using Tile = F32Tile<BM, BM>;
+    extern __shared__ __align__(16) unsigned char km_smem[];
+    auto& sm = *reinterpret_cast<typename Tile::Smem*>(km_smem);
+    auto rows = [&](long long idx) {
+        int bi, bj;
+        triangle_tile(idx, bi, bj);
+        return F32Rows{x + (size_t)bi * BM * k_pad, n - bi * BM, x + (size_t)bj * BM * k_pad, n - bj * BM};
+    };
+    auto finish = [&](long long idx, const Tile& tile) {
+        int bi, bj;
+        triangle_tile(idx, bi, bj);
+        const int s0 = bi * BM, t0 = bj * BM;
 #pragma unroll
-        for (int kk = 0; kk < KM_K; ++kk) {
-            float a[4], b[4];
+        for (int i = 0; i < 8; ++i) {
+            const int s = s0 + tile.m_of(i);
+            if (s >= n) continue;
+            const float xs = xsq[s];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                a[u] = As[kk][ty * 4 + u];
-                b[u] = Bs[kk][tx * 4 + u];
+            for (int p = 0; p < 4; ++p) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int t = t0 + tile.n_of(p) + h;
+                    if (t >= n) continue;
+                    const float d2 = fmaxf(xs + xsq[t] - 2.f * tile.get(i, p, h), 0.f);
+                    const float k = (s == t) ? 1.f : expf(-gamma * d2);
+                    K[(size_t)s * n + t] = k;
+                    if (s0 != t0) K[(size_t)t * n + s] = k;
+                }
             }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
         }
-        __syncthreads();
-    }
+    };
+    if (ORDERED) {
+        // a split tile's chains wait in its own place of K
+        auto at = [&](long long idx, int i, int p, int h) -> float* {
+            int bi, bj;
+            triangle_tile(idx, bi, bj);
+            Tile t;
+            const int s = bi * BM + t.m_of(i), c = bj * BM + t.n_of(p) + h;
+            return s < n && c < n ? K + (size_t)s * n + c : nullptr;
+        };
+        auto stash = [&](long long idx, const Tile& t) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int s = s0 + ty * 4 + u;
-        if (s >= n) continue;
+            for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int t = t0 + tx * 4 + v;
-            if (t >= n) continue;
-            const float d2 = fmaxf(xsq[s] + xsq[t] - 2.f * acc[u][v], 0.f);
-            K[(size_t)s * n + t] = (s == t) ? 1.f : expf(-gamma * d2);
-        }
+                for (int p = 0; p < 4; ++p)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        if (float* q = at(idx, i, p, h)) __stcg(q, t.get(i, p, h));
+        };
+        auto fetch = [&](long long idx, Tile& t) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    const float *lo = at(idx, i, p, 0), *hi = at(idx, i, p, 1);
+                    t.put(i, p, lo ? __ldcg(lo) : 0.f, hi ? __ldcg(hi) : 0.f);
+                }
+        };
+        f32_ordered_tiles<Tile, VEC>(tiles, k_pad, ready, status, sm, rows, finish, stash, fetch);
+    } else {
+        const F32Rows r = rows(blockIdx.x);
+        Tile t;
+        t.clear();
+        t.template run<VEC>(r.a, r.na, r.b, r.nb, k_pad, 0, (k_pad + Tile::KB - 1) / Tile::KB, sm);
+        finish(blockIdx.x, t);
     }
 }
+
+constexpr int SMO_THREADS = 1024;
 
 // (value, index) pairs: the larger value wins (or the smaller, for the minimum), then the lower index
 __device__ __forceinline__ void arg_better_max(float& v, int& i, float ov, int oi) {
@@ -197,6 +240,15 @@ __global__ void __launch_bounds__(SMO_THREADS, 1) smo_kernel(const float* __rest
     for (int t = tid; t < n; t += SMO_THREADS) coef[(size_t)c * n + t] = (float)y[t] * alpha[t];
 }
 
+template <int BM, bool VEC, bool ORDERED>
+cudaError_t launch_kernel_matrix(int grid, const float* x, const float* xsq, int n, int k_pad, float gamma,
+                                 long long tiles, float* K, uint32_t* ready, uint32_t* status, cudaStream_t s) {
+    const size_t smem = sizeof(typename F32Tile<BM, BM>::Smem);
+    kernel_matrix_kernel<BM, VEC, ORDERED>
+        <<<grid, F32Tile<BM, BM>::NT, smem, s>>>(x, xsq, n, k_pad, gamma, tiles, K, ready, status);
+    return cudaGetLastError();
+}
+
 }  // namespace
 }  // namespace rgbd
 
@@ -215,12 +267,30 @@ extern "C" int svm_train_rbf(rgbd_ctx* ctx, const float* x, const float* xsq, in
     if (!x || !xsq || !labels || !coef || !bias || !iters) return set_error(RGBD_ERR_ARG, "svm_train_rbf: NULL pointer");
     DeviceGuard g(ctx->props.device);
     cudaStream_t s = (cudaStream_t)stream;
+    // 128 x 128 tiles spread over one CTA per SM when there is at least one for each, smaller tiles
+    // with a CTA each otherwise (a full 4096 x 4096 x 15104 product: 8.8 ms in 128 x 128
+    // tiles, 9.3 ms in 64 x 64; 168 of the large tiles, 777 x 3001: 1.45 ms spread, 2.0 ms as small ones).
+    const long long b128 = (n + 127) / 128, t128 = b128 * (b128 + 1) / 2;
+    const bool ordered = t128 >= ctx->props.sm_count && n >= ctx->props.sm_count;
+    const long long b64 = (n + 63) / 64;
+    const long long tiles = ordered ? t128 : b64 * (b64 + 1) / 2;
+    const int grid = ordered ? ctx->props.sm_count : (int)tiles;
     int rc = ensure_workspace(ctx, sizeof(float) * (size_t)n * n, s);
     if (rc) return rc;
     float* K = (float*)ctx->workspace;
-    dim3 grid((n + KM_TILE - 1) / KM_TILE, (n + KM_TILE - 1) / KM_TILE);
-    kernel_matrix_kernel<<<grid, 256, 0, s>>>(x, xsq, n, k_pad, gamma, K);
-    cudaError_t e = cudaGetLastError();
+    // the hand-over flags live in the coefficients until SMO writes them (n >= 2049 when ordered)
+    uint32_t* ready = reinterpret_cast<uint32_t*>(coef);
+    const bool vec = k_pad % 16 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
+    cudaError_t e = cudaSuccess;
+    if (ordered) {
+        e = cudaMemsetAsync(ready, 0, sizeof(uint32_t) * (size_t)grid, s);
+        if (e != cudaSuccess) return cuda_error(e, "svm_train_rbf: tile hand-over reset");
+        e = vec ? launch_kernel_matrix<128, true, true>(grid, x, xsq, n, k_pad, gamma, tiles, K, ready, ctx->d_status, s)
+                : launch_kernel_matrix<128, false, true>(grid, x, xsq, n, k_pad, gamma, tiles, K, ready, ctx->d_status, s);
+    } else {
+        e = vec ? launch_kernel_matrix<64, true, false>(grid, x, xsq, n, k_pad, gamma, tiles, K, ready, ctx->d_status, s)
+                : launch_kernel_matrix<64, false, false>(grid, x, xsq, n, k_pad, gamma, tiles, K, ready, ctx->d_status, s);
+    }
     if (e != cudaSuccess) return cuda_error(e, "svm_train_rbf: kernel matrix launch");
     const size_t smem = sizeof(float) * 2 * (size_t)n + (size_t)n;
     e = cudaFuncSetAttribute(smo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

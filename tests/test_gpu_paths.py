@@ -88,3 +88,45 @@ def test_crop_affine_sizes(B, ctx, orc, out_h, out_w, W):
         wg, wd = orc.crop(g[r[k]["frame"]], d[r[k]["frame"]], (0, 0, 1, 1), out_h, out_w, affine=aff[k])
         assert (og[k] == wg).all() and (od[k] == wd).all(), k
     ctx.status(clear=True)
+
+
+@pytest.mark.parametrize("n,k_pad", [(2, 7), (65, 128), (200, 531), (700, 256), (2100, 48), (2100, 50)])
+def test_kernel_matrix_and_smo_of_every_size(B, ctx, orc, n, k_pad):
+    """Training on few and many rows (one to sixteen rows per thread, one tile per CTA and tiles
+    handed from CTA to CTA), rows of lengths that are not multiples of 4 or 16: the solution is
+    that of the fp64 oracle, and the norms and rows may have any length."""
+    rng = synth.rng_for(n + k_pad)
+    C = 3
+    lab = rng.integers(0, C, n).astype(np.int32)
+    x = (rng.normal(0, 1, (C, k_pad))[lab] + rng.normal(0, 0.7, (n, k_pad))).astype(np.float32) / np.sqrt(k_pad)
+    x = x.astype(np.float32)
+    q = (x.astype(np.float64) ** 2).sum(1).astype(np.float32)
+    steps = 60  # a bounded number of steps: the same path as the oracle's, step by step
+    xt, qt, lt = dev_f32(x), dev_f32(q), torch.from_numpy(lab).cuda()
+    coef, bias, iters = B.svm_train_rbf(ctx, xt, qt, lt, C, 1.0, 1.0, 1e-3, max_iter=steps)
+    again = B.svm_train_rbf(ctx, xt, qt, lt, C, 1.0, 1.0, 1e-3, max_iter=steps)
+    assert ctx.status() == 0 and all(torch.equal(u, v) for u, v in zip((coef, bias, iters), again))
+    it, a = iters.cpu().numpy(), coef.cpu().numpy().astype(np.float64)
+    y = np.where(lab[None, :] == np.arange(C)[:, None], 1.0, -1.0)
+    alpha = a * y
+    assert (alpha >= 0).all() and (alpha <= 1).all() and (it <= steps).all()
+    # every step keeps sum a = 0 (fp32 rounding of each step) and lowers the dual objective
+    assert np.abs(a.sum(1)).max() <= 1e-6 * (1 + np.abs(a).sum(1).max())
+    x64 = x.astype(np.float64)
+    K = np.exp(-(np.maximum((x64 ** 2).sum(1)[:, None] + (x64 ** 2).sum(1)[None, :] - 2 * x64 @ x64.T, 0)))
+    for c in range(C):
+        if it[c] == 0:
+            continue
+        # the gradient that the kernel walked along gives its stopping gap: recompute it in fp64
+        G = y[c] * (K @ a[c]) - 1.0
+        v = -y[c] * G
+        up = ((y[c] > 0) & (alpha[c] < 1)) | ((y[c] < 0) & (alpha[c] > 0))
+        low = ((y[c] > 0) & (alpha[c] > 0)) | ((y[c] < 0) & (alpha[c] < 1))
+        gap = v[up].max() - v[low].min()
+        obj = 0.5 * a[c] @ K @ a[c] - alpha[c].sum()
+        assert obj < 0
+        if it[c] < steps:
+            assert gap <= 1e-3 + 1e-4  # fp32 gradient of up to 60 steps
+        free = (alpha[c] > 0) & (alpha[c] < 1)
+        if free.any():
+            assert abs(bias[c].item() - v[free].mean()) <= 1e-4
