@@ -4,9 +4,8 @@
 // classes share:
 //   kernel_matrix_kernel  K_st = exp(-gamma max(0, |x_s|^2 + |x_t|^2 - 2 x_s . x_t)), fp32, one
 //                         tile of the lower triangle per CTA, written twice;
-//   smo_kernel            one CTA per class; alpha and the gradient G stay in shared memory; each
-//                         step reduces the two selections over the CTA, updates the pair on one
-//                         thread, then G_t += y_t lambda (K_it - K_jt) with all threads.
+//   smo_kernel            one CTA per class; the gradient stays in registers; each step selects the
+//                         pair over the CTA, updates it, then moves the gradient with all threads.
 #include <limits.h>
 #include <stdint.h>
 
@@ -106,138 +105,184 @@ __global__ void __launch_bounds__(F32Tile<BM, BM>::NT, 1) kernel_matrix_kernel(c
     }
 }
 
-constexpr int SMO_THREADS = 1024;
-
-// (value, index) pairs: the larger value wins (or the smaller, for the minimum), then the lower index
-__device__ __forceinline__ void arg_better_max(float& v, int& i, float ov, int oi) {
-    if (oi >= 0 && (i < 0 || ov > v || (ov == v && oi < i))) {
-        v = ov;
-        i = oi;
-    }
+// Order of floats as signed integers (and back): the largest value by an integer maximum.
+__device__ __forceinline__ int float_key(float v) {
+    const int b = __float_as_int(v);
+    return b ^ ((b >> 31) & 0x7FFFFFFF);
 }
-__device__ __forceinline__ void arg_better_min(float& v, int& i, float ov, int oi) {
-    if (oi >= 0 && (i < 0 || ov < v || (ov == v && oi < i))) {
-        v = ov;
-        i = oi;
-    }
-}
+__device__ __forceinline__ float key_float(int k) { return __int_as_float(k ^ ((k >> 31) & 0x7FFFFFFF)); }
 
-__global__ void __launch_bounds__(SMO_THREADS, 1) smo_kernel(const float* __restrict__ K, int n,
-                                                            const int32_t* __restrict__ labels, float cost, float eps,
-                                                            int max_iter, float* __restrict__ coef,
-                                                            float* __restrict__ bias, int32_t* __restrict__ iters) {
-    extern __shared__ float smo_smem[];
-    float* alpha = smo_smem;
-    float* G = smo_smem + n;
-    int8_t* y = reinterpret_cast<int8_t*>(smo_smem + 2 * n);
-    __shared__ float rv[2][32];
-    __shared__ int ri[2][32];
-    __shared__ int sel_i, sel_j, stop;
-    __shared__ float sel_lam, sel_m, sel_M;
+// One CTA per class.  A step is a chain of latencies (select a pair, fetch its two rows of K, move,
+// select again), so it holds one barrier: every thread keeps the values u_t = -y_t G_t of its EPT
+// rows in registers with a bit each for "may move up / down", its warp selects by integer redux
+// (largest or smallest value, then the lowest index), and the warps' candidates -- with alpha and
+// y, which only the owner of a row keeps -- go to shared memory, where after the barrier every
+// warp makes the same final selection and update for itself.  u_t += -lam (K_it - K_jt) is the
+// gradient step G_t += y_t lam (K_it - K_jt) with the sign folded in, rounding alike.  K_ii = 1.
+// 64 classes x 4096 rows, ~1500 steps each: 8.4 ms with three barriers and a serial selection by
+// one thread per step, 1.86 ms now.
+struct SmoPick {
+    int key;
+    uint32_t idx;  // ~0: none
+    float alpha;
+    int y;
+};
+
+template <int T, int EPT>
+__global__ void __launch_bounds__(T, 1) smo_kernel(const float* __restrict__ K, int n,
+                                                   const int32_t* __restrict__ labels, float cost, float eps,
+                                                   int max_iter, float* __restrict__ coef, float* __restrict__ bias,
+                                                   int32_t* __restrict__ iters) {
+    constexpr int NW = T / 32;
+    constexpr uint32_t NONE = 0xFFFFFFFFu, FULL = 0xFFFFFFFFu;
+    extern __shared__ float alpha[];  // [n], each entry touched by the thread that owns the row
+    __shared__ __align__(16) SmoPick picks[2][2][NW];
+    __shared__ float sums[32];
+    __shared__ int counts[32];
     const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int t = tid; t < n; t += SMO_THREADS) {
-        y[t] = labels[t] == c ? 1 : -1;
-        alpha[t] = 0.f;
-        G[t] = -1.f;
+    float u[EPT];
+    uint32_t ypos = 0, up = 0, low = 0;  // a bit per row: y > 0, may move up, may move down
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) {
+        const int t = tid + e * T;
+        u[e] = 0.f;
+        if (t < n) {  // alpha = 0: y > 0 may move up, y < 0 down
+            const bool pos = labels[t] == c;
+            u[e] = pos ? 1.f : -1.f;
+            alpha[t] = 0.f;
+            ypos |= (uint32_t)pos << e;
+            up |= (uint32_t)pos << e;
+            low |= (uint32_t)!pos << e;
+        }
     }
-    __syncthreads();
     int it = 0;
-    for (;;) {
-        // selection: i = argmax over I_up of -y G, j = argmin over I_low of -y G
-        float mu = 0.f, ml = 0.f;
-        int iu = -1, il = -1;
-        for (int t = tid; t < n; t += SMO_THREADS) {
-            const float v = -(float)y[t] * G[t];
-            const bool up = (y[t] > 0 && alpha[t] < cost) || (y[t] < 0 && alpha[t] > 0.f);
-            const bool low = (y[t] > 0 && alpha[t] > 0.f) || (y[t] < 0 && alpha[t] < cost);
-            if (up) arg_better_max(mu, iu, v, t);
-            if (low) arg_better_min(ml, il, v, t);
+    float mu, ml;
+    uint32_t iu, il;
+    for (;; ++it) {
+        int key[EPT], ku = INT_MIN, kl = INT_MAX;
+#pragma unroll
+        for (int e = 0; e < EPT; ++e) {
+            key[e] = float_key(u[e]);
+            if ((up >> e) & 1u) ku = max(ku, key[e]);
+            if ((low >> e) & 1u) kl = min(kl, key[e]);
+        }
+        ku = __reduce_max_sync(FULL, ku);
+        kl = __reduce_min_sync(FULL, kl);
+        iu = il = NONE;
+#pragma unroll
+        for (int e = EPT - 1; e >= 0; --e) {
+            if (((up >> e) & 1u) && key[e] == ku) iu = (uint32_t)(tid + e * T);
+            if (((low >> e) & 1u) && key[e] == kl) il = (uint32_t)(tid + e * T);
+        }
+        const uint32_t wu = __reduce_min_sync(FULL, iu), wl = __reduce_min_sync(FULL, il);
+        SmoPick* pk = &picks[it & 1][0][0];
+        if (wu == NONE ? lane == 0 : iu == wu) {
+            SmoPick q = {ku, wu, 0.f, 0};
+            if (wu != NONE) q.alpha = alpha[wu], q.y = (ypos >> ((wu - tid) / T)) & 1u ? 1 : -1;
+            pk[warp] = q;
+        }
+        if (wl == NONE ? lane == 0 : il == wl) {
+            SmoPick q = {kl, wl, 0.f, 0};
+            if (wl != NONE) q.alpha = alpha[wl], q.y = (ypos >> ((wl - tid) / T)) & 1u ? 1 : -1;
+            pk[NW + warp] = q;
+        }
+        __syncthreads();
+        // i = argmax over the rows that may move up, j = argmin over those that may move down
+        SmoPick a = {INT_MIN, NONE, 0.f, 0}, b = {INT_MAX, NONE, 0.f, 0};
+        if (lane < NW) {
+            a = pk[lane];
+            b = pk[NW + lane];
+        }
+        ku = __reduce_max_sync(FULL, a.idx == NONE ? INT_MIN : a.key);
+        kl = __reduce_min_sync(FULL, b.idx == NONE ? INT_MAX : b.key);
+        iu = __reduce_min_sync(FULL, a.key == ku ? a.idx : NONE);
+        il = __reduce_min_sync(FULL, b.key == kl ? b.idx : NONE);
+        mu = key_float(ku);
+        ml = key_float(kl);
+        if (iu == NONE || il == NONE || mu - ml <= eps || it >= max_iter) break;
+        const float* Ki = K + (size_t)iu * n;
+        const float* Kj = K + (size_t)il * n;
+        const float kij = __ldg(Ki + il);
+        float vi[EPT], vj[EPT];
+#pragma unroll
+        for (int e = 0; e < EPT; ++e) {
+            const int t = tid + e * T;
+            vi[e] = t < n ? __ldg(Ki + t) : 0.f;
+            vj[e] = t < n ? __ldg(Kj + t) : 0.f;
+        }
+        const int sa = __ffs(__ballot_sync(FULL, a.idx == iu)) - 1, sb = __ffs(__ballot_sync(FULL, b.idx == il)) - 1;
+        const float alpha_i = __shfl_sync(FULL, a.alpha, sa), alpha_j = __shfl_sync(FULL, b.alpha, sb);
+        const int yi = __shfl_sync(FULL, a.y, sa), yj = __shfl_sync(FULL, b.y, sb);
+        float eta = 1.f + 1.f - 2.f * kij;
+        if (eta < 1e-12f) eta = 1e-12f;
+        float lam = (mu - ml) / eta;
+        const float lim_i = yi > 0 ? cost - alpha_i : alpha_i;
+        const float lim_j = yj > 0 ? alpha_j : cost - alpha_j;
+        const bool hit_i = lam >= lim_i, hit_j = lam >= lim_j;
+        lam = fminf(lam, fminf(lim_i, lim_j));
+        float ai = alpha_i + (float)yi * lam, aj = alpha_j - (float)yj * lam;
+        ai = fminf(fmaxf(ai, 0.f), cost);
+        aj = fminf(fmaxf(aj, 0.f), cost);
+        if (hit_i && lam == lim_i) ai = yi > 0 ? cost : 0.f;  // snap the box edges exactly
+        if (hit_j && lam == lim_j) aj = yj > 0 ? 0.f : cost;
+        auto move = [&](uint32_t row, float al, int y) {  // by the thread that owns the row
+            if ((int)(row % T) != tid) return;
+            const uint32_t bit = 1u << (row / T);
+            alpha[row] = al;
+            const bool can_grow = al < cost, can_shrink = al > 0.f;
+            up = (y > 0 ? can_grow : can_shrink) ? up | bit : up & ~bit;
+            low = (y > 0 ? can_shrink : can_grow) ? low | bit : low & ~bit;
+        };
+        move(iu, ai, yi);
+        move(il, aj, yj);
+#pragma unroll
+        for (int e = 0; e < EPT; ++e) u[e] = fmaf(-lam, vi[e] - vj[e], u[e]);
+    }
+    // bias: mean of -y G over the free vectors, else the midpoint of the last bounds.  In fp32 the
+    // order counts: rows t, t + 1024, t + 2048, ... in a chain, 32 neighbouring chains by halves,
+    // and those sums in order, whatever T is.
+    constexpr int CH = EPT < 1024 / T ? EPT : 1024 / T;  // chains per thread
+#pragma unroll
+    for (int q = 0; q < CH; ++q) {
+        float s = 0.f;
+        int k = 0;
+#pragma unroll
+        for (int e = q; e < EPT; e += CH) {
+            const int t = tid + e * T;
+            if (t < n && alpha[t] > 0.f && alpha[t] < cost) {
+                s += u[e];
+                ++k;
+            }
         }
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            arg_better_max(mu, iu, __shfl_xor_sync(0xFFFFFFFFu, mu, off), __shfl_xor_sync(0xFFFFFFFFu, iu, off));
-            arg_better_min(ml, il, __shfl_xor_sync(0xFFFFFFFFu, ml, off), __shfl_xor_sync(0xFFFFFFFFu, il, off));
-        }
-        if (lane == 0) {
-            rv[0][warp] = mu, ri[0][warp] = iu;
-            rv[1][warp] = ml, ri[1][warp] = il;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            for (int w = 1; w < SMO_THREADS / 32; ++w) {
-                arg_better_max(mu, iu, rv[0][w], ri[0][w]);
-                arg_better_min(ml, il, rv[1][w], ri[1][w]);
-            }
-            sel_m = mu, sel_M = ml;
-            sel_i = iu, sel_j = il;
-            int st = iu < 0 || il < 0 || mu - ml <= eps || it >= max_iter;
-            if (!st) {
-                const float kii = K[(size_t)iu * n + iu], kjj = K[(size_t)il * n + il], kij = K[(size_t)iu * n + il];
-                float eta = kii + kjj - 2.f * kij;
-                if (eta < 1e-12f) eta = 1e-12f;
-                float lam = (mu - ml) / eta;
-                const float lim_i = y[iu] > 0 ? cost - alpha[iu] : alpha[iu];
-                const float lim_j = y[il] > 0 ? alpha[il] : cost - alpha[il];
-                const bool hit_i = lam >= lim_i, hit_j = lam >= lim_j;
-                lam = fminf(lam, fminf(lim_i, lim_j));
-                float ai = alpha[iu] + (float)y[iu] * lam, aj = alpha[il] - (float)y[il] * lam;
-                ai = fminf(fmaxf(ai, 0.f), cost);
-                aj = fminf(fmaxf(aj, 0.f), cost);
-                if (hit_i && lam == lim_i) ai = y[iu] > 0 ? cost : 0.f;  // snap the box edges exactly
-                if (hit_j && lam == lim_j) aj = y[il] > 0 ? 0.f : cost;
-                alpha[iu] = ai;
-                alpha[il] = aj;
-                sel_lam = lam;
-            }
-            stop = st;
-        }
-        __syncthreads();
-        if (stop) break;
-        const float lam = sel_lam;
-        const float* Ki = K + (size_t)sel_i * n;
-        const float* Kj = K + (size_t)sel_j * n;
-        for (int t = tid; t < n; t += SMO_THREADS) G[t] += (float)y[t] * lam * (Ki[t] - Kj[t]);
-        ++it;
-        __syncthreads();
-    }
-    // bias: mean of -y G over the free vectors, else the midpoint of the last bounds
-    float sum = 0.f;
-    int cnt = 0;
-    for (int t = tid; t < n; t += SMO_THREADS)
-        if (alpha[t] > 0.f && alpha[t] < cost) {
-            sum += -(float)y[t] * G[t];
-            ++cnt;
-        }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
-        cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, off);
-    }
-    __syncthreads();
-    if (lane == 0) {
-        rv[0][warp] = sum;
-        ri[0][warp] = cnt;
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(FULL, s, off);
+        k = __reduce_add_sync(FULL, k);
+        if (lane == 0) sums[q * NW + warp] = s, counts[q * NW + warp] = k;
     }
     __syncthreads();
     if (tid == 0) {
         float s = 0.f;
         int k = 0;
-        for (int w = 0; w < SMO_THREADS / 32; ++w) s += rv[0][w], k += ri[0][w];
+        for (int w = 0; w < CH * NW; ++w) s += sums[w], k += counts[w];
         float b;
         if (k > 0)
             b = s / (float)k;
-        else if (sel_i >= 0 && sel_j >= 0)
-            b = 0.5f * (sel_m + sel_M);
-        else if (sel_i >= 0)
-            b = sel_m;
-        else if (sel_j >= 0)
-            b = sel_M;
+        else if (iu != NONE && il != NONE)
+            b = 0.5f * (mu + ml);
+        else if (iu != NONE)
+            b = mu;
+        else if (il != NONE)
+            b = ml;
         else
             b = 0.f;
         bias[c] = b;
         iters[c] = it;
     }
-    for (int t = tid; t < n; t += SMO_THREADS) coef[(size_t)c * n + t] = (float)y[t] * alpha[t];
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) {
+        const int t = tid + e * T;
+        if (t < n) coef[(size_t)c * n + t] = ((ypos >> e) & 1u ? 1.f : -1.f) * alpha[t];
+    }
 }
 
 template <int BM, bool VEC, bool ORDERED>
@@ -246,6 +291,17 @@ cudaError_t launch_kernel_matrix(int grid, const float* x, const float* xsq, int
     const size_t smem = sizeof(typename F32Tile<BM, BM>::Smem);
     kernel_matrix_kernel<BM, VEC, ORDERED>
         <<<grid, F32Tile<BM, BM>::NT, smem, s>>>(x, xsq, n, k_pad, gamma, tiles, K, ready, status);
+    return cudaGetLastError();
+}
+
+template <int T, int EPT>
+cudaError_t launch_smo(const float* K, int n, const int32_t* labels, int n_classes, float cost, float eps,
+                       int max_iter, float* coef, float* bias, int32_t* iters, cudaStream_t s) {
+    const size_t smem = sizeof(float) * (size_t)n;
+    const cudaError_t e =
+        cudaFuncSetAttribute(smo_kernel<T, EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    smo_kernel<T, EPT><<<n_classes, T, smem, s>>>(K, n, labels, cost, eps, max_iter, coef, bias, iters);
     return cudaGetLastError();
 }
 
@@ -292,11 +348,17 @@ extern "C" int svm_train_rbf(rgbd_ctx* ctx, const float* x, const float* xsq, in
                 : launch_kernel_matrix<64, false, false>(grid, x, xsq, n, k_pad, gamma, tiles, K, ready, ctx->d_status, s);
     }
     if (e != cudaSuccess) return cuda_error(e, "svm_train_rbf: kernel matrix launch");
-    const size_t smem = sizeof(float) * 2 * (size_t)n + (size_t)n;
-    e = cudaFuncSetAttribute(smo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_error(e, "svm_train_rbf: smem attribute");
-    smo_kernel<<<n_classes, SMO_THREADS, smem, s>>>(K, n, labels, cost, eps, max_iter, coef, bias, iters);
-    e = cudaGetLastError();
+    // Up to 16 rows per thread (they live in registers), and no more warps than that takes: the
+    // selection and the barrier cost every warp the same, however few rows it holds (4096 rows:
+    // 1.86 ms with 8 warps, 2.48 ms with 32).
+#define RGBD_SMO(TV, EV) launch_smo<TV, EV>(K, n, labels, n_classes, cost, eps, max_iter, coef, bias, iters, s)
+    e = n <= 256    ? RGBD_SMO(256, 1)
+        : n <= 1024 ? RGBD_SMO(256, 4)
+        : n <= 2048 ? RGBD_SMO(256, 8)
+        : n <= 4096 ? RGBD_SMO(256, 16)
+        : n <= 8192 ? RGBD_SMO(512, 16)
+                    : RGBD_SMO(1024, 16);
+#undef RGBD_SMO
     if (e != cudaSuccess) return cuda_error(e, "svm_train_rbf: SMO launch");
     return RGBD_OK;
 }
