@@ -1033,138 +1033,6 @@ size_t face256_smem(int S) {
            4 * 512 + 16 + 4 * 32;
 }
 
-// ---------------------------------------------------------------------------------------
-// A5 alone: per-cell normalisation of count rows; one CTA per row.
-// ---------------------------------------------------------------------------------------
-__device__ __forceinline__ float store_x(void* out, int dtype, size_t idx, float x, float scale,
-                                         size_t plane = 0) {
-    if (dtype == RGBD_DT_BF16) {
-        const __nv_bfloat16 q = __float2bfloat16_rn(x);
-        reinterpret_cast<uint16_t*>(out)[idx] = __bfloat16_as_ushort(q);
-        return __bfloat162float(q);
-    } else if (dtype == RGBD_DT_BF16X3) {
-        // hi = bf16(x), lo = bf16(x - hi): x = hi + lo to 2^-18 relative
-        const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-        const float hf = __bfloat162float(hi);
-        const __nv_bfloat16 lo = __float2bfloat16_rn(x - hf);
-        reinterpret_cast<uint16_t*>(out)[idx] = __bfloat16_as_ushort(hi);
-        reinterpret_cast<uint16_t*>(out)[idx + plane] = __bfloat16_as_ushort(lo);
-        return hf + __bfloat162float(lo);
-    } else if (dtype == RGBD_DT_FP8) {
-        const __nv_fp8_e4m3 q(x * scale);
-        reinterpret_cast<uint8_t*>(out)[idx] = q.__x;
-        return static_cast<float>(q) * (1.0f / scale);
-    }
-    reinterpret_cast<float*>(out)[idx] = x;
-    return x;
-}
-
-__global__ void normalize_kernel(const uint16_t* __restrict__ feats, int n, int dim, int nbins,
-                                 int x_dtype, void* x_out, int k_pad, float x_scale, float* xsq,
-                                 float* row_max, size_t plane, const float* __restrict__ centre) {
-    extern __shared__ uint32_t nv[];  // [dim / nbins]
-    __shared__ float red[2][32];
-    const int cells = dim / nbins;
-    for (int row = blockIdx.x; row < n; row += gridDim.x) {
-        __syncthreads();
-        const uint16_t* h = feats + (size_t)row * dim;
-        for (int c = threadIdx.x; c < cells; c += blockDim.x) {
-            uint32_t t = 0;
-            for (int b = 0; b < nbins; ++b) t += h[c * nbins + b];
-            nv[c] = t;
-        }
-        __syncthreads();
-        float sq = 0.f, mx = 0.f;
-        for (int j = threadIdx.x; j < k_pad; j += blockDim.x) {
-            float x = 0.f;
-            if (j < dim) {
-                const uint32_t t = nv[j / nbins];
-                x = t ? (float)h[j] / (float)t : 0.f;
-                if (centre) x = __fsub_rn(x, centre[j]);
-            }
-            mx = fmaxf(mx, fabsf(x));
-            const float q = store_x(x_out, x_dtype, (size_t)row * k_pad + j, x, x_scale, plane);
-            sq = fmaf(q, q, sq);
-        }
-        for (int off = 16; off > 0; off >>= 1) {
-            sq += __shfl_xor_sync(FULL, sq, off);
-            mx = fmaxf(mx, __shfl_xor_sync(FULL, mx, off));
-        }
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        if (lane == 0) {
-            red[0][warp] = sq;
-            red[1][warp] = mx;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float t = 0.f, m = 0.f;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-                t += red[0][w];
-                m = fmaxf(m, red[1][w]);
-            }
-            if (xsq) xsq[row] = t;
-            if (row_max) atomicMax(reinterpret_cast<int*>(row_max), __float_as_int(m));  // m >= 0
-        }
-    }
-}
-
-// fp32 rows -> dtype rows (FP8 with `scale`), with squared norms of the stored values.
-__global__ void quantize_kernel(const float* __restrict__ src, int n, int k_pad, int dtype, void* dst,
-                                float scale, float* sq_out, size_t plane) {
-    __shared__ float red[32];
-    for (int row = blockIdx.x; row < n; row += gridDim.x) {
-        __syncthreads();
-        float sq = 0.f;
-        for (int j = threadIdx.x; j < k_pad; j += blockDim.x) {
-            const float q = store_x(dst, dtype, (size_t)row * k_pad + j, src[(size_t)row * k_pad + j], scale, plane);
-            sq = fmaf(q, q, sq);
-        }
-        for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(FULL, sq, off);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float t = 0.f;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-            if (sq_out) sq_out[row] = t;
-        }
-    }
-}
-
-// mu[j] = fp32(sum_i rows[i][j] / n), the sum in fp64 in row order (one thread per column, so
-// the order and the result are fixed); mu[j] = 0 for j >= dim.
-__global__ void column_mean_kernel(const float* __restrict__ rows, int n, int dim, int k_pad, float* __restrict__ mu) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= k_pad) return;
-    double acc = 0.0;
-    if (j < dim)
-        for (int i = 0; i < n; ++i) acc += (double)rows[(size_t)i * k_pad + j];
-    mu[j] = j < dim ? (float)(acc / (double)n) : 0.f;
-}
-
-// rows[i][j] -= mu[j] (fp32, round to nearest even); *absmax = max |result| (non-negative floats
-// order like their bit patterns, so an integer max serves).
-__global__ void centre_kernel(float* __restrict__ rows, int n, int k_pad, const float* __restrict__ mu,
-                              float* absmax) {
-    __shared__ float red[32];
-    for (int row = blockIdx.x; row < n; row += gridDim.x) {
-        float m = 0.f;
-        for (int j = threadIdx.x; j < k_pad; j += blockDim.x) {
-            const size_t idx = (size_t)row * k_pad + j;
-            const float v = __fsub_rn(rows[idx], mu[j]);
-            rows[idx] = v;
-            m = fmaxf(m, fabsf(v));
-        }
-        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, off));
-        __syncthreads();
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, red[w]);
-            atomicMax(reinterpret_cast<int*>(absmax), __float_as_int(m));
-        }
-    }
-}
-
 template <int S, int TPC>
 int launch_fused_t(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
     static int blocks_per_sm = -1;
@@ -1223,41 +1091,6 @@ int launch_lbp_fused(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
         default:
             return set_error(RGBD_ERR_UNSUPPORTED, "lbp_fused_features: crop %d (32, 64, 96 or 128)", a.crop);
     }
-}
-
-int launch_normalize(const uint16_t* feats, int n, int dim, int nbins, int x_dtype, void* x_out,
-                     int k_pad, float x_scale, float* xsq, float* row_max, cudaStream_t s, size_t plane,
-                     const float* centre) {
-    const int cells = dim / nbins;
-    const size_t smem = sizeof(uint32_t) * (size_t)cells;
-    if (smem > 48 * 1024) return set_error(RGBD_ERR_UNSUPPORTED, "normalize: %d cells", cells);
-    const int grid = std::min(n, 8192);
-    if (plane == 0) plane = (size_t)n * k_pad;
-    normalize_kernel<<<grid, 256, smem, s>>>(feats, n, dim, nbins, x_dtype, x_out, k_pad, x_scale,
-                                             xsq, row_max, plane, centre);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_error(e, "lbp_normalize_features: launch");
-    return RGBD_OK;
-}
-
-int launch_quantize_f32(const float* src, int n, int k_pad, int x_dtype, void* dst, float scale,
-                        float* sq, cudaStream_t s, size_t plane) {
-    const int grid = std::min(n, 8192);
-    if (plane == 0) plane = (size_t)n * k_pad;
-    quantize_kernel<<<grid, 256, 0, s>>>(src, n, k_pad, x_dtype, dst, scale, sq, plane);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_error(e, "quantize: launch");
-    return RGBD_OK;
-}
-
-int launch_centre_rows(float* rows, int n, int dim, int k_pad, float* mu, float* absmax, cudaStream_t s) {
-    column_mean_kernel<<<(k_pad + 255) / 256, 256, 0, s>>>(rows, n, dim, k_pad, mu);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_error(e, "centre: mean launch");
-    centre_kernel<<<std::min(n, 8192), 256, 0, s>>>(rows, n, k_pad, mu, absmax);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_error(e, "centre: launch");
-    return RGBD_OK;
 }
 
 }  // namespace rgbd

@@ -90,6 +90,53 @@ def test_crop_affine_sizes(B, ctx, orc, out_h, out_w, W):
     ctx.status(clear=True)
 
 
+@pytest.mark.parametrize("dim,nbins", [(59, 59), (9 * 59, 59), (144 * 59, 59), (256 * 59, 59), (256, 256), (512, 256),
+                                       (24, 8), (70, 7), (70000, 10), (65536, 16)])
+@pytest.mark.parametrize("dt", ["f32", "bf16", "fp8", "bf16x3"])
+def test_normalise_rows_are_ieee_quotients(B, ctx, orc, dim, nbins, dt):
+    """Rows of every staging form (aligned and odd row lengths, one to many lanes per cell, fewer
+    than 8 bins, too long for shared memory): IEEE quotients bit for bit, for counts from 0 to
+    65535, converted as the type says, with and without a centre; norms of the stored values."""
+    rng = synth.rng_for(dim + nbins)
+    cnt = rng.integers(0, 5, (7, dim)).astype(np.uint16)
+    cnt[1] = rng.integers(0, 65536, dim)
+    cnt[2] = 0
+    cnt[3, : nbins] = 65535
+    cnt[4] = rng.poisson(400, dim)
+    mu = rng.uniform(-0.1, 0.3, (dim + 3) // 4 * 4).astype(np.float32)
+    tot = cnt.reshape(7, -1, nbins).astype(np.int64).sum(2, keepdims=True)
+    x32 = (cnt.reshape(7, -1, nbins).astype(np.float32) / np.maximum(tot, 1).astype(np.float32)).reshape(7, dim)
+    for centre in (None, mu):
+        x, q = B.lbp_normalize_features(ctx, dev_u16(cnt), dt, nbins=nbins,
+                                        x_centre=None if centre is None else dev_f32(centre))
+        want = x32 if centre is None else (x32 - mu[None, :dim]).astype(np.float32)
+        if dt == "f32":
+            got = x.cpu().numpy()
+            assert (got[:, :dim].view(np.uint32) == want.view(np.uint32)).all()
+            held = want.astype(np.float64)
+        elif dt == "fp8":
+            got = x.cpu().numpy()
+            codes = orc.f32_to_e4m3((want * np.float32(448.0)).astype(np.float32))
+            assert (got[:, :dim] == codes).all()
+            held = orc.e4m3_to_f64(codes) / 448.0
+        else:
+            got = host_u16(x.view(torch.int16))
+            hi = orc.f32_to_bf16(want)
+            hf = (hi.astype(np.uint32) << 16).view(np.float32)
+            held = hf.astype(np.float64)
+            if dt == "bf16x3":
+                lo = orc.f32_to_bf16((want - hf).astype(np.float32))
+                assert (got[1][:, :dim] == lo).all()
+                held = held + (lo.astype(np.uint32) << 16).view(np.float32)
+                assert not got[1][:, dim:].any()
+                got = got[0]
+            assert (got[:, :dim] == hi).all()
+        assert not got[:, dim:].any()
+        # fp32 sums of at most 2^17 squares: well inside 1e-5 relative
+        assert np.allclose(q.cpu().numpy(), (held ** 2).sum(1), rtol=1e-5, atol=1e-30)
+    assert ctx.status() == 0
+
+
 @pytest.mark.parametrize("n,k_pad", [(2, 7), (65, 128), (200, 531), (700, 256), (2100, 48), (2100, 50)])
 def test_kernel_matrix_and_smo_of_every_size(B, ctx, orc, n, k_pad):
     """Training on few and many rows (one to sixteen rows per thread, one tile per CTA and tiles
