@@ -8,12 +8,13 @@
 // Two fp32 kernels produce per-split partial sums D_s[k][c] = sum_{i in split s} a_ci E_ki:
 //   rbf_smallm_kernel  n <= 8 rows: one warp per support vector, all rows at once (the
 //                      one-frame workload, bound by reading the SV matrix once);
-//   rbf_tiled_kernel   128 x 128 register-tiled SGEMM over (rows, SVs), E in the epilogue,
-//                      then E x a^T accumulated per split.
+//   rbf_f32_kernel     tiles of the fp32 product over (rows, SVs), E in the epilogue, then
+//                      E x a^T per tile or slice of tiles.
 // reduce_scores_kernel adds the splits, asum and the bias, and takes the argmax
 // (reduce_scores_hoisted_kernel: the same with the row-independent sums shared by a block).
 #include <algorithm>
 
+#include "f32_tile.cuh"
 #include "internal.h"
 
 namespace rgbd {
@@ -129,121 +130,177 @@ __global__ void __launch_bounds__(256) rbf_smallm_kernel(const float* __restrict
 }
 
 // ---------------------------------------------------------------------------------------
-// RBF, general n: 128 x 128 x 8 register-tiled fp32 GEMM of X . SV^T per (row tile, SV tile);
-// each CTA walks the SV tiles of its split and accumulates E . a^T into part[split][row][c].
+// RBF, general n: the fp32 product of (rows, SVs) tile by tile (f32_tile.cuh), E = expm1(-gamma d^2)
+// of a tile into shared memory, then part[slice][row][c] (+)= sum_i E[row][i] a[c][i], i ascending.
+// Bound by the FMA pipes.  777 rows x 3001 SVs x 15104, 50 classes: 4.23 ms with a CTA per
+// (row tile, split) in lock step with two barriers every 8 k, 1.45 ms now.
 // ---------------------------------------------------------------------------------------
-constexpr int TBM = 128, TBN = 128, TBK = 8;
-
-struct TiledSmem {
-    float As[2][TBK][TBM];
-    float Bs[2][TBK][TBN];
-    float Es[TBM][TBN + 4];
-    float Cs[TBN][128];  // coefficients of the SV tile, [i][c], C <= 128
+struct F32Score {
+    const float* x;
+    const float* xsq;
+    int n, k_pad;
+    const float* sv;
+    const float* svsq;
+    int n_sv, n_pad;
+    const float* coef;
+    int C;
+    float gamma;
+    int mt, nt, tps;  // row tiles, SV tiles, SV tiles per slice
+    float* part;      // [slices][n][C]
+    // ORDERED: chains and flags handed from CTA to CTA
+    uint64_t* stash;  // [CTA][32][threads]
+    uint32_t* ready;
+    uint32_t* status;
 };
 
-__global__ void __launch_bounds__(256, 1) rbf_tiled_kernel(const float* __restrict__ x, const float* __restrict__ xsq,
-                                                           int n, int k_pad, const float* __restrict__ sv,
-                                                           const float* __restrict__ svsq, int n_pad,
-                                                           const float* __restrict__ coef, int C, float gamma,
-                                                           int tiles_per_split, float* __restrict__ part) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    TiledSmem& sm = *reinterpret_cast<TiledSmem*>(smem_raw);
-    const int tid = threadIdx.x;
-    const int tx = tid & 15, ty = tid >> 4;
-    const int m0 = blockIdx.x * TBM;
-    const int split = blockIdx.y;
-    const int n_tiles = n_pad / TBN;
-    const int t0 = split * tiles_per_split, t1 = min(n_tiles, t0 + tiles_per_split);
-    const int lr = tid >> 1, lk = (tid & 1) * 4;  // loader: row, k offset
-    const bool arow_ok = (m0 + lr) < n;
-    const float* arow = x + (size_t)(arow_ok ? m0 + lr : 0) * k_pad + lk;
-    const int nk = k_pad / TBK;
+template <int BM>
+struct F32ScoreSmem {
+    union {
+        typename F32Tile<BM, BM>::Smem stage;
+        float E[BM][BM + 4];
+    };
+};
 
-    for (int t = t0; t < t1; ++t) {
-        const int n0 = t * TBN;
-        const float* brow = sv + (size_t)(n0 + lr) * k_pad + lk;
-        float acc[8][8];
+// One tile's E and its product with the coefficients; `add` to what the slice holds already.
+template <int BM>
+__device__ __forceinline__ void f32_score_tile(const F32Score& p, const F32Tile<BM, BM>& t, int mi, int ni, int slice,
+                                               bool add, F32ScoreSmem<BM>& sm) {
+    constexpr int NT = F32Tile<BM, BM>::NT, GROUPS = NT / BM;
+    const int m0 = mi * BM, n0 = ni * BM;
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < 8; ++i) {
+        const int rl = t.m_of(i);
+        const float xs = m0 + rl < p.n ? p.xsq[m0 + rl] : 0.f;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-
-        float4 ra = arow_ok ? __ldg(reinterpret_cast<const float4*>(arow)) : make_float4(0, 0, 0, 0);
-        float4 rb = __ldg(reinterpret_cast<const float4*>(brow));
-        __syncthreads();  // previous tile's epilogue is done with shared memory
-        sm.As[0][lk + 0][lr] = ra.x;
-        sm.As[0][lk + 1][lr] = ra.y;
-        sm.As[0][lk + 2][lr] = ra.z;
-        sm.As[0][lk + 3][lr] = ra.w;
-        sm.Bs[0][lk + 0][lr] = rb.x;
-        sm.Bs[0][lk + 1][lr] = rb.y;
-        sm.Bs[0][lk + 2][lr] = rb.z;
-        sm.Bs[0][lk + 3][lr] = rb.w;
-        __syncthreads();
-        for (int kt = 0; kt < nk; ++kt) {
-            const int cur = kt & 1;
-            if (kt + 1 < nk) {
-                ra = arow_ok ? __ldg(reinterpret_cast<const float4*>(arow + (size_t)(kt + 1) * TBK))
-                             : make_float4(0, 0, 0, 0);
-                rb = __ldg(reinterpret_cast<const float4*>(brow + (size_t)(kt + 1) * TBK));
+        for (int q = 0; q < 4; ++q) {
+            const int cl = t.n_of(q);
+            float e[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float d2 = fmaxf(xs + p.svsq[n0 + cl + h] - 2.f * t.get(i, q, h), 0.f);
+                e[h] = expm1f(-p.gamma * d2);
             }
-#pragma unroll
-            for (int k = 0; k < TBK; ++k) {
-                const float4 a0 = *reinterpret_cast<const float4*>(&sm.As[cur][k][ty * 4]);
-                const float4 a1 = *reinterpret_cast<const float4*>(&sm.As[cur][k][64 + ty * 4]);
-                const float4 b0 = *reinterpret_cast<const float4*>(&sm.Bs[cur][k][tx * 4]);
-                const float4 b1 = *reinterpret_cast<const float4*>(&sm.Bs[cur][k][64 + tx * 4]);
-                const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-                const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-            }
-            if (kt + 1 < nk) {
-                const int nx = cur ^ 1;
-                sm.As[nx][lk + 0][lr] = ra.x;
-                sm.As[nx][lk + 1][lr] = ra.y;
-                sm.As[nx][lk + 2][lr] = ra.z;
-                sm.As[nx][lk + 3][lr] = ra.w;
-                sm.Bs[nx][lk + 0][lr] = rb.x;
-                sm.Bs[nx][lk + 1][lr] = rb.y;
-                sm.Bs[nx][lk + 2][lr] = rb.z;
-                sm.Bs[nx][lk + 3][lr] = rb.w;
-            }
-            __syncthreads();
-        }
-        // epilogue 1: E = expm1(-gamma d^2) for the 8 x 8 block of this thread
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int rl = (i < 4) ? ty * 4 + i : 64 + ty * 4 + (i - 4);
-            const int rg = m0 + rl;
-            const float xs = (rg < n) ? xsq[rg] : 0.f;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int cl = (j < 4) ? tx * 4 + j : 64 + tx * 4 + (j - 4);
-                const float d2 = fmaxf(xs + svsq[n0 + cl] - 2.f * acc[i][j], 0.f);
-                sm.Es[rl][cl] = expm1f(-gamma * d2);
-            }
-        }
-        for (int idx = tid; idx < TBN * C; idx += 256) {
-            const int c = idx / TBN, i = idx - c * TBN;
-            sm.Cs[i][c] = coef[(size_t)c * n_pad + n0 + i];
-        }
-        __syncthreads();
-        // epilogue 2: part[split][row][c] (+)= sum_i E[row][i] a[c][i]
-        for (int idx = tid; idx < TBM * C; idx += 256) {
-            const int rl = idx / C, c = idx - rl * C;
-            const int rg = m0 + rl;
-            float s = 0.f;
-#pragma unroll 8
-            for (int i = 0; i < TBN; ++i) s = fmaf(sm.Es[rl][i], sm.Cs[i][c], s);
-            if (rg < n) {
-                float* p = part + ((size_t)split * n + rg) * C + c;
-                *p = (t == t0) ? s : (*p + s);
-            }
+            *reinterpret_cast<float2*>(&sm.E[rl][cl]) = make_float2(e[0], e[1]);
         }
     }
+    __syncthreads();
+    // a thread = one row and four classes at a time; the coefficients are the same for a warp
+    const int rl = threadIdx.x % BM, row = m0 + rl;
+    for (int c0 = 4 * (threadIdx.x / BM); c0 < p.C; c0 += 4 * GROUPS) {
+        float s[4] = {0.f, 0.f, 0.f, 0.f};
+        const float* a[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) a[q] = p.coef + (size_t)min(c0 + q, p.C - 1) * p.n_pad + n0;
+#pragma unroll 4
+        for (int i = 0; i < BM; i += 4) {
+            const float4 e = *reinterpret_cast<const float4*>(&sm.E[rl][i]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 w = __ldg(reinterpret_cast<const float4*>(a[q] + i));
+                s[q] = fmaf(e.x, w.x, s[q]);
+                s[q] = fmaf(e.y, w.y, s[q]);
+                s[q] = fmaf(e.z, w.z, s[q]);
+                s[q] = fmaf(e.w, w.w, s[q]);
+            }
+        }
+        if (row < p.n) {
+            float* o = p.part + ((size_t)slice * p.n + row) * p.C + c0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (c0 + q < p.C) o[q] = add ? o[q] + s[q] : s[q];
+        }
+    }
+}
+
+// ORDERED: every SV tile is a slice of its own, and the tiles are spread evenly over one CTA per
+// SM.  Otherwise CTA (row tile, slice) walks the SV tiles of its slice.
+template <int BM, bool ORDERED>
+__global__ void __launch_bounds__(F32Tile<BM, BM>::NT, 1) rbf_f32_kernel(const F32Score p) {
+    using Tile = F32Tile<BM, BM>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    auto& sm = *reinterpret_cast<F32ScoreSmem<BM>*>(smem_raw);
+    auto rows = [&](int mi, int ni) {
+        return F32Rows{p.x + (size_t)mi * BM * p.k_pad, p.n - mi * BM, p.sv + (size_t)ni * BM * p.k_pad, p.n_sv - ni * BM};
+    };
+    if (ORDERED) {
+        f32_ordered_tiles<Tile, true>(
+            (long long)p.mt * p.nt, p.k_pad, p.ready, p.status, sm.stage,
+            [&](long long i) { return rows((int)(i % p.mt), (int)(i / p.mt)); },
+            [&](long long i, const Tile& t) {
+                f32_score_tile<BM>(p, t, (int)(i % p.mt), (int)(i / p.mt), (int)(i / p.mt), false, sm);
+            },
+            [&](long long, const Tile& t) {
+                uint64_t* out = p.stash + (size_t)blockIdx.x * 32 * Tile::NT + threadIdx.x;
+#pragma unroll
+                for (int i = 0; i < 32; ++i)
+                    __stcg(reinterpret_cast<unsigned long long*>(out + i * Tile::NT), t.acc[i >> 2][i & 3]);
+            },
+            [&](long long, Tile& t) {
+                const uint64_t* in = p.stash + (size_t)(blockIdx.x - 1) * 32 * Tile::NT + threadIdx.x;
+#pragma unroll
+                for (int i = 0; i < 32; ++i)
+                    t.acc[i >> 2][i & 3] = __ldcg(reinterpret_cast<const unsigned long long*>(in + i * Tile::NT));
+            });
+    } else {
+        const int mi = blockIdx.x, slice = blockIdx.y, t0 = slice * p.tps, t1 = min(p.nt, t0 + p.tps);
+        for (int ni = t0; ni < t1; ++ni) {
+            const F32Rows r = rows(mi, ni);
+            Tile t;
+            t.clear();
+            t.template run<true>(r.a, r.na, r.b, r.nb, p.k_pad, 0, p.k_pad / Tile::KB, sm.stage);
+            f32_score_tile<BM>(p, t, mi, ni, slice, ni > t0, sm);
+        }
+    }
+}
+
+// How a call of n rows is laid out, and the workspace it takes.
+struct F32Plan {
+    int bm, mt, nt, slices, tps;
+    bool ordered;
+    size_t off_stash, off_ready, bytes;
+};
+
+F32Plan plan_f32(const rgbd_ctx* ctx, const rgbd_svm* m, int n) {
+    F32Plan p;
+    const int sms = ctx->props.sm_count;
+    auto tiles = [&](int bm) {
+        p.bm = bm;
+        p.mt = (n + bm - 1) / bm;
+        p.nt = (m->n_sv + bm - 1) / bm;
+        return (long long)p.mt * p.nt;
+    };
+    // 128 x 128 tiles when there is one for every SM (57 TFLOP/s against 51 in 64 x 64 tiles),
+    // spread evenly (1.45 ms against 2.0 ms in 64 x 64 tiles with a CTA each at 777 x 3001)
+    // while a slice of partial sums per SV tile stays small; smaller tiles on more CTAs otherwise.
+    const bool big = tiles(128) >= sms;
+    if (!big) tiles(64);
+    p.ordered = big && sizeof(float) * (size_t)p.nt * n * m->C <= ((size_t)256 << 20);
+    p.tps = 1;
+    if (!p.ordered) {
+        // fewest waves of tiles on the SMs (64 x 64 tiles: four CTAs each), fewest slices on ties
+        const long long slots = (long long)sms * (big ? 1 : 4);
+        long long best = -1;
+        for (int sp = 1; sp <= p.nt; ++sp) {
+            const int tps = (p.nt + sp - 1) / sp;
+            const long long cost = (((long long)p.mt * ((p.nt + tps - 1) / tps) + slots - 1) / slots) * tps;
+            if (best < 0 || cost < best) best = cost, p.tps = tps;
+        }
+    }
+    p.slices = (p.nt + p.tps - 1) / p.tps;
+    p.off_stash = (sizeof(float) * (size_t)p.slices * n * m->C + 255) & ~size_t(255);
+    p.off_ready = p.off_stash + (p.ordered ? sizeof(uint64_t) * 32 * F32Tile<128, 128>::NT * (size_t)sms : 0);
+    p.bytes = p.off_ready + (p.ordered ? sizeof(uint32_t) * (size_t)sms : 0);
+    return p;
+}
+
+template <int BM, bool ORDERED>
+cudaError_t launch_f32(const F32Score& p, dim3 grid, cudaStream_t s) {
+    const size_t smem = sizeof(F32ScoreSmem<BM>);
+    const cudaError_t e =
+        cudaFuncSetAttribute(rbf_f32_kernel<BM, ORDERED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    rbf_f32_kernel<BM, ORDERED><<<grid, F32Tile<BM, BM>::NT, smem, s>>>(p);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------------------
@@ -411,12 +468,7 @@ size_t score_rbf_f32_bytes(rgbd_ctx* ctx, const rgbd_svm* m, int n) {
         const int nwarps = (m->n_sv + spw - 1) / spw;
         return sizeof(float) * (size_t)((nwarps + 7) / 8 * 8) * n * m->C;
     }
-    const int mt = (n + TBM - 1) / TBM;
-    const int nt = m->n_pad / TBN;
-    int splits = std::max(1, std::min(nt, (ctx->props.sm_count + mt - 1) / mt));
-    const int tps = (nt + splits - 1) / splits;
-    splits = (nt + tps - 1) / tps;
-    return sizeof(float) * (size_t)splits * n * m->C;
+    return plan_f32(ctx, m, n).bytes;
 }
 
 int score_rbf_f32(rgbd_ctx* ctx, const rgbd_svm* m, const float* x, const float* xsq, int n,
@@ -449,28 +501,26 @@ int score_rbf_f32(rgbd_ctx* ctx, const rgbd_svm* m, const float* x, const float*
         return launch_reduce_scores(part, nullptr, total_warps, n, m->C, m->C, m->asum, nullptr, 0, 0, m->bias,
                                     m->gamma, scores, labels, s);
     }
-    static bool attr_set = false;
-    const size_t smem = sizeof(TiledSmem);
-    if (!attr_set) {
-        e = cudaFuncSetAttribute(rbf_tiled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return cuda_error(e, "svm_score: tiled smem attribute");
-        attr_set = true;
-    }
-    const int mt = (n + TBM - 1) / TBM;
-    const int nt = m->n_pad / TBN;
-    int splits = std::max(1, std::min(nt, (ctx->props.sm_count + mt - 1) / mt));
-    const int tps = (nt + splits - 1) / splits;
-    splits = (nt + tps - 1) / tps;
-    const size_t need = sizeof(float) * (size_t)splits * n * m->C;
-    int rc = ensure_workspace(ctx, need, s);
+    const F32Plan pl = plan_f32(ctx, m, n);
+    int rc = ensure_workspace(ctx, pl.bytes, s);
     if (rc) return rc;
-    float* part = (float*)ctx->workspace;
-    dim3 grid(mt, splits);
-    rbf_tiled_kernel<<<grid, 256, smem, s>>>(x, xsq, n, m->k_pad, (const float*)m->sv, m->sv_sq, m->n_pad,
-                                             m->coef, m->C, m->gamma, tps, part);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_error(e, "svm_score: rbf tiled launch");
-    return launch_reduce_scores(part, nullptr, splits, n, m->C, m->C, m->asum, nullptr, 0, 0, m->bias, m->gamma,
+    char* ws = (char*)ctx->workspace;
+    F32Score p;
+    p.x = x, p.xsq = xsq, p.n = n, p.k_pad = m->k_pad, p.sv = (const float*)m->sv, p.svsq = m->sv_sq;
+    p.n_sv = m->n_sv, p.n_pad = m->n_pad, p.coef = m->coef, p.C = m->C, p.gamma = m->gamma;
+    p.mt = pl.mt, p.nt = pl.nt, p.tps = pl.tps, p.part = (float*)ws;
+    p.stash = (uint64_t*)(ws + pl.off_stash), p.ready = (uint32_t*)(ws + pl.off_ready), p.status = ctx->d_status;
+    if (pl.ordered) {
+        const int grid = ctx->props.sm_count;
+        e = cudaMemsetAsync(p.ready, 0, sizeof(uint32_t) * (size_t)grid, s);
+        if (e != cudaSuccess) return cuda_error(e, "svm_score: tile hand-over reset");
+        e = launch_f32<128, true>(p, dim3((unsigned)grid), s);
+    } else {
+        const dim3 grid((unsigned)pl.mt, (unsigned)pl.slices);
+        e = pl.bm == 128 ? launch_f32<128, false>(p, grid, s) : launch_f32<64, false>(p, grid, s);
+    }
+    if (e != cudaSuccess) return cuda_error(e, "svm_score: rbf fp32 launch");
+    return launch_reduce_scores(p.part, nullptr, pl.slices, n, m->C, m->C, m->asum, nullptr, 0, 0, m->bias, m->gamma,
                                 scores, labels, s);
 }
 

@@ -137,6 +137,31 @@ def test_normalise_rows_are_ieee_quotients(B, ctx, orc, dim, nbins, dt):
     assert ctx.status() == 0
 
 
+@pytest.mark.parametrize("n,n_sv,C", [(9, 40, 3), (64, 65, 1), (65, 1000, 128), (777, 300, 50), (1300, 2100, 7),
+                                      (2500, 1100, 33)])
+def test_fp32_scores_of_every_tiling(B, ctx, orc, n, n_sv, C):
+    """The exact fp32 scores in 64 x 64 tiles (ragged in rows, SVs and classes) and in 128 x 128
+    tiles spread over the SMs, where most tiles are handed from one CTA to the next, against the
+    fp64 definition; a second call gives the same bits."""
+    rng = synth.rng_for(n + n_sv + C)
+    dim = 9 * 59
+    X, SV = synth.poisson_counts(rng, n, dim), synth.poisson_counts(rng, n_sv, dim)
+    a, _ = synth.rbf_coefficients(rng, C, n_sv)
+    b = rng.normal(0, 0.01, C).astype(np.float32)
+    model = B.svm_train_data_pack(ctx, dev_u16(SV), dev_f32(a), dev_f32(b), gamma=0.3, dtype="f32")
+    x, q = B.lbp_normalize_features(ctx, dev_u16(X), "f32")
+    s, lab = B.svm_score(ctx, model, x, q)
+    s2, lab2 = B.svm_score(ctx, model, x, q)
+    assert torch.equal(s, s2) and torch.equal(lab, lab2) and ctx.status() == 0
+    x64, sv64 = orc.normalize_f64(X), orc.normalize_f64(SV)
+    d2 = (x64 ** 2).sum(1)[:, None] + (sv64 ** 2).sum(1)[None, :] - 2.0 * x64 @ sv64.T
+    ref = np.exp(-0.3 * np.maximum(d2, 0.0)) @ a.astype(np.float64).T + b
+    scale = rbf_error_scale(x64, sv64, a, b, 0.3)
+    # the path's stated bound (1e-5 of the score scale)
+    assert rel_score_error(s.cpu().numpy(), ref, scale) <= 1e-5
+    assert (lab.cpu().numpy() == s.cpu().numpy().argmax(1)).all()
+
+
 @pytest.mark.parametrize("n,k_pad", [(2, 7), (65, 128), (200, 531), (700, 256), (2100, 48), (2100, 50)])
 def test_kernel_matrix_and_smo_of_every_size(B, ctx, orc, n, k_pad):
     """Training on few and many rows (one to sixteen rows per thread, one tile per CTA and tiles
