@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kCropThreads) crop_rect_kernel(const CropArgs 
     extern __shared__ __align__(16) unsigned char crop_smem[];
     uint4* cm = reinterpret_cast<uint4*>(crop_smem);                  // [2][ow4]: taps of a column pair
     uint32_t* nn = reinterpret_cast<uint32_t*>(cm + 2 * a.ow4);       // [2][ow4]: its nearest columns
-    uint2* rm = reinterpret_cast<uint2*>(nn + 2 * a.ow4);             // [rows]
+    uint4* rm = reinterpret_cast<uint4*>(crop_smem + (((sizeof(uint4) + sizeof(uint32_t)) * 2 * (size_t)a.ow4 + 15) & ~size_t(15)));  // [rows]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int v0 = blockIdx.x * a.rows, v1 = min(a.oh, v0 + a.rows);
     const int lpr = 1 << a.lanes_log2, rpw = 32 >> a.lanes_log2;      // lanes per row, rows per warp
@@ -72,75 +72,28 @@ __global__ void __launch_bounds__(kCropThreads) crop_rect_kernel(const CropArgs 
         }
         const uint8_t* gsrc = a.grey + (size_t)r.frame * a.H * a.W;
         const uint16_t* dsrc = a.depth + (size_t)r.frame * a.H * a.W;
-        const bool pair_win = r.w <= 2 * a.ow && (a.W & 3) == 0 && a.W >= 8 &&
-                              (reinterpret_cast<size_t>(a.grey) & 3) == 0;
+        const bool win = windows(r.w, a.ow, a.grey, a.W);
         __syncthreads();  // the taps of the rect before are no longer read
         for (int i = tid; i < 2 * a.ow4 + (v1 - v0); i += kCropThreads) {
-            if (i < 2 * a.ow4) {  // columns 2i, 2i + 1 (past the crop's edge: its last column again)
-                const uint2 t0 = make_tap(rect_coord_q16(r.x, r.w, a.ow, min(2 * i, a.ow - 1)), a.W);
-                const uint2 t1 = make_tap(rect_coord_q16(r.x, r.w, a.ow, min(2 * i + 1, a.ow - 1)), a.W);
-                uint4 c = make_uint4(t0.x, 0u, t1.x, 0u);
-                if (pair_win) {
-                    // .x / .z = byte selector (o, o + dx, o) of each column in the window that starts at
-                    // byte wb (kept above .x's selector), .y / .w = byte weights (255 - fx, fx, 1, 0):
-                    // a permute and a dot product give 256 p(o) + fx (p(o + dx) - p(o)).  Neighbouring
-                    // taps are at most 2 apart, so every offset is at most 7.
-                    const uint32_t wb = min(t0.x & 0xFFFCu, (uint32_t)a.W - 8u);
-                    auto sel = [&](uint32_t t) {
-                        const uint32_t o = (t & 0xFFFFu) - wb, od = o + ((t >> 16) & 1u);
-                        return o | (od << 4) | (o << 8);
-                    };
-                    auto wts = [](uint32_t t) { return (255u - (t >> 24)) | ((t >> 24) << 8) | (1u << 16); };
-                    c = make_uint4(sel(t0.x) | (wb << 16), wts(t0.x), sel(t1.x), wts(t1.x));
-                }
+            if (i < 2 * a.ow4) {
+                const PairTaps p = make_pair_taps(r.x, r.w, a.ow, i, a.W, win);
                 const int at = (i & 1) * a.ow4 + (i >> 1);
-                cm[at] = c;
-                nn[at] = t0.y | (t1.y << 16);
+                cm[at] = p.c;
+                nn[at] = p.nearest;
             } else {
                 const int v = i - 2 * a.ow4;
-                rm[v] = make_tap(rect_coord_q16(r.y, r.h, a.oh, v0 + v), a.H);
+                rm[v] = make_row_taps(r.y, r.h, a.oh, v0 + v, a.H, a.W);
             }
         }
         __syncthreads();
+#pragma unroll 2
         for (int v = vl; v < v1; v += vstep) {
-            const uint2 ry = rm[v - v0];
-            const uint32_t fy = ry.x >> 24;
-            const uint8_t* g0 = gsrc + (size_t)(ry.x & 0xFFFFu) * a.W;
-            const uint8_t* g1 = g0 + (size_t)((ry.x >> 16) & 1u) * a.W;
-            const uint16_t* drow = dsrc + (size_t)ry.y * a.W;
+            const uint4 ry = rm[v - v0];
             for (int q = ql; q < a.ow4; q += lpr) {
-                uint32_t acc[4], dv[4];  // acc: the grey value in byte 2
-#pragma unroll
-                for (int e2 = 0; e2 < 2; ++e2) {
-                    const uint4 c = cm[e2 * a.ow4 + q];
-                    const uint32_t cols = nn[e2 * a.ow4 + q];
-                    if (pair_win) {
-                        const uint32_t* w0 = reinterpret_cast<const uint32_t*>(g0 + (c.x >> 16));
-                        const uint32_t* w1 = reinterpret_cast<const uint32_t*>(g1 + (c.x >> 16));
-                        const uint32_t a0 = __ldg(w0), a1 = __ldg(w0 + 1), b0 = __ldg(w1), b1 = __ldg(w1 + 1);
-#pragma unroll
-                        for (int j = 0; j < 2; ++j) {
-                            const uint32_t h0 = __dp4a(__byte_perm(a0, a1, j ? c.z : c.x), j ? c.w : c.y, 0u);
-                            const uint32_t h1 = __dp4a(__byte_perm(b0, b1, j ? c.z : c.x), j ? c.w : c.y, 0u);
-                            acc[2 * e2 + j] = h0 * (256u - fy) + (h1 * fy + 32768u);
-                        }
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 2; ++j) {
-                            const uint32_t t = j ? c.z : c.x;
-                            const uint32_t xa = t & 0xFFFFu, dx = (t >> 16) & 1u, fx = t >> 24;
-                            const uint32_t h0 = (256u - fx) * __ldg(g0 + xa) + fx * __ldg(g0 + xa + dx);
-                            const uint32_t h1 = (256u - fx) * __ldg(g1 + xa) + fx * __ldg(g1 + xa + dx);
-                            acc[2 * e2 + j] = h0 * (256u - fy) + (h1 * fy + 32768u);
-                        }
-                    }
-                    dv[2 * e2] = __ldg(drow + (cols & 0xFFFFu));
-                    dv[2 * e2 + 1] = __ldg(drow + (cols >> 16));
-                }
-                const uint32_t gw = __byte_perm(__byte_perm(acc[0], acc[1], 0x0062u),
-                                                __byte_perm(acc[2], acc[3], 0x0062u), 0x5410u);
-                store_group(a, crop0 + (size_t)v * a.ow + 4 * q, 4 * q, gw, dv[0] | (dv[1] << 16),
-                            dv[2] | (dv[3] << 16));
+                const PairTaps pair[2] = {{cm[q], nn[q]}, {cm[a.ow4 + q], nn[a.ow4 + q]}};
+                uint32_t gw, d01, d23;
+                sample_group(gsrc, dsrc, ry, pair, win, gw, d01, d23);
+                store_group(a, crop0 + (size_t)v * a.ow + 4 * q, 4 * q, gw, d01, d23);
             }
         }
     }
@@ -199,11 +152,12 @@ int launch_crop_affine(rgbd_ctx* ctx, const uint8_t* grey, const uint16_t* depth
     const long long strips = std::max(1LL, std::min((want + n - 1) / n, (long long)(out_h + pass - 1) / pass));
     a.rows = (int)((out_h + strips - 1) / strips);
     const dim3 grid((unsigned)((out_h + a.rows - 1) / a.rows), (unsigned)std::min(n, 65535));
-    const size_t smem = (sizeof(uint4) + sizeof(uint32_t)) * 2 * (size_t)a.ow4 + sizeof(uint2) * (size_t)a.rows;
+    const size_t smem = (((sizeof(uint4) + sizeof(uint32_t)) * 2 * (size_t)a.ow4 + 15) & ~size_t(15)) +
+                        sizeof(uint4) * (size_t)a.rows;
     if (affine) {
         crop_affine_kernel<<<grid, kCropThreads, 0, s>>>(a);
     } else {
-        // crops up to 4096 columns and rows: 41 KB of column taps and 33 KB of row taps at most
+        // crops up to 4096 columns and rows: 41 KB of column taps and 66 KB of row taps at most
         if (smem > 48 * 1024) {
             const cudaError_t e =
                 cudaFuncSetAttribute(crop_rect_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

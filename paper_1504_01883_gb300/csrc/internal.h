@@ -127,6 +127,8 @@ struct LbpArgs {
     uint32_t* face_counter;  // NULL: faces strided over CTAs; else a zeroed queue counter
 };
 int launch_lbp_fused(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s);
+// The 0-255 face histogram (RGBD_LBP_FACE_HIST256).
+int launch_face256(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s);
 
 // plane: RGBD_DT_BF16X3 offset (elements) of the lo plane; 0 means n * k_pad.
 int launch_normalize(const uint16_t* feats, int n, int dim, int nbins, int x_dtype, void* x_out,

@@ -34,6 +34,7 @@
 #include <algorithm>
 
 #include "internal.h"
+#include "lbp_codes.cuh"
 #include "resample.cuh"
 
 namespace rgbd {
@@ -63,15 +64,6 @@ __device__ __forceinline__ void prefetch_rect_rows(const uint8_t* grey, const ui
             if (pp >= last - 127) break;
         }
     }
-}
-
-// ---------------------------------------------------------------------------------------
-// A3 helper: byte-SIMD "a > b" (or >=) on four packed pixels.  cb = (b & 0x7f7f7f7f) + 1 per
-// byte for the strict test, without the +1 for >=.  Result: 0x80 in each byte where it holds.
-// ---------------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t cmp_msb(uint32_t a, uint32_t b, uint32_t cb) {
-    const uint32_t d = (a | 0x80808080u) - cb;  // per byte: low 7 bits of a vs b, no borrows
-    return ((a & ~b) | (~(a ^ b) & d)) & 0x80808080u;
 }
 
 // Slot of quotient-table entry i = 128 n + h: bits 1..5 of h are XOR-ed with the low bits of n.
@@ -795,244 +787,6 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::MINB) lbp_fused_
     }
 }
 
-// ---------------------------------------------------------------------------------------
-// Section 3's own descriptor: one 0-255 histogram of the raw LBP codes per face (crop up to
-// 255 x 255; the paper uses 200 x 200).  Same resample, median mask and codes as the fused
-// kernel, written plainly (one pixel per thread step): this is the paper-literal variant, not
-// the throughput path.  One CTA of 1024 threads per face, persistent over faces.
-// ---------------------------------------------------------------------------------------
-constexpr int F256_THREADS = 1024;
-constexpr int F256_COPIES = 8;  // histogram copies (warp % 8) to spread same-code atomics
-
-__global__ void __launch_bounds__(F256_THREADS, 1) lbp_face256_kernel(LbpArgs a) {
-    const int S = a.crop, SS = S * S;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    uint16_t* depth = reinterpret_cast<uint16_t*>(smem_raw);           // [SS], later the mask bytes
-    uint8_t* grey = smem_raw + 2 * ((SS + 7) & ~7);                     // [SS]
-    uint32_t* hist = reinterpret_cast<uint32_t*>(grey + ((SS + 15) & ~15));  // [COPIES][256]
-    uint2* colmap = reinterpret_cast<uint2*>(hist + F256_COPIES * 256);     // [S]
-    uint2* rowmap = colmap + S;                                             // [S]
-    uint32_t* h1 = reinterpret_cast<uint32_t*>(rowmap + S);                 // [256]
-    uint32_t* h2 = h1 + 256;                                                // [256]
-    int* info = reinterpret_cast<int*>(h2 + 256);                           // [4]
-    float* red = reinterpret_cast<float*>(info + 4);                        // [32]
-    uint8_t* mask = reinterpret_cast<uint8_t*>(depth);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool strict = !(a.flags & RGBD_LBP_GE);
-    const bool nbr_ignore = (a.flags & RGBD_LBP_NBR_IGNORE_MASK) != 0;
-    const int x_dtype = a.x_out ? a.x_dtype : 0;
-    const int iters = (SS + F256_THREADS - 1) / F256_THREADS;
-
-    for (int face = blockIdx.x; face < a.n; face += gridDim.x) {
-        __syncthreads();
-        bool ok = true;
-        rgbd_rect r = {0, 0, 0, S, S};
-        const uint8_t* gsrc = a.grey;
-        const uint16_t* dsrc = a.depth;
-        int64_t aff[6] = {0, 0, 0, 0, 0, 0};
-        if (a.rects) {
-            r = a.rects[face];
-            ok = r.frame >= 0 && r.frame < a.n_frames && r.w > 0 && r.h > 0;
-            if (!ok && tid == 0) atomicOr(a.status, RGBD_STATUS_BAD_RECT);
-            if (ok) {
-                gsrc += (size_t)r.frame * a.H * a.W;
-                dsrc += (size_t)r.frame * a.H * a.W;
-                if (a.affine) {
-                    for (int i = 0; i < 6; ++i) aff[i] = a.affine[6 * (size_t)face + i];
-                } else {
-                    for (int i = tid; i < 2 * S; i += F256_THREADS) {
-                        if (i < S)
-                            colmap[i] = make_tap(rect_coord_q16(r.x, r.w, S, i), a.W);
-                        else
-                            rowmap[i - S] = make_tap(rect_coord_q16(r.y, r.h, S, i - S), a.H);
-                    }
-                }
-            }
-        } else {
-            gsrc += (size_t)face * SS;
-            dsrc += (size_t)face * SS;
-        }
-        for (int i = tid; i < F256_COPIES * 256; i += F256_THREADS) hist[i] = 0;
-        for (int i = tid; i < 256; i += F256_THREADS) {
-            h1[i] = 0;
-            h2[i] = 0;
-        }
-        __syncthreads();
-        // resample and the depth high-byte histogram
-        for (int it = 0; it < iters; ++it) {
-            const int pidx = tid + it * F256_THREADS;
-            uint32_t d = 0;
-            if (pidx < SS && ok) {
-                const int v = pidx / S, u = pidx - v * S;
-                uint32_t g;
-                if (!a.rects) {
-                    g = gsrc[pidx];
-                    d = dsrc[pidx];
-                } else if (!a.affine) {
-                    const uint2 tx = colmap[u], ty = rowmap[v];
-                    g = bilerp(gsrc, a.W, tx.x, ty.x);
-                    d = __ldg(dsrc + (size_t)ty.y * a.W + tx.y);
-                } else {
-                    const int64_t xq = aff[0] * u + aff[1] * v + aff[2];
-                    const int64_t yq = aff[3] * u + aff[4] * v + aff[5];
-                    const uint2 tx = make_tap(xq, a.W), ty = make_tap(yq, a.H);
-                    g = bilerp(gsrc, a.W, tx.x, ty.x);
-                    d = __ldg(dsrc + (size_t)ty.y * a.W + tx.y);
-                }
-                grey[pidx] = (uint8_t)g;
-            }
-            if (pidx < SS) depth[pidx] = (uint16_t)d;
-            if (d) atomicAdd(&h1[d >> 8], 1u);
-        }
-        __syncthreads();
-        // lower median of the non-zero depths (radix select over the high, then low byte)
-        if (warp == 0) {
-            uint32_t c = 0;
-            for (int i = lane; i < 256; i += 32) c += h1[i];
-            for (int off = 16; off > 0; off >>= 1) c += __shfl_xor_sync(FULL, c, off);
-            if (lane == 0) {
-                int b1 = -1, k1 = 0;
-                if (c > 0) {
-                    const uint32_t k = (c - 1) / 2;
-                    uint32_t acc = 0;
-                    for (int b = 0; b < 256; ++b) {
-                        if (k < acc + h1[b]) {
-                            b1 = b;
-                            k1 = (int)(k - acc);
-                            break;
-                        }
-                        acc += h1[b];
-                    }
-                }
-                info[0] = b1;
-                info[1] = k1;
-            }
-        }
-        __syncthreads();
-        const int b1 = info[0];
-        int med = -1;
-        if (b1 >= 0) {
-            for (int pidx = tid; pidx < SS; pidx += F256_THREADS) {
-                const uint32_t d = depth[pidx];
-                if (d && (int)(d >> 8) == b1) atomicAdd(&h2[d & 255u], 1u);
-            }
-            __syncthreads();
-            if (tid == 0) {
-                const uint32_t k1 = (uint32_t)info[1];
-                uint32_t acc = 0;
-                int b2 = 0;
-                for (int b = 0; b < 256; ++b) {
-                    if (k1 < acc + h2[b]) {
-                        b2 = b;
-                        break;
-                    }
-                    acc += h2[b];
-                }
-                info[2] = b1 * 256 + b2;
-            }
-            __syncthreads();
-            med = info[2];
-        }
-        // mask: valid bits to registers first, then bytes over the depth buffer
-        uint32_t vbits[4] = {0, 0, 0, 0};  // up to 128 pixels per thread (255^2 / 1024 < 64)
-        for (int it = 0; it < iters; ++it) {
-            const int pidx = tid + it * F256_THREADS;
-            if (pidx < SS) {
-                const int d = depth[pidx];
-                const int diff = d - med;
-                if (med >= 0 && d != 0 && diff < a.mask_mm && -diff < a.mask_mm) vbits[it >> 5] |= 1u << (it & 31);
-            }
-        }
-        __syncthreads();
-        for (int it = 0; it < iters; ++it) {
-            const int pidx = tid + it * F256_THREADS;
-            if (pidx < SS) mask[pidx] = (uint8_t)((vbits[it >> 5] >> (it & 31)) & 1u);
-        }
-        __syncthreads();
-        // codes and the 0-255 histogram
-        uint32_t* myh = hist + (warp % F256_COPIES) * 256;
-        for (int pidx = tid; pidx < SS; pidx += F256_THREADS) {
-            if (!mask[pidx]) continue;
-            const int i = pidx / S, j = pidx - i * S;
-            const int gc = grey[pidx];
-            int code = 0;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                // ring p0..p7 clockwise from the top-left neighbour, y down
-                const int dx = (q == 0 || q == 6 || q == 7) ? -1 : ((q == 1 || q == 5) ? 0 : 1);
-                const int dy = (q <= 2) ? -1 : ((q == 3 || q == 7) ? 0 : 1);
-                const int rr = min(max(i + dy, 0), S - 1), cc = min(max(j + dx, 0), S - 1);
-                const int gp = grey[rr * S + cc];
-                const bool nb = nbr_ignore || mask[rr * S + cc];
-                if (nb && (strict ? gp > gc : gp >= gc)) code |= 1 << q;
-            }
-            atomicAdd(&myh[code], 1u);
-        }
-        __syncthreads();
-        // merge the copies, write counts, the normalised row and its squared norm
-        uint32_t cnt = 0;
-        if (tid < 256) {
-            for (int k = 0; k < F256_COPIES; ++k) cnt += hist[k * 256 + tid];
-            hist[tid] = cnt;  // copy 0 now holds the totals (each thread owns its bin)
-        }
-        __syncthreads();
-        if (warp == 0) {
-            uint32_t t = 0;
-            for (int i = lane; i < 256; i += 32) t += hist[i];
-            for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(FULL, t, off);
-            if (lane == 0) info[3] = (int)t;
-        }
-        __syncthreads();
-        const uint32_t nvalid = (uint32_t)info[3];
-        float sq = 0.f;
-        const int len = x_dtype ? a.k_pad : 256;
-        for (int j = tid; j < len; j += F256_THREADS) {
-            const uint32_t h = j < 256 ? hist[j] : 0u;
-            if (j < 256 && a.feats) a.feats[(size_t)face * 256 + j] = (uint16_t)h;
-            if (x_dtype) {
-                float x = (j < 256 && nvalid) ? (float)h / (float)nvalid : 0.f;
-                if (a.x_centre && j < 256) x = __fsub_rn(x, a.x_centre[j]);
-                const size_t idx = (size_t)face * a.k_pad + j;
-                float qv = x;
-                if (x_dtype == RGBD_DT_BF16) {
-                    const __nv_bfloat16 b = __float2bfloat16_rn(x);
-                    reinterpret_cast<uint16_t*>(a.x_out)[idx] = __bfloat16_as_ushort(b);
-                    qv = __bfloat162float(b);
-                } else if (x_dtype == RGBD_DT_BF16X3) {
-                    const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-                    const __nv_bfloat16 lo = __float2bfloat16_rn(x - __bfloat162float(hi));
-                    reinterpret_cast<uint16_t*>(a.x_out)[idx] = __bfloat16_as_ushort(hi);
-                    reinterpret_cast<uint16_t*>(a.x_out)[idx + a.x_plane] = __bfloat16_as_ushort(lo);
-                    qv = __bfloat162float(hi) + __bfloat162float(lo);
-                } else if (x_dtype == RGBD_DT_FP8) {
-                    const __nv_fp8_e4m3 b(x * a.x_scale);
-                    reinterpret_cast<uint8_t*>(a.x_out)[idx] = b.__x;
-                    qv = static_cast<float>(b) * (1.0f / a.x_scale);
-                } else {
-                    reinterpret_cast<float*>(a.x_out)[idx] = x;
-                }
-                sq = fmaf(qv, qv, sq);
-            }
-        }
-        if (a.xsq) {
-            for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(FULL, sq, off);
-            if (lane == 0) red[warp] = sq;
-            __syncthreads();
-            if (tid == 0) {
-                float t = 0.f;
-                for (int w = 0; w < F256_THREADS / 32; ++w) t += red[w];
-                a.xsq[face] = t;
-            }
-        }
-    }
-}
-
-size_t face256_smem(int S) {
-    const size_t SS = (size_t)S * S;
-    return 2 * ((SS + 7) & ~size_t(7)) + ((SS + 15) & ~size_t(15)) + 4 * F256_COPIES * 256 + 2 * 8 * (size_t)S +
-           4 * 512 + 16 + 4 * 32;
-}
-
 template <int S, int TPC>
 int launch_fused_t(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
     static int blocks_per_sm = -1;
@@ -1064,17 +818,7 @@ int launch_fused_t(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
 }  // namespace
 
 int launch_lbp_fused(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
-    if (a.flags & RGBD_LBP_FACE_HIST256) {
-        const size_t smem = face256_smem(a.crop);
-        cudaError_t e = cudaFuncSetAttribute(lbp_face256_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return cuda_error(e, "lbp_fused_features: 0-255 histogram smem attribute");
-        const int grid = std::min(a.n, ctx->props.sm_count);
-        lbp_face256_kernel<<<grid, F256_THREADS, smem, s>>>(a);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return cuda_error(e, "lbp_fused_features: 0-255 histogram launch");
-        return RGBD_OK;
-    }
+    if (a.flags & RGBD_LBP_FACE_HIST256) return launch_face256(ctx, a, s);
     // tile shape (crops 64 and 128): one thread per cell (tuning value 1), per half cell (2, the
     // default), per quarter cell (3: 1024-thread CTAs, measured 7 % slower even when every face
     // has an SM of its own, and 50 % slower on full batches)

@@ -202,3 +202,36 @@ def test_kernel_matrix_and_smo_of_every_size(B, ctx, orc, n, k_pad):
         free = (alpha[c] > 0) & (alpha[c] < 1)
         if free.any():
             assert abs(bias[c].item() - v[free].mean()) <= 1e-4
+
+
+@pytest.mark.parametrize("crop", [8, 9, 50, 131, 255])
+@pytest.mark.parametrize("flags", [0, 1, 2, 3])
+def test_face_histogram_256_sizes_and_rules(B, ctx, orc, crop, flags):
+    """The 0-255 histogram at the smallest and largest side and at every number of pixels in a row's
+    last word, under every neighbour rule: rects inside and outside frames of even and odd width
+    (one frame all holes), pre-cut crops and a general affine map, bit-exact with the oracle."""
+    fl = flags | B.LBP_FACE_HIST256
+    for W in (200, 203):
+        g, d, r = synth.frames_with_rects(crop + flags + W, 3, 3, 20, 160, H=120, W=W)
+        d[2] = 0
+        want = orc.features_batch(g, d, r, crop, cell=crop, nbins=256, flags=flags)
+        f, x, q = B.lbp_fused_features(ctx, dev_u8(g), dev_u16(d), B.rects_tensor(r), crop=crop, flags=fl,
+                                       x_dtype="bf16")
+        assert (host_u16(f) == want).all(), W
+        x32 = orc.normalize_f32(want, nbins=256)
+        assert (host_u16(x.view(torch.int16))[:, :256] == orc.f32_to_bf16(x32)).all()
+    gc, dc = synth.crops(crop, 2, crop)
+    want = orc.features_batch(gc, dc, None, crop, cell=crop, nbins=256, flags=flags)
+    f, _, _ = B.lbp_fused_features(ctx, dev_u8(gc), dev_u16(dc), None, crop=crop, flags=fl)
+    assert (host_u16(f) == want).all()
+    n = r.shape[0]
+    aff = np.zeros((n, 6), np.int32)
+    for k in range(n):
+        sc = r[k]["w"] / float(crop)
+        aff[k] = [int(0.9 * sc * 65536), int(-0.3 * sc * 65536), int(r[k]["x"] * 65536),
+                  int(0.3 * sc * 65536), int(0.9 * sc * 65536), int(r[k]["y"] * 65536)]
+    want = orc.features_batch(g, d, r, crop, cell=crop, nbins=256, flags=flags, affine=aff)
+    f, _, _ = B.lbp_fused_features(ctx, dev_u8(g), dev_u16(d), B.rects_tensor(r), crop=crop, flags=fl,
+                                   affine=torch.from_numpy(aff).cuda())
+    assert (host_u16(f) == want).all()
+    assert ctx.status() == 0
