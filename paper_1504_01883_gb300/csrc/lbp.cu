@@ -31,7 +31,10 @@
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 
+#include <stddef.h>
+
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.h"
 #include "lbp_codes.cuh"
@@ -74,6 +77,14 @@ __device__ __forceinline__ int qbf_slot(int i) { return i ^ (((i >> 7) & 31) << 
 // The same for two 16-bit indices (count | centres << 7) packed in one word.
 __device__ __forceinline__ uint32_t qbf_slot2(uint32_t w) { return w ^ ((w >> 6) & 0x003E003Eu); }
 
+// bf16 bits of the IEEE single quotient h / n (r = 1 / n rounded; 0 for n = 0): Markstein's one-fma
+// correction of h r, then round to nearest even.
+__device__ __forceinline__ uint16_t bf16_quotient(int n, int h, float r) {
+    const float n_f = (float)n, h_f = (float)h;
+    const float q0 = __fmul_rn(h_f, r);
+    return __bfloat16_as_ushort(__float2bfloat16_rn(__fmaf_rn(__fmaf_rn(-q0, n_f, h_f), r, q0)));
+}
+
 // Tile shape of the fused kernel: TPC threads per 8 x 8 cell (2: one per 4 x 8 half cell, 1: one
 // per cell, 4: one per 4 x 4 quarter cell), so a CTA of NT = TPC (S/8)^2 threads works on one
 // face; each thread resamples IPT groups of 4 crop pixels.  Four threads per cell make 1024-thread
@@ -86,11 +97,18 @@ struct Cfg {
     static constexpr int IPT = S * S / 4 / NT;  // 4-pixel groups per thread
     static constexpr int DIM = G * G * kBins;
     static constexpr int HW = 15;            // histogram words per thread (60 bins / 4)
-    static constexpr int MINB = (S == 128 && TPC <= 2) ? 2 : 1;
+    // CTAs per SM that the registers are to allow (64 to 72 a thread): smaller crops need more of
+    // them to hide the same latencies.  585 faces at 96 x 96: 67 us at one CTA of 206 registers per SM,
+    // 51 us at three.
+    static constexpr int MINB = S == 32 ? 16 : (TPC == 4 ? 1 : (S == 128 ? 2 : (S == 96 ? 3 : 8)));
     static constexpr int RPT = TPC == 4 ? 4 : 8;        // cell rows a thread walks in P5
     static constexpr int WPT = (HW + TPC - 1) / TPC;    // histogram words a thread stages in P6
     static_assert(TPC == 1 || TPC == 2 || TPC == 4, "one, two or four threads per cell");
 };
+
+// Where a face's pixels come from: nowhere (a bad rect), crops cut beforehand, a rect by 8-byte
+// windows or by byte gathers, a general affine map.
+enum { SRC_NONE, SRC_CROPS, SRC_WINDOWS, SRC_RECT, SRC_AFFINE };
 
 template <int S, int TPC = 2>
 struct __align__(16) Smem {
@@ -118,10 +136,13 @@ struct __align__(16) Smem {
     uint16_t lut[257];                 // byte offset of each code's counter in a thread's histogram
                                        // (entry 256: the unused bin 59, where invalid centres go
                                        // under the rules other than the default one)
-    uint16_t qbf[65 * 128];            // bf16 bits of the quotient h / n, entry 128 n + h (n, h <= 64)
+    float rcpn[65];                    // IEEE reciprocals of the centre counts (0 for 0)
+    __align__(16) uint16_t qbf[65 * 128];  // bf16 bits of the quotient h / n, entry 128 n + h (n, h <= 64);
+                                       // last: only launches that use it have it
 };
 
-template <int S, int TPC>
+// TABLE: bf16 quotients from a table in shared memory.
+template <int S, int TPC, bool TABLE>
 __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::MINB) lbp_fused_kernel(LbpArgs a) {
     using C = Cfg<S, TPC>;
     constexpr int IPT = C::IPT;
@@ -149,26 +170,24 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::MINB) lbp_fused_
         }
         if (lane == 0) sm.lut[256] = (uint16_t)(((59 >> 2) * NT) * 4 + (59 & 3));
     }
+    const int x_dtype = a.x_out ? a.x_dtype : 0;
+    const bool centred = a.x_centre != nullptr;
     // Quotient table of the bf16 output: a cell has at most 64 centres, so every normalised value
     // is one of the 65 x 65 quotients h / n (stored at qbf_slot(128 n + h)), computed once per
     // CTA exactly as the other output
     // types compute them (IEEE single quotient by the reciprocal and Markstein's one-fma
     // correction, then round to nearest even bf16).  Entry
     // 128 n + h, so that a staged count with its cell's centre count above it is the index.
-    for (int i = tid; i < 65 * 128; i += NT) {
-        const int n = i >> 7, hh = min(i & 127, 64);
-        const float n_f = (float)n, r_f = n ? __frcp_rn(n_f) : 0.f, h_f = (float)hh;
-        const float q0 = __fmul_rn(h_f, r_f);
-        const float rem = __fmaf_rn(-q0, n_f, h_f);
-        sm.qbf[qbf_slot(i)] = __bfloat16_as_ushort(__float2bfloat16_rn(__fmaf_rn(rem, r_f, q0)));
-    }
+    if (TABLE)
+        for (int i = tid; i < 65 * 128; i += NT)
+            sm.qbf[qbf_slot(i)] = bf16_quotient(i >> 7, min(i & 127, 64), (i >> 7) ? __frcp_rn((float)(i >> 7)) : 0.f);
+    for (int i = tid; i < 65; i += NT) sm.rcpn[i] = i ? __frcp_rn((float)i) : 0.f;
 
     for (int i = tid; i < 65; i += NT) sm.ctab[i] = i < 8 ? 1ull << (8 * i) : 0ull;
 
     const bool strict = !(a.flags & RGBD_LBP_GE);
     const bool nbr_ignore = (a.flags & RGBD_LBP_NBR_IGNORE_MASK) != 0;
     const bool masked_grey = strict && !nbr_ignore;  // the default rule (readings c2, c7)
-    const int x_dtype = a.x_out ? a.x_dtype : 0;
 
     // Faces: the first one by CTA index, then from the launch's queue counter (a CTA that
     // finishes early takes the next face), or strided over the CTAs when there is no counter.
@@ -236,27 +255,29 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::MINB) lbp_fused_
         __syncthreads();
 
         // ---- P1: resample; grey and depth to shared memory, coarse depth histogram ----------
-        // One group of 4 pixels per iteration, not unrolled: each group's gathers are
-        // independent, other warps hide their latency, and the rolled loop keeps the group's
-        // registers free of spills (unrolled, the loop ran 4.5 % slower at 64 registers).
         // The next face is claimed now (the atomic's latency hides behind P1) and published at
         // the end of P1; its rect is copied into shared memory asynchronously during P5.
         int next_face = 0;
         if (tid == 0)
             next_face = a.face_counter ? (int)gridDim.x + (int)atomicAdd(a.face_counter, 1u) : face + (int)gridDim.x;
         unsigned long long cnt8 = 0;  // coarse depth histogram, see below
+        // One group of 4 pixels per iteration, not unrolled: each group's gathers are
+        // independent, other warps hide their latency, and the rolled loop keeps the group's
+        // registers free of spills (unrolled, the loop ran 4.5 % slower at 64 registers, and a
+        // single face, whose code is fetched for it alone, 10 to 20 % slower at 128).
+        auto resample = [&](auto source) {
+            constexpr int SRC = decltype(source)::value;
 #pragma unroll 1
-        for (int k = 0; k < IPT; ++k) {
-            const int item = tid + k * NT;  // = v * SW + q
-            const int v = item / SW, q = item - v * SW;
-            uint32_t gw = 0, d01 = 0, d23 = 0;
-            if (ok) {
-                if (!a.rects) {
+            for (int k = 0; k < IPT; ++k) {
+                const int item = tid + k * NT;  // = v * SW + q
+                const int v = item / SW, q = item - v * SW;
+                uint32_t gw = 0, d01 = 0, d23 = 0;
+                if constexpr (SRC == SRC_CROPS) {
                     gw = __ldg(reinterpret_cast<const uint32_t*>(gsrc) + item);
                     const uint2 dd = __ldg(reinterpret_cast<const uint2*>(dsrc) + item);
                     d01 = dd.x;
                     d23 = dd.y;
-                } else if (!a.affine) {
+                } else if constexpr (SRC == SRC_WINDOWS || SRC == SRC_RECT) {
                     const uint2 rm = sm.rowmap[v];
                     const uint32_t fy = rm.x >> 24;
                     const uint8_t* g0 = gsrc + (size_t)(rm.x & 0xFFFFu) * a.W;
@@ -264,55 +285,50 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::MINB) lbp_fused_
                     const uint16_t* drow = dsrc + (size_t)rm.y * a.W;
                     const uint4* cm4 = reinterpret_cast<const uint4*>(sm.colmap);
                     uint32_t dv[4];
-                    uint32_t accv[4];  // pair windows: (acc + 2^15) per pixel, the rounded value in byte 2
-                    if (pair_win) {
+                    uint32_t accv[4];  // (acc + 2^15) per pixel, the rounded value in byte 2
 #pragma unroll
                     for (int e2 = 0; e2 < 2; ++e2) {
                         const uint4 cc = cm4[e2 * SW + q];  // taps of columns 4q + 2 e2 and + 1
-                        const uint32_t nn = reinterpret_cast<const uint32_t*>(sm.ncol)[e2 * SW + q];
-                        const uint32_t wb = cc.x >> 16;
-                        const uint32_t* wa = reinterpret_cast<const uint32_t*>(g0 + wb);
-                        const uint32_t* wv = reinterpret_cast<const uint32_t*>(g1 + wb);
-                        const uint32_t a0 = __ldg(wa), a1 = __ldg(wa + 1), b0 = __ldg(wv), b1 = __ldg(wv + 1);
+                        if constexpr (SRC == SRC_WINDOWS) {
+                            const uint32_t nn = reinterpret_cast<const uint32_t*>(sm.ncol)[e2 * SW + q];
+                            const uint32_t wb = cc.x >> 16;
+                            const uint32_t* wa = reinterpret_cast<const uint32_t*>(g0 + wb);
+                            const uint32_t* wv = reinterpret_cast<const uint32_t*>(g1 + wb);
+                            const uint32_t a0 = __ldg(wa), a1 = __ldg(wa + 1), b0 = __ldg(wv), b1 = __ldg(wv + 1);
 #pragma unroll
-                        for (int j = 0; j < 2; ++j) {
-                            const uint32_t sel = j ? cc.z : cc.x, wts = j ? cc.w : cc.y;
-                            // h = 256 p0 + fx (p1 - p0) for the two source rows, then
-                            // (256 - fy) h0 + fy h1 = 256 h0 + fy (h1 - h0), exactly
-                            const uint32_t h0 = __dp4a(__byte_perm(a0, a1, sel), wts, 0u);
-                            const uint32_t h1 = __dp4a(__byte_perm(b0, b1, sel), wts, 0u);
-                            const int e = 2 * e2 + j;
-                            accv[e] = h0 * (256u - fy) + (h1 * fy + 32768u);  // < 2^24
-                            dv[e] = __ldg(drow + (j ? (nn >> 16) : (nn & 0xFFFFu)));
+                            for (int j = 0; j < 2; ++j) {
+                                const uint32_t sel = j ? cc.z : cc.x, wts = j ? cc.w : cc.y;
+                                // h = 256 p0 + fx (p1 - p0) for the two source rows, then
+                                // (256 - fy) h0 + fy h1 = 256 h0 + fy (h1 - h0), exactly
+                                const uint32_t h0 = __dp4a(__byte_perm(a0, a1, sel), wts, 0u);
+                                const uint32_t h1 = __dp4a(__byte_perm(b0, b1, sel), wts, 0u);
+                                const int e = 2 * e2 + j;
+                                accv[e] = h0 * (256u - fy) + (h1 * fy + 32768u);  // < 2^24
+                                dv[e] = __ldg(drow + (j ? (nn >> 16) : (nn & 0xFFFFu)));
+                            }
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 2; ++j) {
+                                const uint32_t cx = j ? cc.z : cc.x;
+                                const uint32_t xa = cx & 0xFFFFu, dx = (cx >> 16) & 1u;
+                                const int fx = (int)(cx >> 24);
+                                const int p00 = __ldg(g0 + xa), p01 = __ldg(g0 + xa + dx);
+                                const int p10 = __ldg(g1 + xa), p11 = __ldg(g1 + xa + dx);
+                                // (256 - f) a + f b = 256 a + f (b - a), exactly
+                                const int h0 = (p00 << 8) + fx * (p01 - p00);
+                                const int h1 = (p10 << 8) + fx * (p11 - p10);
+                                const int e = 2 * e2 + j;
+                                accv[e] = (uint32_t)((h0 << 8) + (int)fy * (h1 - h0) + 32768);
+                                dv[e] = __ldg(drow + (j ? cc.w : cc.y));
+                            }
                         }
                     }
                     // byte 2 of each rounded sum is the pixel: gather the four with byte permutes
-                    gw = __byte_perm(__byte_perm(accv[0], accv[1], 0x0062u), __byte_perm(accv[2], accv[3], 0x0062u),
-                                     0x5410u);
-                    } else {
-#pragma unroll
-                    for (int e2 = 0; e2 < 2; ++e2) {
-                        const uint4 cc = cm4[e2 * SW + q];  // taps of columns 4q + 2 e2 and + 1
-#pragma unroll
-                        for (int j = 0; j < 2; ++j) {
-                            const uint32_t cx = j ? cc.z : cc.x;
-                            const uint32_t xa = cx & 0xFFFFu, dx = (cx >> 16) & 1u;
-                            const int fx = (int)(cx >> 24);
-                            const int p00 = __ldg(g0 + xa), p01 = __ldg(g0 + xa + dx);
-                            const int p10 = __ldg(g1 + xa), p11 = __ldg(g1 + xa + dx);
-                            // (256 - f) a + f b = 256 a + f (b - a), exactly
-                            const int h0 = (p00 << 8) + fx * (p01 - p00);
-                            const int h1 = (p10 << 8) + fx * (p11 - p10);
-                            const int acc = (h0 << 8) + (int)fy * (h1 - h0);
-                            const int e = 2 * e2 + j;
-                            gw |= (uint32_t)((acc + 32768) >> 16) << (8 * e);
-                            dv[e] = __ldg(drow + (j ? cc.w : cc.y));
-                        }
-                    }
-                    }
+                    gw = __byte_perm(__byte_perm(accv[0], accv[1], 0x0062u),
+                                     __byte_perm(accv[2], accv[3], 0x0062u), 0x5410u);
                     d01 = dv[0] | (dv[1] << 16);
                     d23 = dv[2] | (dv[3] << 16);
-                } else {
+                } else if constexpr (SRC == SRC_AFFINE) {
                     uint32_t dv[4];
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
@@ -326,17 +342,27 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::MINB) lbp_fused_
                     d01 = dv[0] | (dv[1] << 16);
                     d23 = dv[2] | (dv[3] << 16);
                 }
-            }
-            sm.img[(v + 1) * SP + q + 1] = gw;
-            reinterpret_cast<uint2*>(sm.dep)[item] = make_uint2(d01, d23);
+                sm.img[(v + 1) * SP + q + 1] = gw;
+                reinterpret_cast<uint2*>(sm.dep)[item] = make_uint2(d01, d23);
 #pragma unroll
-            for (int hh = 0; hh < 4; ++hh) {
-                const uint32_t d = ((hh < 2 ? d01 : d23) >> (16 * (hh & 1))) & 0xFFFFu;
-                const uint32_t key = min((d - 1u) >> 10, 64u);  // a hole (d = 0) wraps to 64
-                cnt8 += sm.ctab[key];
-                if (key - 8u < 56u) atomicAdd(&sm.h1[key], 1u);
+                for (int hh = 0; hh < 4; ++hh) {
+                    const uint32_t d = ((hh < 2 ? d01 : d23) >> (16 * (hh & 1))) & 0xFFFFu;
+                    const uint32_t key = min((d - 1u) >> 10, 64u);  // a hole (d = 0) wraps to 64
+                    cnt8 += sm.ctab[key];
+                    if (key - 8u < 56u) atomicAdd(&sm.h1[key], 1u);
+                }
             }
-        }
+        };
+        if (!ok)
+            resample(std::integral_constant<int, SRC_NONE>{});
+        else if (!a.rects)
+            resample(std::integral_constant<int, SRC_CROPS>{});
+        else if (a.affine)
+            resample(std::integral_constant<int, SRC_AFFINE>{});
+        else if (pair_win)
+            resample(std::integral_constant<int, SRC_WINDOWS>{});
+        else
+            resample(std::integral_constant<int, SRC_RECT>{});
         {
             // coarse histogram of the non-zero depths, keyed by (d - 1) >> 10 (bins of 1024 mm;
             // any monotone key serves the select, and this one needs no test for holes): a thread
@@ -643,7 +669,6 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::MINB) lbp_fused_
                 prefetch_rect_rows(a.grey, a.depth, a.H, a.W, rn, tid, NT);
         }
         float sq = 0.f;
-        const bool centred = a.x_centre != nullptr;
         const bool wide = x_dtype == RGBD_DT_BF16 && !centred && (a.k_pad & 7) == 0 && (DIM & 7) == 0 &&
                           ((reinterpret_cast<size_t>(a.feats) | reinterpret_cast<size_t>(a.x_out)) & 15) == 0;
         if (wide) {
@@ -657,10 +682,20 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::MINB) lbp_fused_
                     if (a.feats)
                         *reinterpret_cast<uint4*>(a.feats + (size_t)face * DIM + j) =
                             make_uint4(hv.x & 0x007F007Fu, hv.y & 0x007F007Fu, hv.z & 0x007F007Fu, hv.w & 0x007F007Fu);
-                    const uint32_t hw[4] = {qbf_slot2(hv.x), qbf_slot2(hv.y), qbf_slot2(hv.z), qbf_slot2(hv.w)};
+                    const uint32_t hs[4] = {hv.x, hv.y, hv.z, hv.w};
+                    uint32_t hw[4];
+                    if (TABLE)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) hw[e] = qbf_slot2(hs[e]);
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        const uint32_t qb = sm.qbf[(hw[e >> 1] >> (16 * (e & 1))) & 0xFFFFu];
+                        uint32_t qb;
+                        if (TABLE) {
+                            qb = sm.qbf[(hw[e >> 1] >> (16 * (e & 1))) & 0xFFFFu];
+                        } else {
+                            const int w = (int)((hs[e >> 1] >> (16 * (e & 1))) & 0xFFFFu);
+                            qb = bf16_quotient(w >> 7, w & 127, sm.rcpn[w >> 7]);
+                        }
                         const float f = __uint_as_float(qb << 16);
                         sq = fmaf(f, f, sq);
                         pk[e >> 1] |= qb << (16 * (e & 1));
@@ -680,7 +715,7 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::MINB) lbp_fused_
                     *reinterpret_cast<uint2*>(a.feats + (size_t)face * DIM + j) =
                         make_uint2(hv.x & 0x007F007Fu, hv.y & 0x007F007Fu);
             }
-            if (x_dtype == RGBD_DT_BF16 && !centred) {
+            if (TABLE && x_dtype == RGBD_DT_BF16 && !centred) {
                 // bf16 rows: one table read per value
                 uint32_t pk[2] = {0u, 0u};
                 if (j < DIM) {
@@ -721,7 +756,7 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::MINB) lbp_fused_
                         x[3] = __fsub_rn(x[3], mu.w);
                     }
                 }
-                if (x_dtype == RGBD_DT_BF16) {  // centred bf16 rows (round to nearest even)
+                if (x_dtype == RGBD_DT_BF16) {  // bf16 rows without the table (round to nearest even)
                     uint32_t pk[2] = {0u, 0u};
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
@@ -787,20 +822,22 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::MINB) lbp_fused_
     }
 }
 
-template <int S, int TPC>
+template <int S, int TPC, bool TABLE>
 int launch_fused_t(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
-    static int blocks_per_sm = -1;
-    const size_t smem = sizeof(Smem<S, TPC>);
-    if (blocks_per_sm < 0) {
-        cudaError_t e = cudaFuncSetAttribute(lbp_fused_kernel<S, TPC>,
+    using Shared = Smem<S, TPC>;
+    const size_t smem = TABLE ? sizeof(Shared) : offsetof(Shared, qbf);  // the table comes last
+    static int blocks = -1;
+    if (blocks < 0) {
+        cudaError_t e = cudaFuncSetAttribute(lbp_fused_kernel<S, TPC, TABLE>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return cuda_error(e, "lbp_fused_features: smem attribute");
         int b = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, lbp_fused_kernel<S, TPC>, Cfg<S, TPC>::NT, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, lbp_fused_kernel<S, TPC, TABLE>, Cfg<S, TPC>::NT, smem);
         if (e != cudaSuccess) return cuda_error(e, "lbp_fused_features: occupancy");
-        blocks_per_sm = b > 0 ? b : 1;
+        blocks = b > 0 ? b : 1;
     }
-    const int per_sm = ctx->tune_lbp_ctas_per_sm > 0 ? std::min(ctx->tune_lbp_ctas_per_sm, blocks_per_sm) : blocks_per_sm;
+    // the tuning value counts the CTAs of the 128 x 128 shape, whose occupancy is 2
+    const int per_sm = ctx->tune_lbp_ctas_per_sm > 0 ? std::min(ctx->tune_lbp_ctas_per_sm, blocks) : blocks;
     const int grid = (int)std::min<long long>((long long)a.n, (long long)per_sm * ctx->props.sm_count);
     LbpArgs la = a;
     if (grid >= a.n) {
@@ -809,10 +846,19 @@ int launch_fused_t(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
         cudaError_t e = cudaMemsetAsync(la.face_counter, 0, sizeof(uint32_t), s);
         if (e != cudaSuccess) return cuda_error(e, "lbp_fused_features: face queue reset");
     }
-    lbp_fused_kernel<S, TPC><<<grid, Cfg<S, TPC>::NT, smem, s>>>(la);
+    lbp_fused_kernel<S, TPC, TABLE><<<grid, Cfg<S, TPC>::NT, smem, s>>>(la);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "lbp_fused_features: launch");
     return RGBD_OK;
+}
+
+// The quotient table (8320 entries) serves uncentred bf16 rows where a CTA makes many values: crops
+// of 96 and 128 (8496 and 15104 values a face), more faces than SMs (7 faces of 128 x 128: 20.6 us
+// with the table, 18.9 us without).
+template <int S, int TPC>
+int launch_fused_s(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
+    const bool table = S >= 96 && a.n > ctx->props.sm_count && a.x_out && a.x_dtype == RGBD_DT_BF16 && !a.x_centre;
+    return table ? launch_fused_t<S, TPC, S >= 96>(ctx, a, s) : launch_fused_t<S, TPC, false>(ctx, a, s);
 }
 
 }  // namespace
@@ -820,18 +866,19 @@ int launch_fused_t(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
 int launch_lbp_fused(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
     if (a.flags & RGBD_LBP_FACE_HIST256) return launch_face256(ctx, a, s);
     // tile shape (crops 64 and 128): one thread per cell (tuning value 1), per half cell (2, the
-    // default), per quarter cell (3: 1024-thread CTAs, measured 7 % slower even when every face
-    // has an SM of its own, and 50 % slower on full batches)
+    // default), per quarter cell (3: 1024-thread CTAs at 128, 50 % slower on full batches).  Crops of
+    // 32 have a cell's quarter per thread: one warp of halves is 16 us for a face and 22.8 us for 2048,
+    // two of quarters 8.4 and 20.4 us.
     const int shape = ctx->tune_lbp_shape == 0 ? 2 : ctx->tune_lbp_shape;
     switch (a.crop) {
-        case 32: return launch_fused_t<32, 2>(ctx, a, s);
+        case 32: return launch_fused_s<32, 4>(ctx, a, s);
         case 64:
-            return shape == 1 ? launch_fused_t<64, 1>(ctx, a, s)
-                              : (shape == 3 ? launch_fused_t<64, 4>(ctx, a, s) : launch_fused_t<64, 2>(ctx, a, s));
-        case 96: return launch_fused_t<96, 2>(ctx, a, s);
+            return shape == 1 ? launch_fused_s<64, 1>(ctx, a, s)
+                              : (shape == 3 ? launch_fused_s<64, 4>(ctx, a, s) : launch_fused_s<64, 2>(ctx, a, s));
+        case 96: return launch_fused_s<96, 2>(ctx, a, s);
         case 128:
-            return shape == 1 ? launch_fused_t<128, 1>(ctx, a, s)
-                              : (shape == 3 ? launch_fused_t<128, 4>(ctx, a, s) : launch_fused_t<128, 2>(ctx, a, s));
+            return shape == 1 ? launch_fused_s<128, 1>(ctx, a, s)
+                              : (shape == 3 ? launch_fused_s<128, 4>(ctx, a, s) : launch_fused_s<128, 2>(ctx, a, s));
         default:
             return set_error(RGBD_ERR_UNSUPPORTED, "lbp_fused_features: crop %d (32, 64, 96 or 128)", a.crop);
     }

@@ -235,3 +235,22 @@ def test_face_histogram_256_sizes_and_rules(B, ctx, orc, crop, flags):
                                    affine=torch.from_numpy(aff).cuda())
     assert (host_u16(f) == want).all()
     assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("crop", [32, 64, 96, 128])
+@pytest.mark.parametrize("dt", ["bf16", "fp8"])
+def test_rows_with_and_without_the_quotient_table(B, ctx, orc, crop, dt):
+    """Few faces (quotients computed) and more faces than SMs (bf16 quotients from the table at 96 and
+    128): the same faces give the same rows and norms, and the rows are the oracle's."""
+    g, d, r = synth.frames_with_rects(crop, 2, 5, 30, 160, H=160, W=200)
+    many = np.concatenate([r] * 40)  # 400 faces
+    f, x, q = B.lbp_fused_features(ctx, dev_u8(g), dev_u16(d), B.rects_tensor(r), crop=crop, x_dtype=dt)
+    fm, xm, qm = B.lbp_fused_features(ctx, dev_u8(g), dev_u16(d), B.rects_tensor(many), crop=crop, x_dtype=dt)
+    want = orc.features_batch(g, d, r, crop)
+    assert (host_u16(f) == want).all()
+    x32 = orc.normalize_f32(want)
+    rows = orc.f32_to_bf16(x32) if dt == "bf16" else orc.f32_to_e4m3((x32 * np.float32(448.0)).astype(np.float32))
+    got = host_u16(x.view(torch.int16)) if dt == "bf16" else x.cpu().numpy()
+    assert (got[:, :want.shape[1]] == rows).all()
+    for k in range(0, 400, 10):
+        assert torch.equal(fm[k:k + 10], f) and torch.equal(xm[k:k + 10], x) and torch.equal(qm[k:k + 10], q)
