@@ -204,6 +204,27 @@ def test_kernel_matrix_and_smo_of_every_size(B, ctx, orc, n, k_pad):
             assert abs(bias[c].item() - v[free].mean()) <= 1e-4
 
 
+@pytest.mark.parametrize("n", [1, 3, 700])
+@pytest.mark.parametrize("dim,C", [(59, 1), (3776, 5), (15104, 64), (531, 256)])
+def test_linear_scores(B, ctx, orc, n, dim, C):
+    """Linear scores with one and with four rows per CTA (a last group of one to three rows), class
+    counts around the groups of eight, short and long rows; ties go to the lowest class."""
+    rng = synth.rng_for(n + dim + C)
+    w, b = synth.linear_model(rng, C, dim)
+    if C > 3:
+        w[C - 1], b[C - 1] = w[1], b[1]  # an exact tie
+        w[C // 2], b[C // 2] = w[1], b[1]
+    x = rng.uniform(0, 0.1, (n, B.k_pad_for(dim))).astype(np.float32)
+    x[:, dim:] = 0
+    model = B.svm_train_data_pack(ctx, None, dev_f32(w), dev_f32(b), kernel=B.KERNEL_LINEAR, dim=dim)
+    s, lab = B.svm_score(ctx, model, dev_f32(x))
+    x64 = x[:, :dim].astype(np.float64)
+    ref = x64 @ w.astype(np.float64).T + b
+    scale = np.abs(x64) @ np.abs(w.astype(np.float64)).T + np.abs(b)
+    assert np.all(np.abs(s.cpu().numpy() - ref) <= 1e-5 * scale)
+    assert (lab.cpu().numpy() == s.cpu().numpy().argmax(1)).all()
+
+
 @pytest.mark.parametrize("crop", [8, 9, 50, 131, 255])
 @pytest.mark.parametrize("flags", [0, 1, 2, 3])
 def test_face_histogram_256_sizes_and_rules(B, ctx, orc, crop, flags):
