@@ -918,7 +918,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 // takes as long as 4096 rows take per CTA.  Here the K extent (the k-blocks of every pass) of
 // each SV tile is cut into `kz` ranges, one CTA per (tile, range), so that all SMs stream the
 // SVs; each CTA writes its partial G = X . SV_t^T of the valid rows to `gpart`
-// ([kz][n_pad][n]), and rbf_splitk_epilogue_kernel adds the ranges, finishes the tile and, in
+// ([kz][n][n_pad]), and rbf_splitk_epilogue_kernel adds the ranges, finishes the tile and, in
 // the last CTA of each row group, combines the tiles into scores and labels.
 // Warps: 0 the TMA producer (4 stages of X and SV k-blocks), 1 the TMEM owner and MMA issuer,
 // 2-5 the epilogue (one thread per row, TMEM lane quarter = warp % 4).  The X copies hold only
@@ -942,7 +942,7 @@ struct SkParams {
     int kpz;        // k-blocks (over all passes) per K range
     uint32_t x_bytes;  // bytes of one X k-block: only the valid rows, rounded up to 8, are copied
     uint32_t idesc;
-    float* gpart;   // [kz][n_pad][n]
+    float* gpart;   // [kz][n][n_pad]
     uint32_t* counters;  // [n_groups]: finished tiles per row group of the epilogue, zeroed here
     int n_groups;
     uint32_t* status;
@@ -1062,7 +1062,7 @@ __global__ void __launch_bounds__(SK_WARPS * 32, 1)
         if (__shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0)) {
             tc_fence_after();
             const uint32_t g_tmem = tmem + ((uint32_t)(quarter * 32) << 16);
-            float* out = p.gpart + ((size_t)z * p.n_pad + (size_t)tile * BN) * p.n + row;
+            float* out = p.gpart + ((size_t)z * p.n + row) * p.n_pad + (size_t)tile * BN;
 #pragma unroll 1
             for (int c = 0; c < BN; c += 32) {
                 uint32_t v[32];
@@ -1070,7 +1070,10 @@ __global__ void __launch_bounds__(SK_WARPS * 32, 1)
                 tc_wait_ld();
                 if (row < p.n) {
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) out[(size_t)(c + j) * p.n] = __uint_as_float(v[j]);
+                    for (int j = 0; j < 32; j += 4)
+                        *reinterpret_cast<float4*>(out + c + j) =
+                            make_float4(__uint_as_float(v[j]), __uint_as_float(v[j + 1]), __uint_as_float(v[j + 2]),
+                                        __uint_as_float(v[j + 3]));
                 }
             }
         }
@@ -1090,154 +1093,164 @@ __global__ void __launch_bounds__(SK_WARPS * 32, 1)
 // d^2 = |x|^2 + |sv|^2 - 2 G, the row's reference distance r (mean d^2 over the tile's real SVs),
 // F = expm1(-gamma (d^2 - r)) and D_c = sum_i a_ci F_i with the fp32 coefficients.  Each tile
 // is one split of the split combine (D and r per tile); the last CTA of a row group to finish
-// (counters[row group], zeroed by the split-K kernel) adds the tiles of its rows and takes the
-// argmax, with the terms of the combine kernels of launch_reduce_scores.  The loads of each step
-// are issued together: the kernel is a short chain of dependent L2 round trips.
+// (counters[row group], zeroed by the kernel before) adds the tiles of its rows and takes the
+// argmax, with the terms of the combine kernels of launch_reduce_scores.
+// A chain of L2 round trips and short steps between them: the coefficients are asked for (into
+// shared memory) before waiting for the kernel before, a warp holds a row's distances in registers
+// from the partials to F, a warp makes four classes of eight rows at a time (F is read from shared
+// memory once for the four), and 16 warps make most steps a single pass.  7 rows x 32 tiles, 64
+// classes, from the end of the kernel before: 17 us with 8 warps, a class at a time and block-wide
+// passes for r and F (5.8 us the classes, 5.3 us the combine), 10 us now.
+// d2_min: least d^2 (0 for the exact fp32 path, -infinity for the tensor-core paths).
 constexpr int SKE_ROWS = 16;
-constexpr int SKE_THREADS = 256;
-constexpr int SKE_CPW = 8;  // classes per warp and pass (their coefficients loaded at once)
+constexpr int SKE_THREADS = 32 * SKE_ROWS;
+size_t ske_smem(int C) { return sizeof(float) * (size_t)((C + 3) / 4 * 4 + SKE_ROWS) * BN; }
+
 __global__ void __launch_bounds__(SKE_THREADS) rbf_splitk_epilogue_kernel(
     const float* __restrict__ gpart, int kz, int n_pad, int n, const float* __restrict__ xsq,
     const float* __restrict__ svsq, int n_sv, const float* __restrict__ coef, int C, int C_pad, float gamma,
-    float gscale, float* __restrict__ part, float* __restrict__ ref, uint32_t* __restrict__ counters, int nt,
-    const float* __restrict__ asum, const float* __restrict__ asum_tile, const float* __restrict__ bias,
+    float gscale, float d2_min, float* __restrict__ part, float* __restrict__ ref, uint32_t* __restrict__ counters,
+    int nt, const float* __restrict__ asum, const float* __restrict__ asum_tile, const float* __restrict__ bias,
     float* __restrict__ scores, int32_t* __restrict__ labels) {
-    __shared__ float F[SKE_ROWS][BN];
-    __shared__ float r_row[SKE_ROWS];
+    extern __shared__ __align__(16) float ske_smem_raw[];
+    float* F = ske_smem_raw;            // [SKE_ROWS][BN]; later the combine's
+    float* A = F + SKE_ROWS * BN;       // [C rounded up to 4][BN]: the tile's coefficients
+    const float4* F4 = reinterpret_cast<const float4*>(F);
+    const float4* A4 = reinterpret_cast<const float4*>(A);
     __shared__ int last;
-    // launched as a programmatic dependent of the split-K kernel: wait for it to complete
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    constexpr int W4 = BN / 4, PER = BN / 32;  // 4-column groups of a tile, columns per lane
     const int tile = blockIdx.x, k0 = blockIdx.y * SKE_ROWS;
-    const int rows = min(SKE_ROWS, n - k0);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = SKE_THREADS / 32;
-    static_assert(SKE_THREADS == BN, "one thread per SV column of the tile");
+    const int rows = min(SKE_ROWS, n - k0), valid = min(BN, n_sv - tile * BN);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     {
-        // thread = column: every K range's partial of every row, all loads issued together
-        const int col = tile * BN + threadIdx.x;
-        const size_t zs = (size_t)n_pad * n;
-        const float* gp = gpart + (size_t)col * n + k0;
-        float g[SKE_ROWS];
-#pragma unroll
-        for (int k = 0; k < SKE_ROWS; ++k) g[k] = 0.f;
-        for (int zz = 0; zz < kz; ++zz) {
-#pragma unroll
-            for (int k = 0; k < SKE_ROWS; ++k)
-                if (k < rows) g[k] += gp[zz * zs + k];
-        }
-        const bool real = col < n_sv;
-        const float svs = real ? svsq[col] : 0.f;
-#pragma unroll
-        for (int k = 0; k < SKE_ROWS; ++k)
-            if (k < rows) F[k][threadIdx.x] = real ? xsq[k0 + k] + svs - 2.f * gscale * g[k] : 0.f;
+        const uint32_t dst = smem_u32(A);
+        const float* src = coef + (size_t)tile * BN;
+#pragma unroll 4
+        for (int i = tid; i < C * W4; i += SKE_THREADS)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16u * i),
+                         "l"(src + (size_t)(i / W4) * n_pad + 4 * (i % W4))
+                         : "memory");
     }
-    __syncthreads();
-    const int valid = min(BN, n_sv - tile * BN);
-    for (int k = warp; k < rows; k += nw) {
+    float sv[PER];
+    const float xs = warp < rows ? xsq[k0 + warp] : 0.f;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) sv[j] = svsq[tile * BN + lane + 32 * j];
+    // launched as a programmatic dependent of the partial-product kernel: wait for it to complete
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (warp < rows) {
+        const float* gp = gpart + (size_t)(k0 + warp) * n_pad + tile * BN + lane;
+        float g[PER];
+#pragma unroll
+        for (int j = 0; j < PER; ++j) g[j] = 0.f;
+#pragma unroll 4
+        for (int z = 0; z < kz; ++z) {
+#pragma unroll
+            for (int j = 0; j < PER; ++j) g[j] += __ldcg(gp + (size_t)z * n_pad * n + 32 * j);
+        }
         float sum = 0.f;
-        for (int i = lane; i < valid; i += 32) sum += F[k][i];
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            g[j] = fmaxf(xs + sv[j] - 2.f * gscale * g[j], d2_min);
+            if (lane + 32 * j < valid) sum += g[j];
+        }
         for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
-        if (lane == 0) r_row[k] = sum / (float)max(valid, 1);
+        const float r = sum / (float)max(valid, 1);
+#pragma unroll
+        for (int j = 0; j < PER; ++j)
+            F[warp * BN + lane + 32 * j] = lane + 32 * j < valid ? expm1_near0(-gamma * (g[j] - r)) : 0.f;
+        if (lane == 0) ref[(size_t)tile * n + k0 + warp] = r;
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    for (int k = 0; k < rows; ++k) {
-        const int i = threadIdx.x;
-        F[k][i] = i < valid ? expm1_near0(-gamma * (F[k][i] - r_row[k])) : 0.f;
-    }
-    __syncthreads();
-    for (int c0 = warp * SKE_CPW; c0 < C; c0 += nw * SKE_CPW) {
-        float a[SKE_CPW][BN / 32];
+    // a warp = four classes and eight rows at a time: 32 sums over the lanes, halved over the values
+    // until lane l holds that of row l / 4 and class l % 4
+    const int groups = (rows + 7) / 8;
+#pragma unroll 1
+    for (int i = warp; i < (C + 3) / 4 * groups; i += SKE_THREADS / 32) {
+        const int c0 = i / groups * 4, kb = (i % groups) * 8;
+        float v[32];
 #pragma unroll
-        for (int cc = 0; cc < SKE_CPW; ++cc)
+        for (int u = 0; u < 32; ++u) v[u] = 0.f;
 #pragma unroll
-            for (int j = 0; j < BN / 32; ++j)
-                a[cc][j] = c0 + cc < C ? coef[(size_t)(c0 + cc) * n_pad + tile * BN + lane + 32 * j] : 0.f;
-        for (int k = 0; k < rows; ++k) {
-            float sk[SKE_CPW];
+        for (int half = 0; half < 2; ++half) {
+            float4 a[4];
 #pragma unroll
-            for (int cc = 0; cc < SKE_CPW; ++cc) {
-                float t = 0.f;
+            for (int q = 0; q < 4; ++q) a[q] = A4[(c0 + q) * W4 + 32 * half + lane];
 #pragma unroll
-                for (int j = 0; j < BN / 32; ++j) t = fmaf(F[k][lane + 32 * j], a[cc][j], t);
-                sk[cc] = t;
-            }
+            for (int u = 0; u < 8; ++u) {  // (rows past the last are not used)
+                const float4 f = F4[(kb + u) * W4 + 32 * half + lane];
 #pragma unroll
-            for (int cc = 0; cc < SKE_CPW; ++cc)
-                for (int off = 16; off > 0; off >>= 1) sk[cc] += __shfl_xor_sync(0xFFFFFFFFu, sk[cc], off);
-            if (lane < SKE_CPW && c0 + lane < C) {
-                float v = sk[0];
-#pragma unroll
-                for (int cc = 1; cc < SKE_CPW; ++cc) v = lane == cc ? sk[cc] : v;
-                part[((size_t)tile * n + k0 + k) * C_pad + c0 + lane] = v;
-            }
-        }
-    }
-    if (threadIdx.x < rows) ref[(size_t)tile * n + k0 + threadIdx.x] = r_row[threadIdx.x];
-
-    // ---- the last tile of this row group to finish adds the tiles ----
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(counters + blockIdx.y, 1u) == (uint32_t)nt - 1u;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    // shared memory (F reused): delta_s per row and tile, the tiles' coefficient sums when they
-    // fit, then the scores of the group's rows
-    float* s_del = &F[0][0];                       // [rows][nt] (nt <= 256)
-    float* s_as = s_del + rows * nt;               // [nt][C] or unused
-    const bool as_fit = rows * nt + nt * C + rows * C <= SKE_ROWS * BN;
-    float* s_sc = as_fit ? s_as + nt * C : s_del + rows * nt;  // [rows][C]
-    const bool sc_fit = (int)(s_sc - s_del) + rows * C <= SKE_ROWS * BN;
-    for (int idx = threadIdx.x; idx < rows * nt; idx += SKE_THREADS) {
-        const int k = idx / nt, t = idx - k * nt;
-        s_del[idx] = t == 0 ? 0.f : expm1f(-gamma * (__ldcg(ref + (size_t)t * n + k0 + k) - __ldcg(ref + k0 + k)));
-    }
-    if (as_fit)
-        for (int idx = threadIdx.x; idx < nt * C; idx += SKE_THREADS) {
-            const int t = idx / C, c = idx - t * C;
-            s_as[idx] = t == 0 ? 0.f : __ldg(asum_tile + (size_t)t * C_pad + c);
-        }
-    __syncthreads();
-    // thread = (row, class), two of them at a time: the tiles' partial sums loaded 32 at a time
-    // for both (one L2 round trip per chunk), then added in tile order
-    const size_t ts = (size_t)n * C_pad;
-    for (int i0 = threadIdx.x; i0 < rows * C; i0 += 2 * SKE_THREADS) {
-        const int i1 = i0 + SKE_THREADS;
-        const bool two = i1 < rows * C;
-        const int ka = i0 / C, ca = i0 - ka * C;
-        const int kb = two ? i1 / C : ka, cb = two ? i1 - kb * C : ca;
-        const float* pa = part + (size_t)(k0 + ka) * C_pad + ca;
-        const float* pb = part + (size_t)(k0 + kb) * C_pad + cb;
-        float acc_a = 0.f, acc_b = 0.f;
-        for (int t0 = 0; t0 < nt; t0 += 32) {
-            float da[32], db[32];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                da[j] = t0 + j < nt ? __ldcg(pa + (t0 + j) * ts) : 0.f;
-                db[j] = (two && t0 + j < nt) ? __ldcg(pb + (t0 + j) * ts) : 0.f;
-            }
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                if (t0 + j < nt) {
-                    const int t = t0 + j;
-                    const float asa = as_fit ? s_as[t * C + ca] : (t == 0 ? 0.f : __ldg(asum_tile + (size_t)t * C_pad + ca));
-                    const float asb = as_fit ? s_as[t * C + cb] : (t == 0 ? 0.f : __ldg(asum_tile + (size_t)t * C_pad + cb));
-                    acc_a += da[j] + s_del[ka * nt + t] * (asa + da[j]);
-                    acc_b += db[j] + s_del[kb * nt + t] * (asb + db[j]);
+                for (int q = 0; q < 4; ++q) {
+                    float t = v[4 * u + q];
+                    t = fmaf(f.x, a[q].x, t);
+                    t = fmaf(f.y, a[q].y, t);
+                    t = fmaf(f.z, a[q].z, t);
+                    v[4 * u + q] = fmaf(f.w, a[q].w, t);
                 }
             }
         }
-        const float sa = expf(-gamma * __ldcg(ref + k0 + ka)) * (__ldg(asum + ca) + acc_a) + __ldg(bias + ca);
-        scores[(size_t)(k0 + ka) * C + ca] = sa;
-        if (sc_fit) s_sc[i0] = sa;
-        if (two) {
-            const float sb = expf(-gamma * __ldcg(ref + k0 + kb)) * (__ldg(asum + cb) + acc_b) + __ldg(bias + cb);
-            scores[(size_t)(k0 + kb) * C + cb] = sb;
-            if (sc_fit) s_sc[i1] = sb;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            const bool upper = (lane & off) != 0;
+#pragma unroll
+            for (int u = 0; u < off; ++u) {
+                const float other = __shfl_xor_sync(0xFFFFFFFFu, upper ? v[u] : v[u + off], off);
+                v[u] = (upper ? v[u + off] : v[u]) + other;
+            }
         }
+        const int k = kb + lane / 4, c = c0 + lane % 4;
+        if (k < rows && c < C) part[((size_t)tile * n + k0 + k) * C_pad + c] = v[0];
+    }
+
+    // ---- the last tile of this row group to finish adds the tiles ----
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();  // the CTA's sums (ordered before it by the barrier) are visible before it counts
+        last = atomicAdd(counters + blockIdx.y, 1u) == (uint32_t)nt - 1u;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    // Shared memory reused: in F delta_s per row and tile and the scores behind them when they fit, in
+    // A the tiles' coefficient sums (read by every row from global memory instead, they were 8 of
+    // the 11 us of this part).
+    float* s_del = F;               // [rows][nt] (nt <= 256)
+    float* s_sc = F + rows * nt;    // [rows][C]
+    const bool sc_fit = rows * nt + rows * C <= SKE_ROWS * BN;
+    float* s_as = A;                // [nt][C]
+#pragma unroll 4
+    for (int i = tid; i < nt * C; i += SKE_THREADS) s_as[i] = __ldcg(asum_tile + (size_t)(i / C) * C_pad + i % C);
+#pragma unroll 1
+    for (int idx = tid; idx < rows * nt; idx += SKE_THREADS) {
+        const int k = idx / nt, t = idx - k * nt;
+        s_del[idx] = t == 0 ? 0.f : expm1f(-gamma * (__ldcg(ref + (size_t)t * n + k0 + k) - __ldcg(ref + k0 + k)));
+    }
+    __syncthreads();
+    // thread = (row, class): the tiles' partial sums 16 at a time, added in tile order
+    const size_t ts = (size_t)n * C_pad;
+#pragma unroll 1
+    for (int i = tid; i < rows * C; i += SKE_THREADS) {
+        const int k = i / C, c = i - k * C;
+        const float* pd = part + (size_t)(k0 + k) * C_pad + c;
+        const float r0 = __ldcg(ref + k0 + k), as = __ldg(asum + c), bs = __ldg(bias + c);
+        float acc = 0.f;
+#pragma unroll 1
+        for (int t0 = 0; t0 < nt; t0 += 16) {
+            float d[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) d[j] = t0 + j < nt ? __ldcg(pd + (size_t)(t0 + j) * ts) : 0.f;
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                if (t0 + j < nt) acc += d[j] + s_del[k * nt + t0 + j] * (s_as[(t0 + j) * C + c] + d[j]);
+        }
+        const float sc = expf(-gamma * r0) * (as + acc) + bs;
+        scores[(size_t)(k0 + k) * C + c] = sc;
+        if (sc_fit) s_sc[i] = sc;
     }
     if (!labels) return;
     __syncthreads();
-    for (int k = warp; k < rows; k += nw) {
+    if (warp < rows) {
+        const int k = warp;
         float best = -INFINITY;
         int bi = 0x7FFFFFFF;
         for (int c = lane; c < C; c += 32) {
@@ -1503,22 +1516,8 @@ int launch_tc(rgbd_ctx* ctx, const rgbd_svm* m, const void* x, const float* xsq,
             default: e = launch_splitk<3>(pl, sp, m, tm_x, tm_x2, s); break;
         }
         if (e != cudaSuccess) return cuda_error(e, "svm_score: split-K launch");
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)pl.nt, (unsigned)sp.n_groups, 1);
-        cfg.blockDim = dim3(SKE_THREADS, 1, 1);
-        cfg.dynamicSmemBytes = 0;
-        cfg.stream = s;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, rbf_splitk_epilogue_kernel, (const float*)sp.gpart, pl.kz, m->n_pad, n, xsq,
-                               (const float*)m->sv_sq, m->n_sv, (const float*)m->coef, m->C, m->C_pad, m->gamma,
-                               gscale, part, ref, sp.counters, pl.nt, (const float*)m->asum,
-                               (const float*)m->asum_tile, (const float*)m->bias, scores, labels);
-        if (e != cudaSuccess) return cuda_error(e, "svm_score: split-K epilogue launch");
-        return RGBD_OK;
+        return launch_rows_epilogue(m, sp.gpart, pl.kz, n, xsq, gscale, -INFINITY, part, ref, sp.counters, scores,
+                                    labels, s);
     }
     // Mode: tuning value 2 = single CTAs, 3 = 2-CTA MMA pairs, 0 = auto (the 2-CTA pairs).
     // Pairs need at least two 128-row blocks.
@@ -1597,6 +1596,31 @@ __global__ void expm1_probe_kernel(const float* __restrict__ z, float* __restric
 }
 
 }  // namespace
+
+int launch_rows_epilogue(const rgbd_svm* m, const float* gpart, int kz, int n, const float* xsq, float gscale,
+                         float d2_min, float* part, float* ref, uint32_t* counters, float* scores, int32_t* labels,
+                         cudaStream_t s) {
+    const int nt = m->n_pad / BN;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nt, (unsigned)((n + SKE_ROWS - 1) / SKE_ROWS), 1);
+    cfg.blockDim = dim3(SKE_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = ske_smem(m->C);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaFuncSetAttribute(rbf_splitk_epilogue_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)ske_smem(MAX_CPAD));
+    if (e != cudaSuccess) return cuda_error(e, "svm_score: split-K epilogue smem attribute");
+    e = cudaLaunchKernelEx(
+        &cfg, rbf_splitk_epilogue_kernel, gpart, kz, m->n_pad, n, xsq, (const float*)m->sv_sq, m->n_sv,
+        (const float*)m->coef, m->C, m->C_pad, m->gamma, gscale, d2_min, part, ref, counters, nt,
+        (const float*)m->asum, (const float*)m->asum_tile, (const float*)m->bias, scores, labels);
+    if (e != cudaSuccess) return cuda_error(e, "svm_score: split-K epilogue launch");
+    return RGBD_OK;
+}
 
 int score_rbf_tc(rgbd_ctx* ctx, const rgbd_svm* m, const void* x, const float* xsq, int n, float x_scale,
                  float* scores, int32_t* labels, cudaStream_t s) {

@@ -225,6 +225,28 @@ def test_linear_scores(B, ctx, orc, n, dim, C):
     assert (lab.cpu().numpy() == s.cpu().numpy().argmax(1)).all()
 
 
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 8])
+@pytest.mark.parametrize("n_sv,C,cells", [(1, 1, 1), (17, 10, 256), (333, 128, 70), (700, 64, 256)])
+def test_fp32_scores_of_up_to_eight_rows(B, ctx, orc, n, n_sv, C, cells):
+    """The exact fp32 scores of one to eight rows: K in one slice and in eight with a short last one,
+    an odd last support vector, one and several SV tiles, class counts around the groups of eight."""
+    rng = synth.rng_for(n + 10 * n_sv + C)
+    dim = cells * 59
+    X, SV = synth.poisson_counts(rng, n, dim), synth.poisson_counts(rng, n_sv, dim)
+    X[0] = SV[0]  # a row that is a support vector
+    a = rng.normal(0, 1, (C, n_sv)).astype(np.float32)
+    b = rng.normal(0, 0.01, C).astype(np.float32)
+    model = B.svm_train_data_pack(ctx, dev_u16(SV), dev_f32(a), dev_f32(b), gamma=0.3, dtype="f32")
+    x, q = B.lbp_normalize_features(ctx, dev_u16(X), "f32")
+    s, lab = B.svm_score(ctx, model, x, q)
+    assert ctx.status() == 0
+    x64, sv64 = orc.normalize_f64(X), orc.normalize_f64(SV)
+    ref = orc.svm_rbf(x64, sv64, a, b, 0.3)
+    # the path's stated bound (1e-5 of the score scale)
+    assert rel_score_error(s.cpu().numpy(), ref, rbf_error_scale(x64, sv64, a, b, 0.3)) <= 1e-5
+    assert (lab.cpu().numpy() == s.cpu().numpy().argmax(1)).all()
+
+
 @pytest.mark.parametrize("crop", [8, 9, 50, 131, 255])
 @pytest.mark.parametrize("flags", [0, 1, 2, 3])
 def test_face_histogram_256_sizes_and_rules(B, ctx, orc, crop, flags):
