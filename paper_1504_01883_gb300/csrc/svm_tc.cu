@@ -109,15 +109,6 @@ struct TcParams {
     uint32_t idesc_main;
     uint32_t idesc_second;
     int passes;       // 1, or 3 for split bf16 operands (RGBD_DT_BF16X3)
-    // split combine inside the kernel (fuse = 1): the last CTA of each 128-row block to finish
-    // adds the splits of its rows (counters[row block] counts finished splits, zeroed per launch)
-    int fuse;
-    uint32_t* counters;
-    const float* asum;       // [C]
-    const float* asum_tile;  // [n_tiles][C_pad]
-    const float* bias;       // [C]
-    float* scores;           // [n][C]
-    int32_t* labels;         // [n] or NULL
 };
 
 // ---------------------------------------------------------------------------------------
@@ -335,12 +326,18 @@ __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sy
           "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),           \
           "=r"(v[15])                                                                                        \
         : "r"(taddr))
-// e^z - 1.  The near-flat RBF gives |z| = gamma |d^2 - r| of order 1e-3, where the Taylor series
-// z + z^2/2! + ... + z^6/6! (Horner form) is exact to fp32 rounding: for |z| < 2^-5 the first
-// omitted term is below 2^-30 |z| / 5040.  Larger arguments use expm1f.
+// e^z - 1.  The near-flat RBF gives |z| = gamma |d^2 - r| of order 1e-3, a trained model (gamma 0.5)
+// a few tenths.  Up to 1/2 the Taylor series z + z^2/2! + ... + z^9/9! (Horner form) is exact to fp32
+// rounding: the first omitted term is below 2^-9 |z| / 10! = 5.4e-10 |z|.  Larger arguments use
+// expm1f.  (300 rows x 8190 SVs, gamma 0.5: 77.8 us, against 79.8 with the series to z^6 below 2^-5
+// apart, so that most warps took two series, and 80.1 with expm1f from 2^-5 on; no difference in a
+// full near-flat batch.)
 __device__ __forceinline__ float expm1_near0(float z) {
-    if (fabsf(z) < 0.03125f) {
-        float q = fmaf(z, 1.0f / 720.0f, 1.0f / 120.0f);
+    if (fabsf(z) < 0.5f) {
+        float q = fmaf(z, 1.0f / 362880.0f, 1.0f / 40320.0f);
+        q = fmaf(z, q, 1.0f / 5040.0f);
+        q = fmaf(z, q, 1.0f / 720.0f);
+        q = fmaf(z, q, 1.0f / 120.0f);
         q = fmaf(z, q, 1.0f / 24.0f);
         q = fmaf(z, q, 1.0f / 6.0f);
         q = fmaf(z, q, 0.5f);
@@ -350,81 +347,6 @@ __device__ __forceinline__ float expm1_near0(float z) {
 }
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-
-// ---------------------------------------------------------------------------------------
-// Split combine (A7), run by the last CTA of a 128-row block to finish: for each row and class
-//   S_c = exp(-gamma r*) (asum_c + sum_s [D_s + delta_s (asum_{c,s} + D_s)]) + b_c,
-// delta_s = expm1(-gamma (r_s - r*)), r* = r_0, asum_{c,s} the coefficient sum of split s's
-// tiles -- the same terms in the same order as the split-combine kernels of
-// launch_reduce_scores -- then the argmax (lowest class on ties).  The other splits' partial sums are read past L1 (__ldcg): their CTAs fenced
-// them before counting themselves finished.  `work` is shared memory of combine_bytes().
-// ---------------------------------------------------------------------------------------
-__host__ __device__ inline size_t combine_bytes(int splits, int C_pad) {
-    return sizeof(float) * ((size_t)splits * C_pad + (size_t)splits * BM + BM + (size_t)BM * C_pad);
-}
-
-__device__ __noinline__ void combine_splits(const TcParams& p, int m0, int splits, float* work) {
-    const int C = p.C, Cs = p.C_pad, tid = threadIdx.x, nth = blockDim.x;
-    float* s_as = work;                          // [splits][C_pad]
-    float* s_delta = s_as + (size_t)splits * Cs;  // [splits][BM]
-    float* s_esc = s_delta + (size_t)splits * BM;  // [BM]
-    float* s_sc = s_esc + BM;                     // [BM][C_pad]
-    for (int i = tid; i < splits * Cs; i += nth) {
-        const int sp = i / Cs, c = i - sp * Cs;
-        float v = 0.f;
-        if (sp > 0 && c < C)
-            for (int t = sp * p.tiles_per_split; t < min(p.n_tiles, (sp + 1) * p.tiles_per_split); ++t)
-                v += __ldg(p.asum_tile + (size_t)t * Cs + c);
-        s_as[i] = v;
-    }
-    for (int i = tid; i < splits * BM; i += nth) {
-        const int sp = i / BM, rl = i - sp * BM, row = m0 + rl;
-        float d = 0.f;
-        if (row < p.n) {
-            const float rstar = __ldcg(p.ref + row);
-            if (sp > 0) d = expm1f(-p.gamma * (__ldcg(p.ref + (size_t)sp * p.n + row) - rstar));
-            else s_esc[rl] = expf(-p.gamma * rstar);
-        }
-        s_delta[i] = d;
-    }
-    __syncthreads();
-    for (int i = tid; i < BM * C; i += nth) {
-        const int rl = i / C, c = i - rl * C, row = m0 + rl;
-        if (row >= p.n) continue;
-        float acc = 0.f;
-        for (int sp = 0; sp < splits; ++sp) {
-            const float d = __ldcg(p.part + ((size_t)sp * p.n + row) * Cs + c);
-            acc += d + s_delta[sp * BM + rl] * (s_as[sp * Cs + c] + d);
-        }
-        const float sc = s_esc[rl] * (__ldg(p.asum + c) + acc) + __ldg(p.bias + c);
-        p.scores[(size_t)row * C + c] = sc;
-        s_sc[rl * Cs + c] = sc;
-    }
-    if (!p.labels) return;
-    __syncthreads();
-    const int lane = tid & 31;
-    for (int rl = tid >> 5; rl < BM; rl += nth >> 5) {
-        if (m0 + rl >= p.n) continue;
-        float best = -INFINITY;
-        int bi = 0x7FFFFFFF;
-        for (int c = lane; c < C; c += 32) {
-            const float v = s_sc[rl * Cs + c];
-            if (v > best) {
-                best = v;
-                bi = c;
-            }
-        }
-        for (int off = 16; off > 0; off >>= 1) {
-            const float ob = __shfl_xor_sync(0xFFFFFFFFu, best, off);
-            const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, off);
-            if (ob > best || (ob == best && oi < bi)) {
-                best = ob;
-                bi = oi;
-            }
-        }
-        if (lane == 0) p.labels[m0 + rl] = bi;
-    }
-}
 
 // ---------------------------------------------------------------------------------------
 // The kernel
@@ -760,6 +682,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         };
         for (int u = 0; u < U && alive; ++u) {
             const int n0 = (t0 + u) * BN;
+            // the tile's norms into L1 while G is computed: read from L2 one batch after the other,
+            // they held up the epilogue of a CTA's first tile for several microseconds
+            if (lane < BN / 32) asm volatile("prefetch.global.L1 [%0];" ::"l"(p.svsq + n0 + 32 * lane));
             // the tile's G: lane 0 polls with short sleeps (a thread suspended in try_wait wakes
             // late, and plain spinning takes issue slots from the warps computing F), then falls
             // back to the bounded wait
@@ -794,10 +719,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                         TC_LD_X32(g_tmem + c * 64 + half * 32, v);
                         tc_wait_ld();
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
+                        for (int j = 0; j < 32; j += 2) {
                             const int col = c * 64 + half * 32 + j;
+                            const float2 sv = __ldg(reinterpret_cast<const float2*>(p.svsq + n0 + col));
                             if (n0 + col < p.n_sv) {
-                                sum += xs + __ldg(p.svsq + n0 + col) - 2.f * p.gscale * __uint_as_float(v[j]);
+                                sum += xs + sv.x - 2.f * p.gscale * __uint_as_float(v[j]);
+                                ++cnt;
+                            }
+                            if (n0 + col + 1 < p.n_sv) {
+                                sum += xs + sv.y - 2.f * p.gscale * __uint_as_float(v[j + 1]);
                                 ++cnt;
                             }
                         }
@@ -827,8 +757,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 #pragma unroll
                     for (int j = 0; j < 32; j += 2) {
                         const int col = n0 + c * 64 + half * 32 + j;
-                        const float d0 = xs + __ldg(p.svsq + col) - 2.f * p.gscale * __uint_as_float(v[half][j]);
-                        const float d1 = xs + __ldg(p.svsq + col + 1) - 2.f * p.gscale * __uint_as_float(v[half][j + 1]);
+                        const float2 sv = __ldg(reinterpret_cast<const float2*>(p.svsq + col));
+                        const float d0 = xs + sv.x - 2.f * p.gscale * __uint_as_float(v[half][j]);
+                        const float d1 = xs + sv.y - 2.f * p.gscale * __uint_as_float(v[half][j + 1]);
                         const float f0 = expm1_near0(-p.gamma * (d0 - r)), f1 = expm1_near0(-p.gamma * (d1 - r));
                         const __nv_bfloat162 hv = __floats2bfloat162_rn(f0, f1);
                         pk[half * 16 + (j >> 1)] = *reinterpret_cast<const uint32_t*>(&hv);
@@ -869,14 +800,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 tc_wait_ld();
                 if (row_ok) {
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) prow[c0 + j] = __uint_as_float(v[j]);
+                    for (int j = 0; j < 16; j += 4)
+                        *reinterpret_cast<float4*>(prow + c0 + j) =
+                            make_float4(__uint_as_float(v[j]), __uint_as_float(v[j + 1]), __uint_as_float(v[j + 2]),
+                                        __uint_as_float(v[j + 3]));
                 }
             }
             if (row_ok) p.ref[(size_t)split * p.n + grow] = r;
-            if (p.fuse) __threadfence();  // this split's sums are visible before it counts as done
         }
     }
 
+    // the split combine may be scheduled now (it waits for this grid to complete); not before: its
+    // blocks would take the SMs without a CTA of this grid from other streams' kernels
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     tc_fence_before();
     __syncwarp();
     if (PAIR)
@@ -892,21 +828,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         else
             asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS)
                          : "memory");
-    }
-    if (p.fuse) {
-        // the last split of this row block to finish adds them all; the ring's shared memory is
-        // free now (every copy and MMA of the CTA has completed)
-        __shared__ int last;
-        if (threadIdx.x == 0) {
-            __threadfence();
-            last = atomicAdd(p.counters + blockIdx.x, 1u) == gridDim.y - 1;
-        }
-        __syncthreads();
-        if (last) {
-            __threadfence();
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the ring was the async proxy's
-            combine_splits(p, m0, (int)gridDim.y, reinterpret_cast<float*>(gbase));
-        }
     }
 }
 
@@ -1430,7 +1351,7 @@ int plan_tc(rgbd_ctx* ctx, const rgbd_svm* m, int n, TcPlan* pl, size_t ws_cap =
     const size_t ref_bytes = sizeof(float) * (size_t)pl->splits * n;
     pl->off_ref = (part_bytes + 255) & ~size_t(255);
     pl->off_cnt = (pl->off_ref + ref_bytes + 255) & ~size_t(255);
-    pl->bytes = pl->off_cnt + sizeof(uint32_t) * (size_t)((pl->mt + 1) / 2 * 2);  // one counter per row block
+    pl->bytes = pl->off_cnt;
     pl->off_gpart = 0;
     return RGBD_OK;
 }
@@ -1543,23 +1464,6 @@ int launch_tc(rgbd_ctx* ctx, const rgbd_svm* m, const void* x, const float* xsq,
     p.idesc_main = make_idesc(pl.fmt, pl.fmt, mma_m, BN);
     p.idesc_second = make_idesc(1, 1, mma_m, m->C_pad);
     p.passes = pl.passes;
-    // Small batches (up to 8 row blocks) combine their splits inside the kernel, in the last CTA
-    // of each row block to finish, which saves a launch on the latency path of a serving batch;
-    // larger ones leave it to the split-combine kernel, which spreads the work over every SM instead
-    // of adding a tail to the last CTAs (on the 4096-row batch the fused combine cost ~9 us more).
-    // The combine also needs its shared memory to fit the ring (every mode's holds >= 140 KB).
-    p.fuse = (pl.mt <= 8 && combine_bytes(pl.splits, m->C_pad) <= (size_t)140 * 1024) ? 1 : 0;
-    p.counters = reinterpret_cast<uint32_t*>(ws + pl.off_cnt);
-    p.asum = m->asum;
-    p.asum_tile = m->asum_tile;
-    p.bias = m->bias;
-    p.scores = scores;
-    p.labels = labels;
-    if (p.fuse) {
-        const cudaError_t ez =
-            cudaMemsetAsync(p.counters, 0, sizeof(uint32_t) * (size_t)((pl.mt + 1) / 2 * 2), s);
-        if (ez != cudaSuccess) return cuda_error(ez, "svm_score: split counters");
-    }
     cudaError_t e;
     switch (mode * 4 + pl.kind) {
         case MODE_SINGLE * 4 + 0: e = launch_mode<MODE_SINGLE, 0>(pl, p, m, tm_x, tm_x2, s); break;
@@ -1572,7 +1476,6 @@ int launch_tc(rgbd_ctx* ctx, const rgbd_svm* m, const void* x, const float* xsq,
         default: e = launch_mode<MODE_PAIR, 3>(pl, p, m, tm_x, tm_x2, s); break;
     }
     if (e != cudaSuccess) return cuda_error(e, "svm_score: tc launch");
-    if (p.fuse) return RGBD_OK;
     return launch_reduce_scores(part, ref, pl.splits, n, m->C, m->C_pad, m->asum, m->asum_tile, pl.tps, pl.nt,
                                 m->bias, m->gamma, scores, labels, s);
 }

@@ -297,3 +297,31 @@ def test_rows_with_and_without_the_quotient_table(B, ctx, orc, crop, dt):
     assert (got[:, :want.shape[1]] == rows).all()
     for k in range(0, 400, 10):
         assert torch.equal(fm[k:k + 10], f) and torch.equal(xm[k:k + 10], x) and torch.equal(qm[k:k + 10], q)
+
+
+@pytest.mark.parametrize("dt,C", [("bf16", 64), ("bf16", 3), ("fp8", 128)])
+def test_split_combines_agree(B, ctx, orc, dt, C):
+    """Up to 1024 rows are combined by a thread per output, more rows by a warp per row: the same
+    terms in the same order, so the same rows give the same bits in a batch of 129, 1024 and 1025
+    rows (one layout of the splits), and they are the fp64 scores within the type's bound."""
+    rng = synth.rng_for(C)
+    n_sv, dim = 5 * 256 + 40, 9 * 59
+    X, SV = synth.poisson_counts(rng, 1025, dim), synth.poisson_counts(rng, n_sv, dim)
+    a, _ = synth.rbf_coefficients(rng, C, n_sv)
+    b = rng.normal(0, 0.01, C).astype(np.float32)
+    model = B.svm_train_data_pack(ctx, dev_u16(SV), dev_f32(a), dev_f32(b), gamma=1.0 / dim, dtype=dt)
+    got = {}
+    ctx.set_tuning(B.TUNE_TC_SPLITS, 3)
+    try:
+        for n in (129, 1024, 1025):
+            x, q = B.lbp_normalize_features(ctx, dev_u16(X[:n]), dt)
+            got[n] = B.svm_score(ctx, model, x, q)
+    finally:
+        ctx.set_tuning(B.TUNE_TC_SPLITS, 0)
+    assert ctx.status() == 0
+    for n in (129, 1024):
+        assert torch.equal(got[n][0], got[1025][0][:n]) and torch.equal(got[n][1], got[1025][1][:n])
+    x64, sv64 = orc.normalize_f64(X[:129]), orc.normalize_f64(SV)
+    ref = orc.svm_rbf(x64, sv64, a, b, 1.0 / dim)
+    err = rel_score_error(got[129][0].cpu().numpy(), ref, rbf_error_scale(x64, sv64, a, b, 1.0 / dim))
+    assert err <= {"bf16": 5e-5, "fp8": 1e-3}[dt]  # the types' stated bounds
