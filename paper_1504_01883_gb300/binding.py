@@ -110,6 +110,10 @@ def _check(rc):
         raise RgbdError(rc, last_error())
 
 
+# Small calls are bound by what runs on the host between two launches, so the per-call helpers stay
+# short: plain integers for pointers (ctypes converts them), the raw stream handle without a Stream
+# object around it, and constant tables at module level.
+
 def _p(t):
     if t is None:
         return None
@@ -117,7 +121,7 @@ def _p(t):
         raise ValueError("tensor must live on the GPU")
     if not t.is_contiguous():
         raise ValueError("tensor must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _centre(c):
@@ -134,9 +138,15 @@ def _centre(c):
     return _p(c)
 
 
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _dt(x):
@@ -147,10 +157,12 @@ def _dt(x):
     return int(x)
 
 
+_X_TORCH = {DT_F32: torch.float32, DT_TF32: torch.float32, DT_BF16: torch.bfloat16, DT_FP8: torch.uint8,
+            DT_BF16X3: torch.bfloat16}
+
+
 def x_torch_dtype(dt):
-    dt = _dt(dt)
-    return {DT_F32: torch.float32, DT_TF32: torch.float32, DT_BF16: torch.bfloat16, DT_FP8: torch.uint8,
-            DT_BF16X3: torch.bfloat16}[dt]
+    return _X_TORCH[_dt(dt)]
 
 
 def x_shape(dt, n, k_pad):
@@ -358,6 +370,7 @@ class SvmModel:
         info = SvmInfo()
         _check(lib().rgbd_svm_get_info(handle, ctypes.byref(info)))
         self.info = info
+        self.n_classes = info.n_classes
 
     @property
     def k_pad(self):
@@ -425,7 +438,7 @@ def svm_train_data_pack(ctx, sv_feats, coef, bias=None, kernel=KERNEL_RBF, gamma
 
 def svm_score(ctx, model, x, xsq=None, x_scale=448.0, scores=None, labels=None, want_labels=True, stream=None):
     n = x.shape[-2]  # rows (a split bf16 buffer is [2][n][k_pad])
-    C = model.info.n_classes
+    C = model.n_classes
     if scores is None:
         scores = torch.empty((n, C), dtype=torch.float32, device=x.device)
     if want_labels and labels is None:
@@ -449,7 +462,7 @@ def svm_score_noalloc(ctx, model, x, xsq, x_scale=448.0, scores=None, labels=Non
     fn.argtypes = [P, P, P, P, ctypes.c_int, ctypes.c_float, P, P, P]
     fn.restype = ctypes.c_int
     n = x.shape[-2]  # rows (a split bf16 buffer is [2][n][k_pad])
-    C = model.info.n_classes
+    C = model.n_classes
     if scores is None:
         scores = torch.empty((n, C), dtype=torch.float32, device=x.device)
     if want_labels and labels is None:
