@@ -46,6 +46,12 @@ struct RoiTest {
         return (uint64_t)(uint32_t)l * d <= parallax && parallax < (uint64_t)(uint32_t)h * d;
     }
 
+    // Whether row i can meet the box's rows between columns ja and jb (Y is linear in the column).
+    __device__ __forceinline__ bool row_meets(int i, int ja, int jb) const {
+        const T Ya = a3 * ja + a4 * i + a5 - Y0, Yb = a3 * jb + a4 * i + a5 - Y0;
+        return !((Ya < 0 && Yb < 0) || (Ya >= Yn && Yb >= Yn));
+    }
+
     // Depths lo .. lo + span outside which no pixel of column j, rows ra..rb, can pass hit();
     // false when there are none.
     __device__ __forceinline__ bool depths(int j, int ra, int rb, uint32_t& lo, uint32_t& span) const {
@@ -63,6 +69,14 @@ struct RoiTest {
     }
 };
 
+// What every face of a launch shares: the range of p(d), and the inverse of the linear part (where
+// there is none to speak of, the whole frame is scanned).
+struct RoiWindow {
+    long long p_lo, p_hi;
+    float ia, ib, ic, id;
+    int degenerate;
+};
+
 // One CTA per face.  The scan covers a window that holds every depth pixel which can map inside
 // the rect: with p(d) = 256 (parallax / d) between p_lo (at d_max) and p_hi (at d_min), a pixel
 // inside needs A = a0 j + a1 i + a2 in [X0 - p_hi, X1 - p_lo) and B = a3 j + a4 i + a5 in [Y0, Y1)
@@ -76,11 +90,13 @@ struct RoiTest {
 // without any pixel is read twice.  What is left is a chain of few L2 or DRAM round trips, so
 // each step issues all its loads first (two rows of the window per warp, 16 rows of a column).
 // 4096 boxes over 256 frames of 640x480, faces of side 48..256: 640 us when every window pixel was
-// tested with a division, 95 us now.
+// tested with a division, 95 us with the scan from the edges, 86 us since rows that cannot meet the box
+// are passed over and what all faces share comes from the host.
 template <typename T>
 __global__ void __launch_bounds__(kRoiThreads) face_roi_kernel(const uint16_t* __restrict__ depth, int n_frames, int H,
-                                                               int W, rgbd_calib c, const rgbd_rect* __restrict__ rects,
-                                                               int n, rgbd_rect* __restrict__ out,
+                                                               int W, rgbd_calib c, RoiWindow wd,
+                                                               const rgbd_rect* __restrict__ rects, int n,
+                                                               rgbd_rect* __restrict__ out,
                                                                uint32_t* __restrict__ status) {
     constexpr int NW = kRoiThreads / 32;
     __shared__ int ext[4];  // least and largest row and column so far
@@ -93,19 +109,18 @@ __global__ void __launch_bounds__(kRoiThreads) face_roi_kernel(const uint16_t* _
         if (bad && tid == 0) atomicOr(status, RGBD_STATUS_BAD_RECT);
         int j0 = 0, j1 = -1, i0 = 0, i1 = -1;  // empty
         if (!bad && cx0 < cx1 && cy0 < cy1) {
-            const long long p_lo = (long long)(c.parallax / c.d_max) * 256;
-            const long long p_hi = (long long)(c.parallax / c.d_min) * 256;
-            const float A[2] = {(float)(cx0 * 65536 - p_hi - c.a[2]), (float)(cx1 * 65536 - p_lo - c.a[2])};
-            const float Bv[2] = {(float)(cy0 * 65536 - c.a[5]), (float)(cy1 * 65536 - c.a[5])};
-            const float det = (float)c.a[0] * (float)c.a[4] - (float)c.a[1] * (float)c.a[3];
-            if (fabsf(det) < 1.0f) {  // degenerate mapping: scan the whole frame
-                j0 = 0, j1 = W - 1, i0 = 0, i1 = H - 1;
+            if (wd.degenerate) {
+                j1 = W - 1, i1 = H - 1;
             } else {
+                const float A[2] = {(float)((T)(cx0 * 65536) - (T)wd.p_hi - c.a[2]),
+                                    (float)((T)(cx1 * 65536) - (T)wd.p_lo - c.a[2])};
+                const float Bv[2] = {(float)((T)(cy0 * 65536) - c.a[5]), (float)((T)(cy1 * 65536) - c.a[5])};
                 float jmn = 3e38f, jmx = -3e38f, imn = 3e38f, imx = -3e38f;
+#pragma unroll
                 for (int u = 0; u < 2; ++u)
+#pragma unroll
                     for (int v = 0; v < 2; ++v) {
-                        const float jj = ((float)c.a[4] * A[u] - (float)c.a[1] * Bv[v]) / det;
-                        const float ii = ((float)c.a[0] * Bv[v] - (float)c.a[3] * A[u]) / det;
+                        const float jj = wd.ia * A[u] + wd.ib * Bv[v], ii = wd.ic * A[u] + wd.id * Bv[v];
                         jmn = fminf(jmn, jj), jmx = fmaxf(jmx, jj);
                         imn = fminf(imn, ii), imx = fmaxf(imx, ii);
                     }
@@ -127,9 +142,11 @@ __global__ void __launch_bounds__(kRoiThreads) face_roi_kernel(const uint16_t* _
             bool top = true, bottom = true;
             for (int s0 = 0; s0 <= i1 - i0 && (top || bottom); s0 += NW) {
                 const int it = i0 + s0 + warp, ib = i1 - s0 - warp;
-                const bool dt = top && it <= i1, db = bottom && ib >= i0;
+                // (a row that is above or below the box at both ends of the window cannot hold one)
+                const bool dt = top && it <= i1 && t.row_meets(it, j0, j1);
+                const bool db = bottom && ib >= i0 && t.row_meets(ib, j0, j1);
                 int tl = INT_MAX, th = -1, bl = INT_MAX, bh = -1;  // columns with a pixel in the two rows
-                for (int jb = j0; jb <= j1; jb += 4 * 32) {
+                for (int jb = j0; jb <= j1 && (dt || db); jb += 4 * 32) {
                     uint32_t d[2][4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
@@ -250,10 +267,23 @@ extern "C" int rgbd_face_roi(rgbd_ctx* ctx, const uint16_t* depth, int n_frames,
         return std::llabs((long long)a) * W + std::llabs((long long)b) * H + std::llabs((long long)o);
     };
     const long long lim = 1ll << 30;
+    RoiWindow wd;
+    wd.p_lo = (long long)(c.parallax / c.d_max) * 256;
+    wd.p_hi = (long long)(c.parallax / c.d_min) * 256;
+    const double det = (double)c.a[0] * c.a[4] - (double)c.a[1] * c.a[3];
+    wd.ia = (float)(c.a[4] / det), wd.ib = (float)(-c.a[1] / det);
+    wd.ic = (float)(-c.a[3] / det), wd.id = (float)(c.a[0] / det);
+    // A window is right to 2 pixels while single precision places its corners to 1; a mapping that
+    // (nearly) collapses a direction has the whole frame scanned.
+    const double a_max = 65536.0 * c.colour_w + (double)wd.p_hi + fabs((double)c.a[2]);
+    const double b_max = 65536.0 * c.colour_h + fabs((double)c.a[5]);
+    const double reach_px = std::max((fabs((double)c.a[4]) * a_max + fabs((double)c.a[1]) * b_max),
+                                     (fabs((double)c.a[3]) * a_max + fabs((double)c.a[0]) * b_max));
+    wd.degenerate = fabs(det) < 1.0 || 4.8e-7 * reach_px > fabs(det);  // 4 roundings of 2^-23
     const bool narrow = reach(c.a[0], c.a[1], c.a[2]) < lim && reach(c.a[3], c.a[4], c.a[5]) < lim &&
-                        c.colour_w < 16384 && c.colour_h < 16384;
+                        c.colour_w < 16384 && c.colour_h < 16384 && wd.p_hi < lim;
     auto kernel = narrow ? face_roi_kernel<int> : face_roi_kernel<long long>;
-    kernel<<<grid, kRoiThreads, 0, (cudaStream_t)stream>>>(depth, n_frames, H, W, c, colour_rects, n, depth_rects,
+    kernel<<<grid, kRoiThreads, 0, (cudaStream_t)stream>>>(depth, n_frames, H, W, c, wd, colour_rects, n, depth_rects,
                                                            ctx->d_status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "rgbd_face_roi: launch");

@@ -55,6 +55,26 @@ def test_face_roi_scan_from_the_edges(B, ctx, orc, shape, colour_w, density):
     ctx.status(clear=True)
 
 
+@pytest.mark.parametrize("a1,a4", [(0, 0), (1, 2), (100, 200), (300, -300), (40000, 70000)])
+def test_face_roi_of_nearly_singular_mappings(B, ctx, orc, a1, a4):
+    """A mapping whose rows are nearly parallel has no window that single precision could place: the
+    whole frame is scanned there, and just short of it the window still holds every pixel."""
+    H, W = 96, 128
+    rng = synth.rng_for(a1 + 7)
+    depth = rng.choice(np.array([0, 0, 0, 900, 1500], np.uint16), (2, H, W))
+    boxes = np.zeros(40, orc.RECT_DTYPE)
+    boxes["frame"] = rng.integers(0, 2, 40)
+    boxes["x"], boxes["y"] = rng.integers(-10, W, 40), rng.integers(-10, H, 40)
+    boxes["w"], boxes["h"] = rng.integers(1, 40, 40), rng.integers(1, 40, 40)
+    cal = synth.calibration(rng, W, H)
+    cal["a"][:] = [65536, a1, 0, 65536, a4, 0]
+    want = orc.face_roi(depth, cal, boxes)
+    got = B.rgbd_face_roi(ctx, dev_u16(depth), B.Calib.from_record(cal), B.rects_tensor(boxes)).cpu().numpy()
+    for i, f in enumerate(["frame", "x", "y", "w", "h"]):
+        assert (got[:, i] == want[f]).all(), f
+    ctx.status(clear=True)
+
+
 @pytest.mark.parametrize("out_h,out_w", [(1, 1), (7, 5), (33, 64), (64, 100), (130, 257), (3, 1300)])
 @pytest.mark.parametrize("W", [8, 101, 320])
 def test_crop_affine_sizes(B, ctx, orc, out_h, out_w, W):
