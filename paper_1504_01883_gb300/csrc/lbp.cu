@@ -386,6 +386,10 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::MINB) lbp_fused_
         }
         if (tid == 0) sm.info[3] = next_face;
         __syncthreads();
+        // With a face per CTA the SMs without one may start on the kernel that follows: the scoring
+        // kernels of few rows load their first SVs while they wait for this grid to complete.  Not
+        // before the pixels are here: against that traffic the 4 us of P1 became 7 to 11.
+        if (a.n <= (int)gridDim.x) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
         // ---- P2: coarse bin of the lower median (rank (n-1)/2 of the non-zero depths) -----
         if (warp == 0) {

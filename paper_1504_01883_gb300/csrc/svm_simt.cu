@@ -137,19 +137,22 @@ constexpr int kSlice = 2048;       // K per slice
 constexpr int kRows8Threads = 256;
 
 template <int MB>
-__global__ void __launch_bounds__(kRows8Threads) rbf_rows8_kernel(const float* __restrict__ x, int n, int k_pad,
+__global__ void __launch_bounds__(kRows8Threads) rbf_rows8_kernel(const float* x, int n, int k_pad,
                                                                   const float* __restrict__ sv, int n_sv, int n_pad,
                                                                   int sv_per_cta, float* __restrict__ gpart,
                                                                   uint32_t* __restrict__ counter) {
     extern __shared__ __align__(16) float xs[];  // [MB][kSlice]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *counter = 0u;  // the epilogue counts on it
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int k0 = blockIdx.x * kSlice, klen = min(kSlice, k_pad - k0);  // a multiple of 128
+    // launched as a programmatic dependent of the kernel that makes the rows (asking L2 for the SVs
+    // before this wait made no difference)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *counter = 0u;  // the epilogue counts on it
     for (int m = 0; m < MB; ++m)
         for (int k = 4 * tid; k < klen; k += 4 * kRows8Threads)
             *reinterpret_cast<float4*>(xs + m * kSlice + k) =
-                __ldg(reinterpret_cast<const float4*>(x + (size_t)min(m, n - 1) * k_pad + k0 + k));
+                __ldcg(reinterpret_cast<const float4*>(x + (size_t)min(m, n - 1) * k_pad + k0 + k));
     __syncthreads();
     const int i1 = min(n_sv, (int)(blockIdx.y + 1) * sv_per_cta);
     for (int i = blockIdx.y * sv_per_cta + 2 * warp; i < i1; i += 2 * (kRows8Threads / 32)) {
@@ -667,9 +670,18 @@ static cudaError_t launch_rows8(const Rows8Plan& p, const float* x, int n, const
     const cudaError_t e =
         cudaFuncSetAttribute(rbf_rows8_kernel<MB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    rbf_rows8_kernel<MB><<<dim3((unsigned)p.kz, (unsigned)p.groups), kRows8Threads, smem, s>>>(
-        x, n, m->k_pad, (const float*)m->sv, m->n_sv, m->n_pad, p.sv_per_cta, gpart, counter);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)p.kz, (unsigned)p.groups, 1);
+    cfg.blockDim = dim3(kRows8Threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, rbf_rows8_kernel<MB>, x, n, m->k_pad, (const float*)m->sv, m->n_sv, m->n_pad,
+                              p.sv_per_cta, gpart, counter);
 }
 
 // Up to 8 rows are bound by reading the SVs; more rows by the products.  The epilogue combines at

@@ -212,6 +212,15 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
         "l"((uint64_t)map), "r"(x), "r"(y), "r"(bar)
         : "memory");
 }
+// The same with an L2 policy.
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar,
+                                            uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, "
+        "{%2, %3}], [%4], %5;" ::"r"(dst),
+        "l"((uint64_t)map), "r"(x), "r"(y), "r"(bar), "l"(policy)
+        : "memory");
+}
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -841,6 +850,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 // SVs; each CTA writes its partial G = X . SV_t^T of the valid rows to `gpart`
 // ([kz][n][n_pad]), and rbf_splitk_epilogue_kernel adds the ranges, finishes the tile and, in
 // the last CTA of each row group, combines the tiles into scores and labels.
+// Launched as a programmatic dependent: behind a feature kernel of few faces its CTAs start on the SMs
+// without a face and hold their first SV blocks when the rows are there (a frame of up to 7 faces
+// against 8192 SVs: 80.7 -> 77.5 us; asking L2 for up to 64 MB more of the SVs meanwhile gained nothing,
+// and slowed the features where it met their pixels).
 // Warps: 0 the TMA producer (4 stages of X and SV k-blocks), 1 the TMEM owner and MMA issuer,
 // 2-5 the epilogue (one thread per row, TMEM lane quarter = warp % 4).  The X copies hold only
 // the batch's rows (rounded up to 8, the swizzle atom's height): the MMA still reads 128 rows,
@@ -887,8 +900,6 @@ __global__ void __launch_bounds__(SK_WARPS * 32, 1)
     const int KT = p.passes * p.k_blocks;
     const int kt0 = z * p.kpz, kt1 = min(KT, kt0 + p.kpz);  // non-empty: the host sizes kz so
 
-    if (blockIdx.x == 0 && blockIdx.y == 0)  // the epilogue kernel that follows counts on these
-        for (int i = threadIdx.x; i < p.n_groups; i += blockDim.x) p.counters[i] = 0u;
     // the epilogue kernel may be scheduled now: its CTAs wait (griddepcontrol.wait) for this grid
     // to complete, so its launch latency hides behind this kernel instead of following it
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -919,15 +930,33 @@ __global__ void __launch_bounds__(SK_WARPS * 32, 1)
         if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0, armed = 0, armed_par = 0;
-            for (int kt = kt0; kt < kt1; ++kt) {
+            // Each SV block is read once a call, and a large model does not fit L2: as the first to be
+            // evicted the blocks make room for one another, so that part of the model stays for the next
+            // call (247 MB of SVs, frame after frame: 72.5 us a frame, 77.5 us without).
+            uint64_t streamed;
+            asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(streamed));
+            auto load_x = [&](int kt, int st) {
                 const int pass = kt / p.k_blocks, kb = kt - pass * p.k_blocks;
-                const CUtensorMap* mx = (pass == 2) ? &tm_x2 : &tm_x;
-                const CUtensorMap* msv = (pass == 1) ? &tm_sv2 : &tm_sv;
+                tma_load_2d(base + (uint32_t)st * SK_STAGE, (pass == 2) ? &tm_x2 : &tm_x, kb * p.k_elems, 0,
+                            bar(SK_FULL + st));
+            };
+            auto load_sv = [&](int kt, int st) {
+                const int pass = kt / p.k_blocks, kb = kt - pass * p.k_blocks;
+                bar_arrive_tx(bar(SK_FULL + st), p.x_bytes + SV_TILE);
+                tma_load_2d(base + (uint32_t)st * SK_STAGE + X_TILE, (pass == 1) ? &tm_sv2 : &tm_sv, kb * p.k_elems,
+                            tile * BN, bar(SK_FULL + st), streamed);
+            };
+            // the model is there before this kernel may start: the first stages' SVs need not wait
+            // (its wait limits, and those of the other warps, count from the kernel before it on)
+            const int first = min(SK_STAGES, kt1 - kt0);
+            for (int i = 0; i < first; ++i) load_sv(kt0 + i, i);
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            if (blockIdx.x == 0 && blockIdx.y == 0)  // the epilogue kernel that follows counts on these
+                for (int i = 0; i < p.n_groups; ++i) p.counters[i] = 0u;
+            for (int kt = kt0; kt < kt1; ++kt) {
                 if (!bar_spin<false>(bar(SK_EMPTY + stage), phase ^ 1u, abort_flag, p.status)) break;
-                const uint32_t sa = base + (uint32_t)stage * SK_STAGE;
-                bar_arrive_tx(bar(SK_FULL + stage), p.x_bytes + SV_TILE);
-                tma_load_2d(sa, mx, kb * p.k_elems, 0, bar(SK_FULL + stage));
-                tma_load_2d(sa + X_TILE, msv, kb * p.k_elems, tile * BN, bar(SK_FULL + stage));
+                if (kt >= kt0 + first) load_sv(kt, stage);
+                load_x(kt, stage);
                 armed |= 1u << stage;
                 armed_par = (armed_par & ~(1u << stage)) | (phase << stage);
                 if (++stage == SK_STAGES) {
@@ -946,6 +975,7 @@ __global__ void __launch_bounds__(SK_WARPS * 32, 1)
     } else if (warp == 1) {
         // ===================== MMA issuer =====================
         if (lane == 0) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
             int stage = 0;
             uint32_t phase = 0;
             bool alive = true;
@@ -979,6 +1009,7 @@ __global__ void __launch_bounds__(SK_WARPS * 32, 1)
         const int quarter = warp & 3;
         const int row = quarter * 32 + lane;
         bool ok = false;
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         if (lane == 0) ok = bar_wait<false>(bar(SK_GFULL), 0, abort_flag, p.status);
         if (__shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0)) {
             tc_fence_after();
@@ -1053,12 +1084,13 @@ __global__ void __launch_bounds__(SKE_THREADS) rbf_splitk_epilogue_kernel(
                          : "memory");
     }
     float sv[PER];
-    const float xs = warp < rows ? xsq[k0 + warp] : 0.f;
 #pragma unroll
     for (int j = 0; j < PER; ++j) sv[j] = svsq[tile * BN + lane + 32 * j];
     // launched as a programmatic dependent of the partial-product kernel: wait for it to complete
+    // (and so for the kernels before it, which it may have overtaken: only the model is read above)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (warp < rows) {
+        const float xs = __ldcg(xsq + k0 + warp);
         const float* gp = gpart + (size_t)(k0 + warp) * n_pad + tile * BN + lane;
         float g[PER];
 #pragma unroll
@@ -1363,9 +1395,17 @@ cudaError_t launch_splitk(const TcPlan& pl, const SkParams& sp, const rgbd_svm* 
     cudaError_t e = cudaFuncSetAttribute(rbf_tc_splitk_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          SK_SMEM);
     if (e != cudaSuccess) return e;
-    rbf_tc_splitk_kernel<KIND><<<dim3((unsigned)pl.nt, (unsigned)pl.kz), SK_WARPS * 32, SK_SMEM, s>>>(
-        tm_x, m->tm_sv, tm_x2, m->tm_sv_lo, sp);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)pl.nt, (unsigned)pl.kz, 1);
+    cfg.blockDim = dim3(SK_WARPS * 32, 1, 1);
+    cfg.dynamicSmemBytes = SK_SMEM;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, rbf_tc_splitk_kernel<KIND>, tm_x, m->tm_sv, tm_x2, m->tm_sv_lo, sp);
 }
 
 // Launches one instantiation: single CTAs on a (row blocks, splits) grid, pairs as clusters of

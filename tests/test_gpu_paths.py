@@ -345,3 +345,38 @@ def test_split_combines_agree(B, ctx, orc, dt, C):
     ref = orc.svm_rbf(x64, sv64, a, b, 1.0 / dim)
     err = rel_score_error(got[129][0].cpu().numpy(), ref, rbf_error_scale(x64, sv64, a, b, 1.0 / dim))
     assert err <= {"bf16": 5e-5, "fp8": 1e-3}[dt]  # the types' stated bounds
+
+
+@pytest.mark.parametrize("dt", ["bf16", "fp8", "bf16x3", "f32"])
+@pytest.mark.parametrize("faces", [1, 7, 40])
+def test_scores_right_behind_their_features(B, ctx, orc, faces, dt):
+    """The scoring kernels of few rows start before the feature kernel in front of them has finished:
+    frame after frame without a pause gives the same bits as with the GPU waited for in between."""
+    rng = synth.rng_for(faces)
+    H, W, n_sv, C, frames = 240, 320, 700, 12, 12
+    grey = dev_u8(rng.integers(0, 256, (frames, H, W), np.uint8))
+    depth = dev_u16(rng.integers(700, 1300, (frames, H, W)).astype(np.uint16))
+    sv = dev_u16(rng.poisson(1.1, (n_sv, 64 * 59)).clip(0, 64).astype(np.uint16))
+    coef = dev_f32(rng.normal(size=(C, n_sv)).astype(np.float32))
+    model = B.svm_train_data_pack(ctx, sv, coef, gamma=0.02, dtype=dt)
+    rects = []
+    for f in range(frames):
+        r = np.zeros(faces, orc.RECT_DTYPE)
+        r["frame"], r["w"], r["h"] = f, rng.integers(30, 120, faces), rng.integers(30, 120, faces)
+        r["x"], r["y"] = rng.integers(0, 200, faces), rng.integers(0, 120, faces)
+        rects.append(B.rects_tensor(r))
+    # one buffer for all frames' rows: rows read too early would be the frame before's
+    _, x, xsq = B.lbp_fused_features(ctx, grey, depth, rects[0], crop=64, feats=False, x_dtype=dt)
+
+    def scores(pause):
+        out = []
+        for r in rects:
+            B.lbp_fused_features(ctx, grey, depth, r, crop=64, feats=False, x_dtype=dt, out={"x": x, "xsq": xsq})
+            if pause:
+                torch.cuda.synchronize()
+            out.append(B.svm_score(ctx, model, x, xsq))
+        return out
+
+    for (s0, l0), (s1, l1) in zip(scores(True), scores(False)):
+        assert torch.equal(s0, s1) and torch.equal(l0, l1)
+    assert ctx.status() == 0
