@@ -135,7 +135,8 @@ int rgbd_ctx_status(rgbd_ctx* ctx, uint32_t* flags, int clear);
  * path; scores change within rounding (the split of the SV sum).
  *   RGBD_TUNE_LBP_CTAS_PER_SM   resident fused-kernel CTAs per SM (1 or 2)
  *   RGBD_TUNE_TC_SPLITS         SV-tile ranges per 128-row block in tensor-core scoring
- *   RGBD_TUNE_LBP_SHAPE         fused-kernel tile shape: 0 = default (2), 1 = one thread
+ *   RGBD_TUNE_LBP_SHAPE         fused-kernel tile shape: 0 = default (2; 3 for crops of 64 and
+ *                               96 and at most a face per SM), 1 = one thread
  *                               per 8 x 8 cell (crops 64 and 128; CTAs of (crop/8)^2
  *                               threads), 2 = one thread per 4 x 8 half cell (CTAs of
  *                               2 (crop/8)^2 threads), 3 = one thread per 4 x 4 quarter

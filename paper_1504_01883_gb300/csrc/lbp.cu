@@ -97,6 +97,9 @@ struct Cfg {
     static constexpr int IPT = S * S / 4 / NT;  // 4-pixel groups per thread
     static constexpr int DIM = G * G * kBins;
     static constexpr int HW = 15;            // histogram words per thread (60 bins / 4)
+    // Threads that write a face's rows: those of two threads per cell for the larger crops, so that the
+    // norm is summed in one order whatever the shape.
+    static constexpr int OT = TPC == 4 && S > 32 ? NT / 2 : NT;
     // CTAs per SM that the registers are to allow (64 to 72 a thread): smaller crops need more of
     // them to hide the same latencies.  585 faces at 96 x 96: 67 us at one CTA of 206 registers per SM,
     // 51 us at three.
@@ -677,7 +680,7 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::MINB) lbp_fused_
                           ((reinterpret_cast<size_t>(a.feats) | reinterpret_cast<size_t>(a.x_out)) & 15) == 0;
         if (wide) {
             // bf16 rows, 8 values per thread step (16-byte loads and stores)
-            for (int j8 = tid; j8 < a.k_pad / 8; j8 += NT) {
+            for (int j8 = tid; tid < C::OT && j8 < a.k_pad / 8; j8 += C::OT) {
                 const int j = 8 * j8;
                 uint4 hv = make_uint4(0u, 0u, 0u, 0u);
                 uint32_t pk[4] = {0u, 0u, 0u, 0u};
@@ -710,7 +713,7 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::MINB) lbp_fused_
             }
         }
         const int len4 = wide ? 0 : (x_dtype ? a.k_pad : DIM) / 4;
-        for (int j4 = tid; j4 < len4; j4 += NT) {
+        for (int j4 = tid; tid < C::OT && j4 < len4; j4 += C::OT) {
             const int j = 4 * j4;
             uint2 hv = make_uint2(0, 0);
             if (j < DIM) {
@@ -817,7 +820,7 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::MINB) lbp_fused_
             __syncthreads();
             if (tid == 0) {
                 float t = 0.f;
-                for (int w = 0; w < NT / 32; ++w) t += sm.red[w];
+                for (int w = 0; w < C::OT / 32; ++w) t += sm.red[w];
                 a.xsq[face] = t;
             }
         }
@@ -861,25 +864,29 @@ int launch_fused_t(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
 // with the table, 18.9 us without).
 template <int S, int TPC>
 int launch_fused_s(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
-    const bool table = S >= 96 && a.n > ctx->props.sm_count && a.x_out && a.x_dtype == RGBD_DT_BF16 && !a.x_centre;
-    return table ? launch_fused_t<S, TPC, S >= 96>(ctx, a, s) : launch_fused_t<S, TPC, false>(ctx, a, s);
+    constexpr bool kTable = S == 128 || (S == 96 && TPC == 2);
+    const bool table = kTable && a.n > ctx->props.sm_count && a.x_out && a.x_dtype == RGBD_DT_BF16 && !a.x_centre;
+    return table ? launch_fused_t<S, TPC, kTable>(ctx, a, s) : launch_fused_t<S, TPC, false>(ctx, a, s);
 }
 
 }  // namespace
 
 int launch_lbp_fused(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
     if (a.flags & RGBD_LBP_FACE_HIST256) return launch_face256(ctx, a, s);
-    // tile shape (crops 64 and 128): one thread per cell (tuning value 1), per half cell (2, the
-    // default), per quarter cell (3: 1024-thread CTAs at 128, 50 % slower on full batches).  Crops of
-    // 32 have a cell's quarter per thread: one warp of halves is 16 us for a face and 22.8 us for 2048,
-    // two of quarters 8.4 and 20.4 us.
-    const int shape = ctx->tune_lbp_shape == 0 ? 2 : ctx->tune_lbp_shape;
+    // tile shape: one thread per cell (tuning value 1; crops 64 and 128), per half cell (2), per quarter
+    // cell (3).  Quarters halve a face's steps where there is a face per SM at most (1 to 152 faces: 12.1
+    // -> 9.5 us at 64, 14.8 -> 13.4 us at 96; 15.5 and 15.9 us at 128, whose CTAs of 512 threads have the
+    // warps already) and cost a full batch half as much again at 128.  Crops of 32 always have a cell's
+    // quarter per thread: one warp of halves is 16 us for a face and 22.8 us for 2048, two of quarters
+    // 8.4 and 20.4 us.
+    const bool few = ctx->tune_lbp_shape == 0 && a.n <= ctx->props.sm_count && a.crop < 128;
+    const int shape = ctx->tune_lbp_shape ? ctx->tune_lbp_shape : (few ? 3 : 2);
     switch (a.crop) {
         case 32: return launch_fused_s<32, 4>(ctx, a, s);
         case 64:
             return shape == 1 ? launch_fused_s<64, 1>(ctx, a, s)
                               : (shape == 3 ? launch_fused_s<64, 4>(ctx, a, s) : launch_fused_s<64, 2>(ctx, a, s));
-        case 96: return launch_fused_s<96, 2>(ctx, a, s);
+        case 96: return few ? launch_fused_s<96, 4>(ctx, a, s) : launch_fused_s<96, 2>(ctx, a, s);
         case 128:
             return shape == 1 ? launch_fused_s<128, 1>(ctx, a, s)
                               : (shape == 3 ? launch_fused_s<128, 4>(ctx, a, s) : launch_fused_s<128, 2>(ctx, a, s));

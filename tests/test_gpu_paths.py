@@ -380,3 +380,19 @@ def test_scores_right_behind_their_features(B, ctx, orc, faces, dt):
     for (s0, l0), (s1, l1) in zip(scores(True), scores(False)):
         assert torch.equal(s0, s1) and torch.equal(l0, l1)
     assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("crop", [64, 96])
+@pytest.mark.parametrize("dt,flags", [("bf16", 0), ("fp8", 3), ("f32", 1), ("bf16x3", 2)])
+def test_few_faces_give_the_bits_of_a_batch(B, ctx, orc, crop, dt, flags):
+    """Up to a face per SM takes four threads per cell, a larger batch two: the same counts, rows and
+    norms to the bit, and counts as the oracle's."""
+    grey, depth, r = synth.frames_with_rects(crop, 10, 17, 20, 110, H=120, W=160)
+    g, d = dev_u8(grey), dev_u16(depth)
+    fb, xb, qb = B.lbp_fused_features(ctx, g, d, B.rects_tensor(r), crop=crop, flags=flags, x_dtype=dt)
+    for k in (1, 40, 152):
+        f, x, q = B.lbp_fused_features(ctx, g, d, B.rects_tensor(r[:k]), crop=crop, flags=flags, x_dtype=dt)
+        whole = xb[:, :k] if dt == "bf16x3" else xb[:k]
+        assert torch.equal(f, fb[:k]) and torch.equal(x, whole) and torch.equal(q, qb[:k])
+    want = orc.features_batch(grey, depth, r[:40], crop, flags=flags)
+    assert (host_u16(fb[:40]) == want).all()
