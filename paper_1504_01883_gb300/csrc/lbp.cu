@@ -100,10 +100,13 @@ struct Cfg {
     // Threads that write a face's rows: those of two threads per cell for the larger crops, so that the
     // norm is summed in one order whatever the shape.
     static constexpr int OT = TPC == 4 && S > 32 ? NT / 2 : NT;
-    // CTAs per SM that the registers are to allow (64 to 72 a thread): smaller crops need more of
-    // them to hide the same latencies.  585 faces at 96 x 96: 67 us at one CTA of 206 registers per SM,
-    // 51 us at three.
-    static constexpr int MINB = S == 32 ? 16 : (TPC == 4 ? 1 : (S == 128 ? 2 : (S == 96 ? 3 : 8)));
+    // CTAs per SM that the registers are to allow (56 to 72 a thread): smaller crops need more of
+    // them to hide the same latencies.  585 faces at 96 x 96, fp8 rows: 67 us at one CTA of 206
+    // registers per SM, 51 us at three, 39 at four (4096 faces: 224 us at three, 215 at four, 229
+    // at five); with the quotient table shared memory holds three.
+    static constexpr int minb(bool table) {
+        return S == 32 ? 16 : (TPC == 4 ? 1 : (S == 128 ? 2 : (S == 96 ? (table ? 3 : 4) : 8)));
+    }
     static constexpr int RPT = TPC == 4 ? 4 : 8;        // cell rows a thread walks in P5
     static constexpr int WPT = (HW + TPC - 1) / TPC;    // histogram words a thread stages in P6
     static_assert(TPC == 1 || TPC == 2 || TPC == 4, "one, two or four threads per cell");
@@ -146,7 +149,7 @@ struct __align__(16) Smem {
 
 // TABLE: bf16 quotients from a table in shared memory.
 template <int S, int TPC, bool TABLE>
-__global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::MINB) lbp_fused_kernel(LbpArgs a) {
+__global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::minb(TABLE)) lbp_fused_kernel(LbpArgs a) {
     using C = Cfg<S, TPC>;
     constexpr int IPT = C::IPT;
     constexpr int NT = C::NT, SW = C::SW, G = C::G, DIM = C::DIM;
