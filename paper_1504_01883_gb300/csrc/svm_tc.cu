@@ -109,6 +109,7 @@ struct TcParams {
     uint32_t idesc_main;
     uint32_t idesc_second;
     int passes;       // 1, or 3 for split bf16 operands (RGBD_DT_BF16X3)
+    int sv_once;      // SV blocks are the first to be evicted from L2
 };
 
 // ---------------------------------------------------------------------------------------
@@ -248,6 +249,20 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
         " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
         "l"((uint64_t)map), "r"(x), "r"(y), "r"(bar_cluster)
         : "memory");
+}
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int x, int y,
+                                                 uint32_t bar_cluster, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2.L2::cache_hint"
+        " [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(dst),
+        "l"((uint64_t)map), "r"(x), "r"(y), "r"(bar_cluster), "l"(policy)
+        : "memory");
+}
+// L2 policy of data read once or by few CTAs at a time: the first to be evicted.
+__device__ __forceinline__ uint64_t policy_evict_first() {
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
 }
 __device__ __forceinline__ void tc_commit2(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -452,6 +467,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             int stage = 0;
             uint32_t phase = 0, armed = 0, armed_par = 0;
             bool alive = true;
+            const uint64_t once = policy_evict_first();
             const int KT = p.passes * p.k_blocks;  // k-blocks per tile
             for (int u = 0; u < U && alive; ++u) {
                 const int n0 = (t0 + u) * BN;
@@ -477,7 +493,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                             bar_arrive_tx(bar(B_FULL + stage / GRP), 2u * L::STAGE * nst);
                         }
                         tma_load_2d_pair(sa, mx, kb * p.k_elems, m0, fb);
-                        tma_load_2d_pair(sa + X_TILE, msv, kb * p.k_elems, n0 + (int)crank * (BN / 2), fb);
+                        if (p.sv_once)
+                            tma_load_2d_pair(sa + X_TILE, msv, kb * p.k_elems, n0 + (int)crank * (BN / 2), fb, once);
+                        else
+                            tma_load_2d_pair(sa + X_TILE, msv, kb * p.k_elems, n0 + (int)crank * (BN / 2), fb);
                     } else {
                         bar_arrive_tx(bar(B_FULL + stage), L::STAGE);
                         tma_load_2d(sa, mx, kb * p.k_elems, m0, bar(B_FULL + stage));
@@ -933,8 +952,7 @@ __global__ void __launch_bounds__(SK_WARPS * 32, 1)
             // Each SV block is read once a call, and a large model does not fit L2: as the first to be
             // evicted the blocks make room for one another, so that part of the model stays for the next
             // call (247 MB of SVs, frame after frame: 72.5 us a frame, 77.5 us without).
-            uint64_t streamed;
-            asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(streamed));
+            const uint64_t streamed = policy_evict_first();
             auto load_x = [&](int kt, int st) {
                 const int pass = kt / p.k_blocks, kb = kt - pass * p.k_blocks;
                 tma_load_2d(base + (uint32_t)st * SK_STAGE, (pass == 2) ? &tm_x2 : &tm_x, kb * p.k_elems, 0,
@@ -1504,6 +1522,11 @@ int launch_tc(rgbd_ctx* ctx, const rgbd_svm* m, const void* x, const float* xsq,
     p.idesc_main = make_idesc(pl.fmt, pl.fmt, mma_m, BN);
     p.idesc_second = make_idesc(1, 1, mma_m, m->C_pad);
     p.passes = pl.passes;
+    // Up to six row blocks, three pairs read an SV block at about the same time and nothing else of the
+    // call reads it again: it makes room in L2 first (fp8 x 8192 SVs: 63.8 -> 62.0 us for 300 rows, 68.2 ->
+    // 64.2 for 500, 98.4 -> 97.5 for 700).  From eight on the pairs drift apart and meet it again: 2 to
+    // 5 % slower at 1000 split bf16 rows and 4096 bf16 rows.
+    p.sv_once = pl.mt <= 6;
     cudaError_t e;
     switch (mode * 4 + pl.kind) {
         case MODE_SINGLE * 4 + 0: e = launch_mode<MODE_SINGLE, 0>(pl, p, m, tm_x, tm_x2, s); break;
