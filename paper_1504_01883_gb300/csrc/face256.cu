@@ -93,10 +93,10 @@ __global__ void __launch_bounds__(F256_THREADS, 1) lbp_face256_kernel(const LbpA
                 if (a.affine) {
                     for (int i = 0; i < 6; ++i) aff[i] = a.affine[6 * (size_t)face + i];
                 } else {
-                    win = windows(r.w, S, a.grey, a.W);
+                    win = windows(r.w, S, a.grey, a.W) != WIN_NONE;  // (pairs: a window per group is 3 % slower here)
                     for (int i = tid; i < 2 * SW + S; i += F256_THREADS) {
                         if (i < 2 * SW) {
-                            const PairTaps p = make_pair_taps(r.x, r.w, S, i, a.W, win);
+                            const PairTaps p = make_pair_taps(r.x, r.w, S, i, a.W, win ? WIN_PAIR : WIN_NONE);
                             const int at = (i & 1) * SW + (i >> 1);
                             cm[at] = p.c;
                             nn[at] = p.nearest;
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(F256_THREADS, 1) lbp_face256_kernel(const LbpA
             if (ok) {
                 if (a.rects && !a.affine) {
                     const PairTaps pair[2] = {{cm[q], nn[q]}, {cm[SW + q], nn[SW + q]}};
-                    sample_group(gsrc, dsrc, rm[v], pair, win, gw, d01, d23);
+                    sample_group(gsrc, dsrc, rm[v], pair, win ? WIN_PAIR : WIN_NONE, gw, d01, d23);
                 } else {
                     uint32_t dv[4];
 #pragma unroll

@@ -47,24 +47,30 @@ __device__ __forceinline__ uint32_t bilerp(const uint8_t* img, int W, uint32_t c
 // column in the aligned 8-byte window that starts at byte wb (kept above .x's selector), .y / .w =
 // byte weights (255 - fx, fx, 1, 0), so that a permute and a 4-way dot product give
 // 256 p(o) + fx (p(o + dx) - p(o)).  Neighbouring taps are at most 2 apart, so every offset is at
-// most 7.  .nearest: the two nearest columns.
+// most 7.  Rects no wider than the crop (WIN_GROUP): taps of the group's four columns are at most 3
+// apart, and both pairs' selectors count from the window of the group's first column.
+// .nearest: the two nearest columns.
 struct PairTaps {
     uint4 c;
     uint32_t nearest;
 };
-__device__ __forceinline__ bool windows(int rect_w, int out, const uint8_t* grey, int W) {
-    return rect_w <= 2 * out && (W & 3) == 0 && W >= 8 && (reinterpret_cast<size_t>(grey) & 3) == 0;
+enum { WIN_NONE = 0, WIN_PAIR = 1, WIN_GROUP = 2 };
+__device__ __forceinline__ int windows(int rect_w, int out, const uint8_t* grey, int W) {
+    if (rect_w > 2 * out || (W & 3) != 0 || W < 8 || (reinterpret_cast<size_t>(grey) & 3) != 0) return WIN_NONE;
+    return rect_w <= out ? WIN_GROUP : WIN_PAIR;
 }
-__device__ __forceinline__ PairTaps make_pair_taps(int x, int w, int out, int i, int W, bool win) {
+__device__ __forceinline__ PairTaps make_pair_taps(int x, int w, int out, int i, int W, int win) {
     const uint2 t0 = make_tap(rect_coord_q16(x, w, out, min(2 * i, out - 1)), W);
     const uint2 t1 = make_tap(rect_coord_q16(x, w, out, min(2 * i + 1, out - 1)), W);
     PairTaps p;
     p.nearest = t0.y | (t1.y << 16);
-    if (!win) {
+    if (win == WIN_NONE) {
         p.c = make_uint4(t0.x, 0u, t1.x, 0u);
         return p;
     }
-    const uint32_t wb = min(t0.x & 0xFFFCu, (uint32_t)W - 8u);
+    const uint32_t first = win == WIN_GROUP && (i & 1) ? make_tap(rect_coord_q16(x, w, out, min(2 * i - 2, out - 1)), W).x
+                                                       : t0.x;
+    const uint32_t wb = min(first & 0xFFFCu, (uint32_t)W - 8u);
     auto sel = [&](uint32_t t) {
         const uint32_t o = (t & 0xFFFFu) - wb, od = o + ((t >> 16) & 1u);
         return o | (od << 4) | (o << 8);
@@ -85,20 +91,23 @@ __device__ __forceinline__ uint4 make_row_taps(int y, int h, int out, int v, int
 // Four neighbouring crop pixels from the taps of their two column pairs and of their row: grey in
 // the bytes of gw, depth in the halves of d01 and d23.
 __device__ __forceinline__ void sample_group(const uint8_t* gsrc, const uint16_t* dsrc, uint4 row,
-                                             const PairTaps (&pair)[2], bool win, uint32_t& gw, uint32_t& d01,
+                                             const PairTaps (&pair)[2], int win, uint32_t& gw, uint32_t& d01,
                                              uint32_t& d23) {
     const uint32_t fy = row.w;
     const uint8_t* g0 = gsrc + row.x;
     const uint8_t* g1 = gsrc + row.y;
     const uint16_t* drow = dsrc + row.z;
     uint32_t acc[4], dv[4];  // acc: the grey value in byte 2
+    uint32_t a0 = 0, a1 = 0, b0 = 0, b1 = 0;
 #pragma unroll
     for (int e2 = 0; e2 < 2; ++e2) {
         const uint4 c = pair[e2].c;
         if (win) {
-            const uint32_t* w0 = reinterpret_cast<const uint32_t*>(g0 + (c.x >> 16));
-            const uint32_t* w1 = reinterpret_cast<const uint32_t*>(g1 + (c.x >> 16));
-            const uint32_t a0 = __ldg(w0), a1 = __ldg(w0 + 1), b0 = __ldg(w1), b1 = __ldg(w1 + 1);
+            if (e2 == 0 || win == WIN_PAIR) {
+                const uint32_t* w0 = reinterpret_cast<const uint32_t*>(g0 + (c.x >> 16));
+                const uint32_t* w1 = reinterpret_cast<const uint32_t*>(g1 + (c.x >> 16));
+                a0 = __ldg(w0), a1 = __ldg(w0 + 1), b0 = __ldg(w1), b1 = __ldg(w1 + 1);
+            }
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 const uint32_t h0 = __dp4a(__byte_perm(a0, a1, j ? c.z : c.x), j ? c.w : c.y, 0u);
