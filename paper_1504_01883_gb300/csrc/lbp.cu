@@ -8,8 +8,8 @@
 // The fused kernel is persistent: one CTA per half-SM slot walks over faces.  Per face:
 //   P1  every thread resamples 8 groups of 4 crop pixels (grey bilinear, depth nearest;
 //       for rects at most 2 S wide the grey taps of two neighbouring pixels come from one
-//       aligned 8-byte window per source row, and each horizontal interpolation is one byte
-//       permute and one 4-way byte dot product); grey and depth go to shared memory (the
+//       aligned 8-byte window per source row, up to S wide those of all four, and each
+//       horizontal interpolation is one byte permute and one 4-way byte dot product); grey and depth go to shared memory (the
 //       depths share their space with the P5 histograms) and the depths are counted into a
 //       coarse histogram of 1024 mm bins (eight 8-bit counters per thread in one 64-bit word,
 //       summed over the warp with redux).
@@ -113,8 +113,9 @@ struct Cfg {
 };
 
 // Where a face's pixels come from: nowhere (a bad rect), crops cut beforehand, a rect by 8-byte
-// windows or by byte gathers, a general affine map.
-enum { SRC_NONE, SRC_CROPS, SRC_WINDOWS, SRC_RECT, SRC_AFFINE };
+// windows of two columns or (no wider than the crop) of four, or by byte gathers, a general affine
+// map.  (Windows of four halve the grey loads: 287.5 -> 284.9 us for 4096 faces of side 48..256.)
+enum { SRC_NONE, SRC_CROPS, SRC_WINDOWS, SRC_GROUP, SRC_RECT, SRC_AFFINE };
 
 template <int S, int TPC = 2>
 struct __align__(16) Smem {
@@ -235,7 +236,9 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::minb(TABLE)) lbp
                             // for S crop columns, neighbouring taps are at most 2 apart, so
                             // o, o + dx <= 7 (the window start is clamped to W - 8).
                             const uint32_t x_prev = __shfl_up_sync(FULL, t.x, 1);
-                            const uint32_t x_first = (i & 1) ? x_prev : t.x;
+                            // (rects no wider than the crop: the group's first column)
+                            const uint32_t x_four = __shfl_sync(FULL, t.x, lane & ~3);
+                            const uint32_t x_first = r.w <= S ? x_four : ((i & 1) ? x_prev : t.x);
                             const uint32_t wb = min((x_first & 0xFFFCu), (uint32_t)a.W - 8u);
                             const uint32_t xa = t.x & 0xFFFFu, dx = (t.x >> 16) & 1u, fx = t.x >> 24;
                             const uint32_t o = xa - wb, od = xa + dx - wb;
@@ -283,7 +286,7 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::minb(TABLE)) lbp
                     const uint2 dd = __ldg(reinterpret_cast<const uint2*>(dsrc) + item);
                     d01 = dd.x;
                     d23 = dd.y;
-                } else if constexpr (SRC == SRC_WINDOWS || SRC == SRC_RECT) {
+                } else if constexpr (SRC == SRC_WINDOWS || SRC == SRC_GROUP || SRC == SRC_RECT) {
                     const uint2 rm = sm.rowmap[v];
                     const uint32_t fy = rm.x >> 24;
                     const uint8_t* g0 = gsrc + (size_t)(rm.x & 0xFFFFu) * a.W;
@@ -291,16 +294,20 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::minb(TABLE)) lbp
                     const uint16_t* drow = dsrc + (size_t)rm.y * a.W;
                     const uint4* cm4 = reinterpret_cast<const uint4*>(sm.colmap);
                     uint32_t dv[4];
+                    uint32_t a0 = 0, a1 = 0, b0 = 0, b1 = 0;  // the window's words in the two rows
                     uint32_t accv[4];  // (acc + 2^15) per pixel, the rounded value in byte 2
 #pragma unroll
                     for (int e2 = 0; e2 < 2; ++e2) {
                         const uint4 cc = cm4[e2 * SW + q];  // taps of columns 4q + 2 e2 and + 1
-                        if constexpr (SRC == SRC_WINDOWS) {
+                        if constexpr (SRC == SRC_WINDOWS || SRC == SRC_GROUP) {
                             const uint32_t nn = reinterpret_cast<const uint32_t*>(sm.ncol)[e2 * SW + q];
                             const uint32_t wb = cc.x >> 16;
                             const uint32_t* wa = reinterpret_cast<const uint32_t*>(g0 + wb);
                             const uint32_t* wv = reinterpret_cast<const uint32_t*>(g1 + wb);
-                            const uint32_t a0 = __ldg(wa), a1 = __ldg(wa + 1), b0 = __ldg(wv), b1 = __ldg(wv + 1);
+                            if (SRC == SRC_WINDOWS || e2 == 0) {
+                                a0 = __ldg(wa), a1 = __ldg(wa + 1);
+                                b0 = __ldg(wv), b1 = __ldg(wv + 1);
+                            }
 #pragma unroll
                             for (int j = 0; j < 2; ++j) {
                                 const uint32_t sel = j ? cc.z : cc.x, wts = j ? cc.w : cc.y;
@@ -365,6 +372,8 @@ __global__ void __launch_bounds__(Cfg<S, TPC>::NT, Cfg<S, TPC>::minb(TABLE)) lbp
             resample(std::integral_constant<int, SRC_CROPS>{});
         else if (a.affine)
             resample(std::integral_constant<int, SRC_AFFINE>{});
+        else if (pair_win && r.w <= S)
+            resample(std::integral_constant<int, SRC_GROUP>{});
         else if (pair_win)
             resample(std::integral_constant<int, SRC_WINDOWS>{});
         else

@@ -396,3 +396,21 @@ def test_few_faces_give_the_bits_of_a_batch(B, ctx, orc, crop, dt, flags):
         assert torch.equal(f, fb[:k]) and torch.equal(x, whole) and torch.equal(q, qb[:k])
     want = orc.features_batch(grey, depth, r[:40], crop, flags=flags)
     assert (host_u16(fb[:40]) == want).all()
+
+
+@pytest.mark.parametrize("crop", [32, 64, 96, 128])
+@pytest.mark.parametrize("W", [8, 60, 200])
+def test_rects_around_the_crop_width(B, ctx, orc, crop, W):
+    """Rects up to the crop's width read the grey taps of four pixels from one window, wider ones those
+    of two: widths on both sides of the line, partly outside the frame, down to the narrowest frame."""
+    rng = synth.rng_for(crop + W)
+    H = 50
+    grey = rng.integers(0, 256, (2, H, W)).astype(np.uint8)
+    depth = rng.integers(800, 1200, (2, H, W)).astype(np.uint16)
+    widths = [1, 2, crop // 2, crop - 1, crop, crop + 1, 2 * crop, 2 * crop + 1]
+    r = np.zeros(4 * len(widths), orc.RECT_DTYPE)
+    r["frame"], r["w"] = rng.integers(0, 2, len(r)), np.repeat(widths, 4)
+    r["h"], r["y"] = rng.integers(1, 60, len(r)), rng.integers(-20, 40, len(r))
+    r["x"] = np.tile([-3, 0, W // 2, W - 2], len(widths)) + rng.integers(0, 4, len(r))
+    f, _, _ = B.lbp_fused_features(ctx, dev_u8(grey), dev_u16(depth), B.rects_tensor(r), crop=crop)
+    assert (host_u16(f) == orc.features_batch(grey, depth, r, crop)).all()
