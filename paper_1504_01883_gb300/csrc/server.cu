@@ -406,11 +406,11 @@ int rgbd_server_create(const rgbd_svm* model, const rgbd_server_config* cfg, rgb
         return rc;
     }
     if (e == cudaSuccess && model->kernel == RGBD_KERNEL_RBF) {
-        // the scoring workspace of the largest batch of either scoring path (at most 128 rows
-        // split over K, more rows by SV tiles), reserved now: growing it during serving would
+        // the largest scoring workspace of any batch size (a few rows, split over K, take more than
+        // some larger batches by tiles), reserved now: growing it during serving would
         // put a cudaFree / cudaMalloc pair, which wait for the device, in a frame's latency
         size_t ws = 0;
-        for (int nq : {std::min(128, c.max_batch_faces), c.max_batch_faces})
+        for (int nq = 1; nq <= c.max_batch_faces; ++nq)
             ws = std::max(ws, model->dtype == RGBD_DT_F32 ? rgbd::score_rbf_f32_bytes(s->ctx, model, nq)
                                                            : rgbd::score_rbf_tc_bytes(s->ctx, model, nq));
         rc = ws ? rgbd::ensure_workspace(s->ctx, ws, nullptr) : RGBD_OK;
