@@ -12,7 +12,8 @@
 //   rbf_f32_kernel     tiles of the fp32 product over (rows, SVs), E in the epilogue, then
 //                      E x a^T per tile or slice of tiles.
 // reduce_scores_kernel adds the splits, asum and the bias, and takes the argmax
-// (reduce_scores_hoisted_kernel: the same with the row-independent sums shared by a block).
+// (reduce_scores_wide_kernel, reduce_scores_hoisted_kernel: the tensor-core splits, the row-independent
+// sums shared by a block; a thread per output, and a warp per row for more than 1024 rows).
 #include <algorithm>
 
 #include "f32_tile.cuh"
