@@ -414,3 +414,19 @@ def test_rects_around_the_crop_width(B, ctx, orc, crop, W):
     r["x"] = np.tile([-3, 0, W // 2, W - 2], len(widths)) + rng.integers(0, 4, len(r))
     f, _, _ = B.lbp_fused_features(ctx, dev_u8(grey), dev_u16(depth), B.rects_tensor(r), crop=crop)
     assert (host_u16(f) == orc.features_batch(grey, depth, r, crop)).all()
+
+
+@pytest.mark.parametrize("mask_mm", [1, 2, 150, 32768, 65535, 65536, 1 << 20])
+@pytest.mark.parametrize("centre", [1, 140, 1000, 40000, 65535])
+def test_depth_mask_at_the_ends_of_its_range(B, ctx, orc, mask_mm, centre):
+    """The mask takes two depths at a time modulo 2^16: medians and windows at both ends of the range,
+    holes, and depths one inside and one outside the window."""
+    rng = synth.rng_for(centre + mask_mm % 1009)
+    near = np.array([centre] * 8 + [centre + k for k in (-mask_mm, 1 - mask_mm, mask_mm - 1, mask_mm, -1, 1)])
+    pool = np.concatenate([near, [0, 0, 1, 2, 65534, 65535]])
+    depth = rng.choice(pool[(pool >= 0) & (pool <= 65535)], (6, 64, 64)).astype(np.uint16)
+    depth[5] = 0
+    grey = rng.integers(0, 256, (6, 64, 64)).astype(np.uint8)
+    for flags in (0, 3):
+        f, _, _ = B.lbp_fused_features(ctx, dev_u8(grey), dev_u16(depth), crop=64, mask_mm=mask_mm, flags=flags)
+        assert (host_u16(f) == orc.features_batch(grey, depth, None, 64, mask_mm=mask_mm, flags=flags)).all()
