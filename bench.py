@@ -45,7 +45,7 @@ X_ELEM = {"f32": 4, "tf32": 4, "bf16": 2, "fp8": 1, "bf16x3": 4}
 # digest covers the source with comments and blank space removed, so only a code change (or a
 # changed layout) reports null.
 MEASURED_TRAFFIC = {
-    "k1": ("lbp.cu", "8b6d698b2a2a9ad1", "shape2/ctas2/bf16", 189_117_440 + 194_996_736),
+    "k1": ("lbp.cu", "2aac33549a94894c", "shape2/ctas2/bf16", 189_068_032 + 194_797_568),
     "k2": ("svm_tc.cu", "de114925748423c5", "splits4/pair/bf16", 616_717_312 + 3_664_128),
 }
 
