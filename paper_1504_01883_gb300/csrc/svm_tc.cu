@@ -1072,6 +1072,12 @@ __global__ void __launch_bounds__(SK_WARPS * 32, 1)
 // classes, from the end of the kernel before: 17 us with 8 warps, a class at a time and block-wide
 // passes for r and F (5.8 us the classes, 5.3 us the combine), 10 us now.
 // d2_min: least d^2 (0 for the exact fp32 path, -infinity for the tensor-core paths).
+// Any gamma: where the mean lies more than kRefReach / gamma above the tile's least distance, r is that
+// far above it, and the combine's reference r* (tile 0's r) is held as near to the least r.  So neither
+// F nor delta exceeds e^20, their product stays far inside fp32, and exp(-gamma r*) is zero only where
+// every kernel value is below e^-64: a row that is itself a support vector of a widely spread model
+// (gamma x mean d^2 above 88) would otherwise be 0 x infinity.  Nearer means are taken as they are.
+constexpr float kRefReach = 20.f;
 constexpr int SKE_ROWS = 16;
 constexpr int SKE_THREADS = 32 * SKE_ROWS;
 size_t ske_smem(int C) { return sizeof(float) * (size_t)((C + 3) / 4 * 4 + SKE_ROWS) * BN; }
@@ -1088,6 +1094,7 @@ __global__ void __launch_bounds__(SKE_THREADS) rbf_splitk_epilogue_kernel(
     const float4* F4 = reinterpret_cast<const float4*>(F);
     const float4* A4 = reinterpret_cast<const float4*>(A);
     __shared__ int last;
+    __shared__ float r_star[SKE_ROWS];
     constexpr int W4 = BN / 4, PER = BN / 32;  // 4-column groups of a tile, columns per lane
     const int tile = blockIdx.x, k0 = blockIdx.y * SKE_ROWS;
     const int rows = min(SKE_ROWS, n - k0), valid = min(BN, n_sv - tile * BN);
@@ -1118,14 +1125,20 @@ __global__ void __launch_bounds__(SKE_THREADS) rbf_splitk_epilogue_kernel(
 #pragma unroll
             for (int j = 0; j < PER; ++j) g[j] += __ldcg(gp + (size_t)z * n_pad * n + 32 * j);
         }
-        float sum = 0.f;
+        float sum = 0.f, least = INFINITY;
 #pragma unroll
         for (int j = 0; j < PER; ++j) {
             g[j] = fmaxf(xs + sv[j] - 2.f * gscale * g[j], d2_min);
-            if (lane + 32 * j < valid) sum += g[j];
+            if (lane + 32 * j < valid) {
+                sum += g[j];
+                least = fminf(least, g[j]);
+            }
         }
-        for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
-        const float r = sum / (float)max(valid, 1);
+        for (int off = 16; off > 0; off >>= 1) {
+            sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
+            least = fminf(least, __shfl_xor_sync(0xFFFFFFFFu, least, off));
+        }
+        const float r = fminf(sum / (float)max(valid, 1), least + kRefReach / gamma);
 #pragma unroll
         for (int j = 0; j < PER; ++j)
             F[warp * BN + lane + 32 * j] = lane + 32 * j < valid ? expm1_near0(-gamma * (g[j] - r)) : 0.f;
@@ -1191,10 +1204,22 @@ __global__ void __launch_bounds__(SKE_THREADS) rbf_splitk_epilogue_kernel(
     float* s_as = A;                // [nt][C]
 #pragma unroll 4
     for (int i = tid; i < nt * C; i += SKE_THREADS) s_as[i] = __ldcg(asum_tile + (size_t)(i / C) * C_pad + i % C);
+    if (warp < rows) {  // a warp = one row: its r* and every tile's delta
+        float* del = s_del + warp * nt;
+        float least = INFINITY;
+#pragma unroll 4
+        for (int t = lane; t < nt; t += 32) {
+            const float rt = __ldcg(ref + (size_t)t * n + k0 + warp);
+            del[t] = rt;
+            least = fminf(least, rt);
+        }
+        for (int off = 16; off > 0; off >>= 1) least = fminf(least, __shfl_xor_sync(0xFFFFFFFFu, least, off));
+        __syncwarp();
+        const float rs = fminf(del[0], least + kRefReach / gamma);
+        __syncwarp();
 #pragma unroll 1
-    for (int idx = tid; idx < rows * nt; idx += SKE_THREADS) {
-        const int k = idx / nt, t = idx - k * nt;
-        s_del[idx] = t == 0 ? 0.f : expm1f(-gamma * (__ldcg(ref + (size_t)t * n + k0 + k) - __ldcg(ref + k0 + k)));
+        for (int t = lane; t < nt; t += 32) del[t] = del[t] == rs ? 0.f : expm1f(-gamma * (del[t] - rs));
+        if (lane == 0) r_star[warp] = rs;
     }
     __syncthreads();
     // thread = (row, class): the tiles' partial sums 16 at a time, added in tile order
@@ -1203,7 +1228,7 @@ __global__ void __launch_bounds__(SKE_THREADS) rbf_splitk_epilogue_kernel(
     for (int i = tid; i < rows * C; i += SKE_THREADS) {
         const int k = i / C, c = i - k * C;
         const float* pd = part + (size_t)(k0 + k) * C_pad + c;
-        const float r0 = __ldcg(ref + k0 + k), as = __ldg(asum + c), bs = __ldg(bias + c);
+        const float as = __ldg(asum + c), bs = __ldg(bias + c);
         float acc = 0.f;
 #pragma unroll 1
         for (int t0 = 0; t0 < nt; t0 += 16) {
@@ -1214,7 +1239,7 @@ __global__ void __launch_bounds__(SKE_THREADS) rbf_splitk_epilogue_kernel(
             for (int j = 0; j < 16; ++j)
                 if (t0 + j < nt) acc += d[j] + s_del[k * nt + t0 + j] * (s_as[(t0 + j) * C + c] + d[j]);
         }
-        const float sc = expf(-gamma * r0) * (as + acc) + bs;
+        const float sc = expf(-gamma * r_star[k]) * (as + acc) + bs;
         scores[(size_t)(k0 + k) * C + c] = sc;
         if (sc_fit) s_sc[i] = sc;
     }

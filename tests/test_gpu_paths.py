@@ -430,3 +430,49 @@ def test_depth_mask_at_the_ends_of_its_range(B, ctx, orc, mask_mm, centre):
     for flags in (0, 3):
         f, _, _ = B.lbp_fused_features(ctx, dev_u8(grey), dev_u16(depth), crop=64, mask_mm=mask_mm, flags=flags)
         assert (host_u16(f) == orc.features_batch(grey, depth, None, 64, mask_mm=mask_mm, flags=flags)).all()
+
+
+@pytest.mark.parametrize("gamma", [0.3, 5.0, 20.0, 200.0])
+@pytest.mark.parametrize("dt,n", [("f32", 1), ("f32", 3), ("f32", 8), ("bf16", 7), ("bf16", 40)])
+def test_few_row_scores_at_any_gamma(B, ctx, orc, gamma, dt, n):
+    """Scores of few rows where the distances of a model spread far over 1 / gamma: rows that are support
+    vectors of the first and of the last SV tile, rows near no support vector, tiles 250 apart in mean
+    distance.  Against fp64; exact fp32 rows also against the same rows in a batch of nine, which another
+    kernel scores."""
+    rng = synth.rng_for(int(10 * gamma) + n)
+    cells, n_sv, C = 256, 700, 6
+    SV = synth.poisson_counts(rng, n_sv, cells * 59)
+    one = np.zeros((257, cells, 59), np.uint16)  # rows with one bin per cell: far from all others
+    np.put_along_axis(one, rng.integers(0, 59, (257, cells, 1)), 64, 2)
+    SV[:256] = one[:256].reshape(256, -1)
+    rows = max(n, 9)
+    X = synth.poisson_counts(rng, rows, cells * 59)
+    X[0], X[1], X[2] = SV[600], SV[3], one[256].reshape(-1)
+    a = rng.normal(0, 1, (C, n_sv)).astype(np.float32)
+    b = rng.normal(0, 0.01, C).astype(np.float32)
+    model = B.svm_train_data_pack(ctx, dev_u16(SV), dev_f32(a), dev_f32(b), gamma=gamma, dtype=dt)
+    x, q = B.lbp_normalize_features(ctx, dev_u16(X[:n]), dt)
+    s, lab = B.svm_score(ctx, model, x, q)
+    s, lab = s.cpu().numpy(), lab.cpu().numpy()
+    assert ctx.status() == 0
+
+    def held(counts):  # the values a row holds, in fp64
+        v = orc.normalize_f64(counts)
+        return v if dt == "f32" else torch.from_numpy(v.astype(np.float32)).bfloat16().double().numpy()
+
+    x64, sv64 = held(X), held(SV)
+    xx, ss, g = (x64 ** 2).sum(1)[:, None], (sv64 ** 2).sum(1)[None, :], x64 @ sv64.T
+    K = np.exp(-gamma * np.maximum(xx + ss - 2 * g, 0))
+    ref = K @ a.astype(np.float64).T + b
+    # a distance is off by the fp32 rounding of two norms and a product: chains of at most 80 additions
+    # (tensor cores: 15104 products in any order, taken as 1024), a kernel value by gamma times that,
+    # the sums by the path's 1e-5 of the score's scale and of the largest kernel value
+    off = gamma * (96 if dt == "f32" else 1024) * 2.0 ** -24 * (xx + ss + 2 * g)
+    absa = np.abs(a.astype(np.float64)).T
+    tol = (K * np.expm1(np.minimum(off, 50))) @ absa + 1e-5 * (K @ absa + np.abs(b)) + 1e-6 * K.max(1, keepdims=True) * absa.sum(0)
+    assert (np.abs(s - ref[:n]) <= tol[:n]).all()
+    assert (lab == s.argmax(1)).all()
+    if dt == "f32":
+        x9, q9 = B.lbp_normalize_features(ctx, dev_u16(X), dt)
+        s9, _ = B.svm_score(ctx, model, x9, q9)
+        assert (np.abs(s - s9.cpu().numpy()[:n]) <= 2 * tol[:n] + 1e-6 * absa.sum(0)).all()
