@@ -520,6 +520,14 @@ int rgbd_debug_expm1(const float* z, float* out, int n, void* stream);
  * Errors: RGBD_ERR_ARG. */
 int rgbd_debug_wait_timeout(rgbd_ctx* ctx, uint64_t limit_ns, int* result, void* stream);
 
+/* rgbd_debug_drop_handover -- for a test of the failure path of the fp32 products that are spread over
+ * the SMs in stages (svm_score of fp32 models, svm_train_rbf): CTA `cta` of the context's following calls
+ * does not say that its part of a shared tile is there, and the CTA that waits for it gives up after
+ * limit_ns (1 us .. 100 ms).  RGBD_STATUS_WAIT_TIMEOUT is set; the rows of that tile get zero scores and
+ * label 0, a training call zero coefficients, biases and steps.  cta -1 restores the normal state.
+ * Errors: RGBD_ERR_ARG. */
+int rgbd_debug_drop_handover(rgbd_ctx* ctx, int cta, uint64_t limit_ns);
+
 #ifdef __cplusplus
 }
 #endif

@@ -82,6 +82,7 @@ def lib():
             "rgbd_track_nearest": [P, P, I, P, I, P, P],
             "rgbd_debug_expm1": [P, P, I, P],
             "rgbd_debug_wait_timeout": [P, ctypes.c_uint64, P, P],
+            "rgbd_debug_drop_handover": [P, I, ctypes.c_uint64],
             "rgbd_face_roi": [P, P, I, I, I, P, P, I, P, P],
             "svm_train_rbf": [P, P, P, I, I, P, I, F, F, F, I, P, P, P, P],
             "rgbd_track_streams": [P, P, P, P, I, I, I, P, P, P, I, P, P, P],
@@ -340,6 +341,11 @@ def rgbd_debug_wait_timeout(ctx, limit_ns, stream=None):
     res = torch.full((1,), -1, dtype=torch.int32, device=torch.device("cuda", ctx.device))
     _check(lib().rgbd_debug_wait_timeout(ctx.handle, int(limit_ns), _p(res), _stream(stream)))
     return res
+
+
+def rgbd_debug_drop_handover(ctx, cta, limit_ns=2_000_000):
+    """Lets CTA `cta` of the spread fp32 products keep its part of a shared tile back (-1: none)."""
+    _check(lib().rgbd_debug_drop_handover(ctx.handle, int(cta), int(limit_ns)))
 
 
 def rgbd_debug_expm1(z, stream=None):

@@ -164,6 +164,15 @@ int rgbd_ctx_set_tuning(rgbd_ctx* ctx, int key, int value) {
     }
 }
 
+int rgbd_debug_drop_handover(rgbd_ctx* ctx, int cta, uint64_t limit_ns) {
+    CHECK_ARG(ctx != nullptr, "rgbd_debug_drop_handover: ctx is NULL");
+    CHECK_ARG(cta >= -1 && (cta < 0 || (limit_ns >= 1000 && limit_ns <= 100000000ull)),
+              "rgbd_debug_drop_handover: CTA %d, limit %llu ns (1 us .. 100 ms)", cta, (unsigned long long)limit_ns);
+    ctx->drop_handover = cta;
+    ctx->handover_ns = cta < 0 ? rgbd_ctx().handover_ns : limit_ns;
+    return RGBD_OK;
+}
+
 int rgbd_crop_affine(rgbd_ctx* ctx, const uint8_t* grey, const uint16_t* depth, int n_frames, int H,
                      int W, const rgbd_rect* rects, const int32_t* affine_q16, int n_rects,
                      int out_h, int out_w, uint8_t* out_grey, uint16_t* out_depth, void* stream) {

@@ -154,13 +154,19 @@ struct F32Rows {
 // then its whole tiles, and last the end of its first tile, whose beginning the CTA before computed
 // first (taken up by fetch(tile index, t), thread by thread what stash left): as a
 // range is at least one tile long, nobody waits for work that has not been done by then.  (A CTA
-// waits only for one of a lower index, which the hardware starts before it; the wait is bounded
-// all the same.)  Without the split 168 tiles on 152 SMs take the time of two.
-// ready: a word per CTA, zero before the launch.
-template <class Tile, bool VEC, class Rows, class Finish, class Stash, class Fetch>
-__device__ __forceinline__ void f32_ordered_tiles(long long tiles, int K, uint32_t* ready, uint32_t* status,
+// waits only for one of a lower index, which the hardware starts before it; the wait is bounded all the
+// same, and a tile whose wait runs out is not finished: fail(tile index), by one thread, lets the outputs
+// that hang on it be zeroed.)  Without the split 168 tiles on 152 SMs take the time of two.
+struct F32HandOver {
+    uint32_t* ready;    // a word per CTA, zero before the launch
+    uint32_t* status;   // RGBD_STATUS_WAIT_TIMEOUT when a wait runs out
+    uint64_t limit_ns;
+    int drop;           // a CTA that hands on nothing (for tests), or -1
+};
+template <class Tile, bool VEC, class Rows, class Finish, class Stash, class Fetch, class Fail>
+__device__ __forceinline__ void f32_ordered_tiles(long long tiles, int K, const F32HandOver& ho,
                                                   typename Tile::Smem& sm, Rows rows, Finish finish, Stash stash,
-                                                  Fetch fetch) {
+                                                  Fetch fetch, Fail fail) {
     __shared__ int gave_up;
     const int stages = (K + Tile::KB - 1) / Tile::KB, tid = threadIdx.x;
     const long long U = tiles * stages;
@@ -175,7 +181,8 @@ __device__ __forceinline__ void f32_ordered_tiles(long long tiles, int K, uint32
         stash(last, t);
         __threadfence();
         __syncthreads();
-        if (tid == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(ready + blockIdx.x), "r"(1u) : "memory");
+        if (tid == 0 && (int)blockIdx.x != ho.drop)
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(ho.ready + blockIdx.x), "r"(1u) : "memory");
     }
     for (long long i = first + (k0 > 0); i < last; ++i) {
         const F32Rows r = rows(i);
@@ -190,13 +197,17 @@ __device__ __forceinline__ void f32_ordered_tiles(long long tiles, int K, uint32
             uint32_t ok = 0;
             int failed = 0;
             for (;;) {
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(ok) : "l"(ready + blockIdx.x - 1) : "memory");
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];"
+                             : "=r"(ok)
+                             : "l"(ho.ready + blockIdx.x - 1)
+                             : "memory");
                 if (ok) break;
                 asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
                 if (since == 0) since = now;
-                if (now - since > 1000000000ull) {  // 1 s: far above a tile's time
+                if (now - since > ho.limit_ns) {
                     failed = 1;
-                    atomicOr(status, RGBD_STATUS_WAIT_TIMEOUT);
+                    atomicOr(ho.status, RGBD_STATUS_WAIT_TIMEOUT);
+                    fail(first);
                     break;
                 }
                 __nanosleep(200);

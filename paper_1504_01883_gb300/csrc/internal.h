@@ -45,6 +45,8 @@ struct rgbd_ctx {
     int tune_tc_pairing = 0;       // CTA pairing: 0 = auto, 2 = none, 3 = 2-CTA MMA pairs
     int tune_lbp_shape = 0;        // fused-kernel threads per cell: 0 = auto, 1 = one, 2 = two, 3 = four
     int tune_tc_splitk = 0;        // K ranges of one-block scoring: 0 = auto, 1 = off, >= 2 forced
+    int drop_handover = -1;        // rgbd_debug_drop_handover: a CTA that hands on nothing ...
+    uint64_t handover_ns = 1000000000ull;  // ... and the limit of the waits for it (1 s: far above a tile's time)
     uint32_t* d_status = nullptr;  // device status word, followed by kFaceCounters face-queue counters
     uint32_t* d_counters = nullptr;
     uint32_t counter_next = 0;     // next counter of the pool (a launch takes one and zeroes it)
@@ -178,10 +180,13 @@ int pack_model_tensor_maps(rgbd_svm* m);
 //   ref   NULL, or [splits][n] per-split reference distances r_s (see svm_tc.cu)
 //   asum_tile  with ref: [n_tiles][C_stride] coefficient sums per SV tile; split s covers
 //              tiles [s * tiles_per_split, (s + 1) * tiles_per_split) clipped to n_tiles
+//   failed  NULL, or a word per block of fail_rows rows (without ref): rows of a block whose word is set
+//              get zero scores and label 0
 int launch_reduce_scores(const float* part, const float* ref, int splits, int n, int C,
                          int C_stride, const float* asum, const float* asum_tile,
                          int tiles_per_split, int n_tiles, const float* bias, float gamma,
-                         float* scores, int32_t* labels, cudaStream_t s);
+                         float* scores, int32_t* labels, cudaStream_t s, const uint32_t* failed = nullptr,
+                         int fail_rows = 1);
 
 // TMA descriptor encoding through the driver entry point (no libcuda link).
 int encode_tmap_2d(CUtensorMap* map, CUtensorMapDataType dt, const void* base, uint64_t inner,

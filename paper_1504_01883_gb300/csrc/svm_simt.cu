@@ -229,8 +229,7 @@ struct F32Score {
     float* part;      // [slices][n][C]
     // ORDERED: chains and flags handed from CTA to CTA
     uint64_t* stash;  // [CTA][32][threads]
-    uint32_t* ready;
-    uint32_t* status;
+    uint32_t* failed;  // [row tile]
 };
 
 template <int BM>
@@ -295,7 +294,7 @@ __device__ __forceinline__ void f32_score_tile(const F32Score& p, const F32Tile<
 // ORDERED: every SV tile is a slice of its own, and the tiles are spread evenly over one CTA per
 // SM.  Otherwise CTA (row tile, slice) walks the SV tiles of its slice.
 template <int BM, bool ORDERED>
-__global__ void __launch_bounds__(F32Tile<BM, BM>::NT, 1) rbf_f32_kernel(const F32Score p) {
+__global__ void __launch_bounds__(F32Tile<BM, BM>::NT, 1) rbf_f32_kernel(const F32Score p, const F32HandOver ho) {
     using Tile = F32Tile<BM, BM>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     auto& sm = *reinterpret_cast<F32ScoreSmem<BM>*>(smem_raw);
@@ -304,7 +303,7 @@ __global__ void __launch_bounds__(F32Tile<BM, BM>::NT, 1) rbf_f32_kernel(const F
     };
     if (ORDERED) {
         f32_ordered_tiles<Tile, true>(
-            (long long)p.mt * p.nt, p.k_pad, p.ready, p.status, sm.stage,
+            (long long)p.mt * p.nt, p.k_pad, ho, sm.stage,
             [&](long long i) { return rows((int)(i % p.mt), (int)(i / p.mt)); },
             [&](long long i, const Tile& t) {
                 f32_score_tile<BM>(p, t, (int)(i % p.mt), (int)(i / p.mt), (int)(i / p.mt), false, sm);
@@ -320,7 +319,8 @@ __global__ void __launch_bounds__(F32Tile<BM, BM>::NT, 1) rbf_f32_kernel(const F
 #pragma unroll
                 for (int i = 0; i < 32; ++i)
                     t.acc[i >> 2][i & 3] = __ldcg(reinterpret_cast<const unsigned long long*>(in + i * Tile::NT));
-            });
+            },
+            [&](long long i) { p.failed[i % p.mt] = 1u; });
     } else {
         const int mi = blockIdx.x, slice = blockIdx.y, t0 = slice * p.tps, t1 = min(p.nt, t0 + p.tps);
         for (int ni = t0; ni < t1; ++ni) {
@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(F32Tile<BM, BM>::NT, 1) rbf_f32_kernel(const F
 struct F32Plan {
     int bm, mt, nt, slices, tps;
     bool ordered;
-    size_t off_stash, off_ready, bytes;
+    size_t off_stash, off_ready, bytes;  // (at off_ready: a word per CTA, then one per row tile)
 };
 
 F32Plan plan_f32(const rgbd_ctx* ctx, const rgbd_svm* m, int n) {
@@ -369,17 +369,17 @@ F32Plan plan_f32(const rgbd_ctx* ctx, const rgbd_svm* m, int n) {
     p.slices = (p.nt + p.tps - 1) / p.tps;
     p.off_stash = (sizeof(float) * (size_t)p.slices * n * m->C + 255) & ~size_t(255);
     p.off_ready = p.off_stash + (p.ordered ? sizeof(uint64_t) * 32 * F32Tile<128, 128>::NT * (size_t)sms : 0);
-    p.bytes = p.off_ready + (p.ordered ? sizeof(uint32_t) * (size_t)sms : 0);
+    p.bytes = p.off_ready + (p.ordered ? sizeof(uint32_t) * ((size_t)sms + p.mt) : 0);
     return p;
 }
 
 template <int BM, bool ORDERED>
-cudaError_t launch_f32(const F32Score& p, dim3 grid, cudaStream_t s) {
+cudaError_t launch_f32(const F32Score& p, const F32HandOver& ho, dim3 grid, cudaStream_t s) {
     const size_t smem = sizeof(F32ScoreSmem<BM>);
     const cudaError_t e =
         cudaFuncSetAttribute(rbf_f32_kernel<BM, ORDERED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    rbf_f32_kernel<BM, ORDERED><<<grid, F32Tile<BM, BM>::NT, smem, s>>>(p);
+    rbf_f32_kernel<BM, ORDERED><<<grid, F32Tile<BM, BM>::NT, smem, s>>>(p, ho);
     return cudaGetLastError();
 }
 
@@ -395,10 +395,16 @@ __global__ void reduce_scores_kernel(const float* __restrict__ part, const float
                                      int splits, int n, int C, int C_stride, const float* __restrict__ asum,
                                      const float* __restrict__ asum_tile, int tps, int nt,
                                      const float* __restrict__ bias, float gamma, float* __restrict__ scores,
-                                     int32_t* __restrict__ labels) {
+                                     int32_t* __restrict__ labels, const uint32_t* __restrict__ failed,
+                                     int fail_rows) {
     const int lane = threadIdx.x & 31;
     const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= n) return;
+    if (failed && failed[row / fail_rows]) {
+        for (int c = lane; c < C; c += 32) scores[(size_t)row * C + c] = 0.f;
+        if (labels && lane == 0) labels[row] = 0;
+        return;
+    }
     float best = -INFINITY;
     int bi = 0x7FFFFFFF;
     const float rstar = ref ? ref[row] : 0.f;
@@ -584,7 +590,8 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_scores_wide_kernel(
 
 int launch_reduce_scores(const float* part, const float* ref, int splits, int n, int C, int C_stride,
                          const float* asum, const float* asum_tile, int tiles_per_split, int n_tiles,
-                         const float* bias, float gamma, float* scores, int32_t* labels, cudaStream_t s) {
+                         const float* bias, float gamma, float* scores, int32_t* labels, cudaStream_t s,
+                         const uint32_t* failed, int fail_rows) {
     // Up to 1024 rows (many splits each): a thread per output.  More rows have few splits and enough
     // warps at a row each (4096 rows, 4 splits, 64 classes: 7 us, against 9 a thread per output).
     const int rows = std::max(1, kReduceThreads / C);
@@ -614,7 +621,7 @@ int launch_reduce_scores(const float* part, const float* ref, int splits, int n,
         const int rows_per_block = 8;
         reduce_scores_kernel<<<(n + rows_per_block - 1) / rows_per_block, 32 * rows_per_block, 0, s>>>(
             part, ref, splits, n, C, C_stride, asum, asum_tile, tiles_per_split, n_tiles, bias, gamma, scores,
-            labels);
+            labels, failed, fail_rows);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return cuda_error(e, "svm_score: reduce launch");
@@ -722,19 +729,21 @@ int score_rbf_f32(rgbd_ctx* ctx, const rgbd_svm* m, const float* x, const float*
     p.x = x, p.xsq = xsq, p.n = n, p.k_pad = m->k_pad, p.sv = (const float*)m->sv, p.svsq = m->sv_sq;
     p.n_sv = m->n_sv, p.n_pad = m->n_pad, p.coef = m->coef, p.C = m->C, p.gamma = m->gamma;
     p.mt = pl.mt, p.nt = pl.nt, p.tps = pl.tps, p.part = (float*)ws;
-    p.stash = (uint64_t*)(ws + pl.off_stash), p.ready = (uint32_t*)(ws + pl.off_ready), p.status = ctx->d_status;
+    p.stash = (uint64_t*)(ws + pl.off_stash);
+    const int grid = ctx->props.sm_count;
+    const F32HandOver ho = {(uint32_t*)(ws + pl.off_ready), ctx->d_status, ctx->handover_ns, ctx->drop_handover};
+    p.failed = ho.ready + grid;
     if (pl.ordered) {
-        const int grid = ctx->props.sm_count;
-        e = cudaMemsetAsync(p.ready, 0, sizeof(uint32_t) * (size_t)grid, s);
+        e = cudaMemsetAsync(ho.ready, 0, sizeof(uint32_t) * ((size_t)grid + pl.mt), s);
         if (e != cudaSuccess) return cuda_error(e, "svm_score: tile hand-over reset");
-        e = launch_f32<128, true>(p, dim3((unsigned)grid), s);
+        e = launch_f32<128, true>(p, ho, dim3((unsigned)grid), s);
     } else {
-        const dim3 grid((unsigned)pl.mt, (unsigned)pl.slices);
-        e = pl.bm == 128 ? launch_f32<128, false>(p, grid, s) : launch_f32<64, false>(p, grid, s);
+        const dim3 tiles((unsigned)pl.mt, (unsigned)pl.slices);
+        e = pl.bm == 128 ? launch_f32<128, false>(p, ho, tiles, s) : launch_f32<64, false>(p, ho, tiles, s);
     }
     if (e != cudaSuccess) return cuda_error(e, "svm_score: rbf fp32 launch");
     return launch_reduce_scores(p.part, nullptr, pl.slices, n, m->C, m->C, m->asum, nullptr, 0, 0, m->bias, m->gamma,
-                                scores, labels, s);
+                                scores, labels, s, pl.ordered ? p.failed : nullptr, pl.bm);
 }
 
 }  // namespace rgbd

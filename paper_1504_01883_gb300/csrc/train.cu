@@ -35,8 +35,8 @@ template <int BM, bool VEC, bool ORDERED>
 __global__ void __launch_bounds__(F32Tile<BM, BM>::NT, 1) kernel_matrix_kernel(const float* __restrict__ x,
                                                                           const float* __restrict__ xsq, int n,
                                                                           int k_pad, float gamma, long long tiles,
-                                                                          float* K, uint32_t* ready,
-                                                                          uint32_t* status) {
+                                                                          float* K, F32HandOver ho, int32_t* failed,
+                                                                          int n_classes) {
     using Tile = F32Tile<BM, BM>;
     extern __shared__ __align__(16) unsigned char km_smem[];
     auto& sm = *reinterpret_cast<typename Tile::Smem*>(km_smem);
@@ -95,7 +95,11 @@ __global__ void __launch_bounds__(F32Tile<BM, BM>::NT, 1) kernel_matrix_kernel(c
                     t.put(i, p, lo ? __ldcg(lo) : 0.f, hi ? __ldcg(hi) : 0.f);
                 }
         };
-        f32_ordered_tiles<Tile, VEC>(tiles, k_pad, ready, status, sm, rows, finish, stash, fetch);
+        // every class hangs on every tile
+        auto fail = [&](long long) {
+            for (int c = 0; c < n_classes; ++c) failed[c] = 1;
+        };
+        f32_ordered_tiles<Tile, VEC>(tiles, k_pad, ho, sm, rows, finish, stash, fetch, fail);
     } else {
         const F32Rows r = rows(blockIdx.x);
         Tile t;
@@ -128,11 +132,12 @@ struct SmoPick {
     int y;
 };
 
+// marked: iters[c] says whether K is incomplete (a tile's hand-over failed); the class gets zeros then.
 template <int T, int EPT>
 __global__ void __launch_bounds__(T, 1) smo_kernel(const float* __restrict__ K, int n,
                                                    const int32_t* __restrict__ labels, float cost, float eps,
                                                    int max_iter, float* __restrict__ coef, float* __restrict__ bias,
-                                                   int32_t* __restrict__ iters) {
+                                                   int32_t* iters, bool marked) {
     constexpr int NW = T / 32;
     constexpr uint32_t NONE = 0xFFFFFFFFu, FULL = 0xFFFFFFFFu;
     extern __shared__ float alpha[];  // [n], each entry touched by the thread that owns the row
@@ -140,6 +145,12 @@ __global__ void __launch_bounds__(T, 1) smo_kernel(const float* __restrict__ K, 
     __shared__ float sums[32];
     __shared__ int counts[32];
     const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (marked && iters[c] != 0) {
+        __syncthreads();  // everyone has read the mark
+        for (int t = tid; t < n; t += T) coef[(size_t)c * n + t] = 0.f;
+        if (tid == 0) bias[c] = 0.f, iters[c] = 0;
+        return;
+    }
     float u[EPT];
     uint32_t ypos = 0, up = 0, low = 0;  // a bit per row: y > 0, may move up, may move down
 #pragma unroll
@@ -287,21 +298,22 @@ __global__ void __launch_bounds__(T, 1) smo_kernel(const float* __restrict__ K, 
 
 template <int BM, bool VEC, bool ORDERED>
 cudaError_t launch_kernel_matrix(int grid, const float* x, const float* xsq, int n, int k_pad, float gamma,
-                                 long long tiles, float* K, uint32_t* ready, uint32_t* status, cudaStream_t s) {
+                                 long long tiles, float* K, const F32HandOver& ho, int32_t* failed, int n_classes,
+                                 cudaStream_t s) {
     const size_t smem = sizeof(typename F32Tile<BM, BM>::Smem);
     kernel_matrix_kernel<BM, VEC, ORDERED>
-        <<<grid, F32Tile<BM, BM>::NT, smem, s>>>(x, xsq, n, k_pad, gamma, tiles, K, ready, status);
+        <<<grid, F32Tile<BM, BM>::NT, smem, s>>>(x, xsq, n, k_pad, gamma, tiles, K, ho, failed, n_classes);
     return cudaGetLastError();
 }
 
 template <int T, int EPT>
 cudaError_t launch_smo(const float* K, int n, const int32_t* labels, int n_classes, float cost, float eps,
-                       int max_iter, float* coef, float* bias, int32_t* iters, cudaStream_t s) {
+                       int max_iter, float* coef, float* bias, int32_t* iters, bool marked, cudaStream_t s) {
     const size_t smem = sizeof(float) * (size_t)n;
     const cudaError_t e =
         cudaFuncSetAttribute(smo_kernel<T, EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    smo_kernel<T, EPT><<<n_classes, T, smem, s>>>(K, n, labels, cost, eps, max_iter, coef, bias, iters);
+    smo_kernel<T, EPT><<<n_classes, T, smem, s>>>(K, n, labels, cost, eps, max_iter, coef, bias, iters, marked);
     return cudaGetLastError();
 }
 
@@ -334,24 +346,26 @@ extern "C" int svm_train_rbf(rgbd_ctx* ctx, const float* x, const float* xsq, in
     int rc = ensure_workspace(ctx, sizeof(float) * (size_t)n * n, s);
     if (rc) return rc;
     float* K = (float*)ctx->workspace;
-    // the hand-over flags live in the coefficients until SMO writes them (n >= 2049 when ordered)
-    uint32_t* ready = reinterpret_cast<uint32_t*>(coef);
+    // the hand-over flags live in the coefficients until SMO writes them (n >= 2049 when ordered), the
+    // marks of a failed one in the step counts
+    const F32HandOver ho = {reinterpret_cast<uint32_t*>(coef), ctx->d_status, ctx->handover_ns, ctx->drop_handover};
     const bool vec = k_pad % 16 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
     cudaError_t e = cudaSuccess;
     if (ordered) {
-        e = cudaMemsetAsync(ready, 0, sizeof(uint32_t) * (size_t)grid, s);
+        e = cudaMemsetAsync(ho.ready, 0, sizeof(uint32_t) * (size_t)grid, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(iters, 0, sizeof(int32_t) * (size_t)n_classes, s);
         if (e != cudaSuccess) return cuda_error(e, "svm_train_rbf: tile hand-over reset");
-        e = vec ? launch_kernel_matrix<128, true, true>(grid, x, xsq, n, k_pad, gamma, tiles, K, ready, ctx->d_status, s)
-                : launch_kernel_matrix<128, false, true>(grid, x, xsq, n, k_pad, gamma, tiles, K, ready, ctx->d_status, s);
+        e = vec ? launch_kernel_matrix<128, true, true>(grid, x, xsq, n, k_pad, gamma, tiles, K, ho, iters, n_classes, s)
+                : launch_kernel_matrix<128, false, true>(grid, x, xsq, n, k_pad, gamma, tiles, K, ho, iters, n_classes, s);
     } else {
-        e = vec ? launch_kernel_matrix<64, true, false>(grid, x, xsq, n, k_pad, gamma, tiles, K, ready, ctx->d_status, s)
-                : launch_kernel_matrix<64, false, false>(grid, x, xsq, n, k_pad, gamma, tiles, K, ready, ctx->d_status, s);
+        e = vec ? launch_kernel_matrix<64, true, false>(grid, x, xsq, n, k_pad, gamma, tiles, K, ho, iters, n_classes, s)
+                : launch_kernel_matrix<64, false, false>(grid, x, xsq, n, k_pad, gamma, tiles, K, ho, iters, n_classes, s);
     }
     if (e != cudaSuccess) return cuda_error(e, "svm_train_rbf: kernel matrix launch");
     // Up to 16 rows per thread (they live in registers), and no more warps than that takes: the
     // selection and the barrier cost every warp the same, however few rows it holds (4096 rows:
     // 1.86 ms with 8 warps, 2.48 ms with 32).
-#define RGBD_SMO(TV, EV) launch_smo<TV, EV>(K, n, labels, n_classes, cost, eps, max_iter, coef, bias, iters, s)
+#define RGBD_SMO(TV, EV) launch_smo<TV, EV>(K, n, labels, n_classes, cost, eps, max_iter, coef, bias, iters, ordered, s)
     e = n <= 256    ? RGBD_SMO(256, 1)
         : n <= 1024 ? RGBD_SMO(256, 4)
         : n <= 2048 ? RGBD_SMO(256, 8)

@@ -476,3 +476,61 @@ def test_few_row_scores_at_any_gamma(B, ctx, orc, gamma, dt, n):
         x9, q9 = B.lbp_normalize_features(ctx, dev_u16(X), dt)
         s9, _ = B.svm_score(ctx, model, x9, q9)
         assert (np.abs(s - s9.cpu().numpy()[:n]) <= 2 * tol[:n] + 1e-6 * absa.sum(0)).all()
+
+
+def _waits(tiles, stages, sms):
+    """CTAs whose range of the even split begins inside a tile, and that tile."""
+    starts = [tiles * stages * g // sms for g in range(sms)]
+    return {g: u // stages for g, u in enumerate(starts) if u % stages}
+
+
+def test_fp32_rows_of_a_lost_handover_are_zero(B, ctx, orc):
+    """A CTA waits in vain for the first part of a tile: the status says so, the rows of that tile get zero
+    scores and label 0, the other rows their bits, and the next call is whole again."""
+    rng = synth.rng_for(11)
+    n, n_sv, C, dim = 1300, 2100, 7, 9 * 59
+    X, SV = synth.poisson_counts(rng, n, dim), synth.poisson_counts(rng, n_sv, dim)
+    a = rng.normal(0, 1, (C, n_sv)).astype(np.float32)
+    model = B.svm_train_data_pack(ctx, dev_u16(SV), dev_f32(a), dev_f32(np.ones(C, np.float32)), gamma=0.3, dtype="f32")
+    x, q = B.lbp_normalize_features(ctx, dev_u16(X), "f32")
+    want, labels = B.svm_score(ctx, model, x, q)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    mt, nt = -(-n // 128), -(-n_sv // 128)
+    waits = _waits(mt * nt, model.k_pad // 16, sms)
+    ctx.status(clear=True)
+    for cta in list(waits)[3::40]:
+        B.rgbd_debug_drop_handover(ctx, cta - 1)
+        try:
+            s, lab = B.svm_score(ctx, model, x, q)
+        finally:
+            B.rgbd_debug_drop_handover(ctx, -1)
+        assert ctx.status(clear=True) == B.STATUS_WAIT_TIMEOUT
+        lost = slice(128 * (waits[cta] % mt), min(n, 128 * (waits[cta] % mt + 1)))
+        assert not s[lost].any() and not lab[lost].any()
+        s[lost], lab[lost] = want[lost], labels[lost]
+        assert torch.equal(s, want) and torch.equal(lab, labels)
+    s, lab = B.svm_score(ctx, model, x, q)
+    assert torch.equal(s, want) and torch.equal(lab, labels) and ctx.status() == 0
+
+
+def test_training_of_a_lost_handover_gives_zeros(B, ctx):
+    """The same in the kernel matrix, on which every class hangs."""
+    rng = synth.rng_for(12)
+    n, k_pad = 2100, 48
+    x = rng.normal(0, 0.4, (n, k_pad)).astype(np.float32)
+    q = (x.astype(np.float64) ** 2).sum(1).astype(np.float32)
+    args = (dev_f32(x), dev_f32(q), torch.from_numpy(rng.integers(0, 3, n).astype(np.int32)).cuda(), 3, 1.0, 1.0, 1e-3)
+    want = B.svm_train_rbf(ctx, *args, max_iter=60)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    t = -(-n // 128)
+    cta = list(_waits(t * (t + 1) // 2, k_pad // 16, sms))[20]
+    ctx.status(clear=True)
+    B.rgbd_debug_drop_handover(ctx, cta - 1)
+    try:
+        got = B.svm_train_rbf(ctx, *args, max_iter=60)
+    finally:
+        B.rgbd_debug_drop_handover(ctx, -1)
+    assert ctx.status(clear=True) == B.STATUS_WAIT_TIMEOUT
+    assert not any(t.any() for t in got)
+    assert all(torch.equal(u, v) for u, v in zip(B.svm_train_rbf(ctx, *args, max_iter=60), want))
+    assert ctx.status() == 0
