@@ -171,9 +171,10 @@ int launch_crop_affine(rgbd_ctx* ctx, const uint8_t* grey, const uint16_t* depth
         crop_affine_kernel<<<grid, kCropThreads, 0, s>>>(a);
     } else {
         // crops up to 4096 columns and rows: 41 KB of column taps and 66 KB of row taps at most
+        constexpr size_t most = (sizeof(uint4) + sizeof(uint32_t)) * 2 * 1024 + sizeof(uint4) * 4096;
         if (smem > 48 * 1024) {
             const cudaError_t e =
-                cudaFuncSetAttribute(crop_rect_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                cudaFuncSetAttribute(crop_rect_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
             if (e != cudaSuccess) return cuda_error(e, "rgbd_crop_affine: smem attribute");
         }
         crop_rect_kernel<<<grid, kCropThreads, smem, s>>>(a);

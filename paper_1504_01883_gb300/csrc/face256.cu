@@ -405,8 +405,8 @@ __global__ void __launch_bounds__(F256_THREADS, 1) lbp_face256_kernel(const LbpA
 
 int launch_face256(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
     const F256Layout l = f256_layout(a.crop);
-    cudaError_t e =
-        cudaFuncSetAttribute(lbp_face256_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.bytes);
+    static const int most = (int)f256_layout(255).bytes;
+    cudaError_t e = cudaFuncSetAttribute(lbp_face256_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e != cudaSuccess) return cuda_error(e, "lbp_fused_features: 0-255 histogram smem attribute");
     const int grid = std::min(a.n, ctx->props.sm_count);
     const uint32_t sw_inv = (uint32_t)((0x100000000ull + l.SW - 1) / l.SW);  // i / SW, exact for i < 2^16

@@ -99,6 +99,10 @@ struct DeviceGuard {
     }
 };
 
+// The dynamic shared memory a kernel may be launched with is one setting of the whole process and
+// device: launchers set the largest their kernel takes, whatever the call's own size, so that calls of
+// different sizes from several threads cannot lower it under one another.
+
 // Grows the workspace of ctx to `bytes`.  Refuses while `stream` is capturing.
 int ensure_workspace(rgbd_ctx* ctx, size_t bytes, cudaStream_t stream);
 

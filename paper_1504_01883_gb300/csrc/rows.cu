@@ -336,7 +336,8 @@ int launch_normalize(const uint16_t* feats, int n, int dim, int nbins, int x_dty
         else if (x_dtype == RGBD_DT_BF16X3)
             kernel = centred ? normalize_rows_kernel<RGBD_DT_BF16X3, true> : normalize_rows_kernel<RGBD_DT_BF16X3, false>;
         if (staged > 48 * 1024) {
-            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)staged);
+            constexpr size_t most = 2 * (size_t)65536 + sizeof(float2) * (65536 / 8 + 2);
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
             if (e != cudaSuccess) return cuda_error(e, "lbp_normalize_features: smem attribute");
         }
         kernel<<<n, kRowThreads, staged, s>>>(feats, n, dim, nbins, inv, lpc, wide, x_out, k_pad, x_scale, xsq,

@@ -310,8 +310,8 @@ template <int T, int EPT>
 cudaError_t launch_smo(const float* K, int n, const int32_t* labels, int n_classes, float cost, float eps,
                        int max_iter, float* coef, float* bias, int32_t* iters, bool marked, cudaStream_t s) {
     const size_t smem = sizeof(float) * (size_t)n;
-    const cudaError_t e =
-        cudaFuncSetAttribute(smo_kernel<T, EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = cudaFuncSetAttribute(smo_kernel<T, EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)sizeof(float) * T * EPT);
     if (e != cudaSuccess) return e;
     smo_kernel<T, EPT><<<n_classes, T, smem, s>>>(K, n, labels, cost, eps, max_iter, coef, bias, iters, marked);
     return cudaGetLastError();

@@ -534,3 +534,41 @@ def test_training_of_a_lost_handover_gives_zeros(B, ctx):
     assert not any(t.any() for t in got)
     assert all(torch.equal(u, v) for u, v in zip(B.svm_train_rbf(ctx, *args, max_iter=60), want))
     assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("call", ["crop", "normalise", "face256"])
+def test_threads_with_different_sizes(B, call):
+    """Two threads, each with a context and a stream, make calls that take different amounts of shared
+    memory: a limit that one sets must not be lowered by the other before the launch."""
+    import threading
+    rects = torch.zeros((1000, 5), dtype=torch.int32, device="cuda")
+    rects[:, 3:] = 16
+    grey = torch.zeros((1, 16, 16), dtype=torch.uint8, device="cuda")
+    depth = torch.ones((1, 16, 16), dtype=torch.int16, device="cuda")
+    rows = {d: torch.ones((2, d), dtype=torch.int16, device="cuda") for d in (59 * 450, 59 * 1100)}
+    work = {"crop": lambda c, s, big: B.rgbd_crop_affine(c, grey, depth, rects, 4096 if big else 3100, 4, stream=s),
+            "normalise": lambda c, s, big: B.lbp_normalize_features(c, rows[59 * (1100 if big else 450)], "bf16", stream=s),
+            "face256": lambda c, s, big: B.lbp_fused_features(c, grey, depth, rects[:2], crop=255 if big else 40,
+                                                              flags=B.LBP_FACE_HIST256, stream=s)}[call]
+    torch.cuda.synchronize()
+    errors, start = [], threading.Barrier(2)
+
+    def loop(big):
+        c, s = B.Context(0), torch.cuda.Stream()
+        try:
+            start.wait()
+            with torch.cuda.stream(s):
+                for _ in range(400):
+                    work(c, s, big)
+        except B.RgbdError as e:
+            errors.append(str(e))
+        finally:
+            s.synchronize()
+            c.close()
+
+    threads = [threading.Thread(target=loop, args=(big,)) for big in (False, True)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[0]
