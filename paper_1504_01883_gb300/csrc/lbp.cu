@@ -34,6 +34,7 @@
 #include <stddef.h>
 
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "internal.h"
@@ -845,15 +846,21 @@ template <int S, int TPC, bool TABLE>
 int launch_fused_t(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
     using Shared = Smem<S, TPC>;
     const size_t smem = TABLE ? sizeof(Shared) : offsetof(Shared, qbf);  // the table comes last
-    static int blocks = -1;
-    if (blocks < 0) {
+    // resident CTAs per SM, asked once per device (0: not yet), as is the shared-memory limit set: both
+    // hold for the device that is current
+    constexpr int kDevices = 64;
+    static std::atomic<int> known[kDevices];
+    const int dev = ctx->props.device;
+    int blocks = dev < kDevices ? known[dev].load(std::memory_order_acquire) : 0;
+    if (blocks == 0) {
         cudaError_t e = cudaFuncSetAttribute(lbp_fused_kernel<S, TPC, TABLE>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return cuda_error(e, "lbp_fused_features: smem attribute");
-        int b = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, lbp_fused_kernel<S, TPC, TABLE>, Cfg<S, TPC>::NT, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, lbp_fused_kernel<S, TPC, TABLE>, Cfg<S, TPC>::NT,
+                                                          smem);
         if (e != cudaSuccess) return cuda_error(e, "lbp_fused_features: occupancy");
-        blocks = b > 0 ? b : 1;
+        blocks = std::max(blocks, 1);
+        if (dev < kDevices) known[dev].store(blocks, std::memory_order_release);
     }
     // the tuning value counts the CTAs of the 128 x 128 shape, whose occupancy is 2
     const int per_sm = ctx->tune_lbp_ctas_per_sm > 0 ? std::min(ctx->tune_lbp_ctas_per_sm, blocks) : blocks;
