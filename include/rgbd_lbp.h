@@ -133,7 +133,9 @@ int rgbd_ctx_status(rgbd_ctx* ctx, uint32_t* flags, int clear);
 /* Launch-shape knobs of a context, set by an autotuner (0 restores the built-in choice).
  * They change only how work is laid out on the GPU, never a result bit of the integer
  * path; scores change within rounding (the split of the SV sum).
- *   RGBD_TUNE_LBP_CTAS_PER_SM   resident fused-kernel CTAs per SM (1 or 2)
+ *   RGBD_TUNE_LBP_CTAS_PER_SM   resident fused-kernel CTAs per SM, counted for crops of 128, of
+ *                               which two fit: 1 or 2; other crops have half of their CTAs
+ *                               resident (1), or all (2)
  *   RGBD_TUNE_TC_SPLITS         SV-tile ranges per 128-row block in tensor-core scoring
  *   RGBD_TUNE_LBP_SHAPE         fused-kernel tile shape: 0 = default (2; 3 for crops of 64 and
  *                               96 and at most a face per SM), 1 = one thread

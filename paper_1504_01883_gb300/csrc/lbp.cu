@@ -862,8 +862,8 @@ int launch_fused_t(rgbd_ctx* ctx, const LbpArgs& a, cudaStream_t s) {
         blocks = std::max(blocks, 1);
         if (dev < kDevices) known[dev].store(blocks, std::memory_order_release);
     }
-    // the tuning value counts the CTAs of the 128 x 128 shape, whose occupancy is 2
-    const int per_sm = ctx->tune_lbp_ctas_per_sm > 0 ? std::min(ctx->tune_lbp_ctas_per_sm, blocks) : blocks;
+    // the tuning value counts the CTAs of the 128 x 128 shape, which fits twice: half of what fits, or all
+    const int per_sm = ctx->tune_lbp_ctas_per_sm == 1 ? std::max(1, blocks / 2) : blocks;
     const int grid = (int)std::min<long long>((long long)a.n, (long long)per_sm * ctx->props.sm_count);
     LbpArgs la = a;
     if (grid >= a.n) {

@@ -572,3 +572,34 @@ def test_threads_with_different_sizes(B, call):
     for t in threads:
         t.join()
     assert not errors, errors[0]
+
+
+@pytest.mark.parametrize("crop", [32, 64, 96])
+def test_two_ctas_per_sm_are_those_of_a_128_crop(B, ctx, crop):
+    """A context tuned for 128 x 128 batches (two CTAs per SM, all that fit) keeps the occupancy of smaller
+    crops, of which 4 to 16 fit: as fast as untuned (at two, 32 x 32 crops take several times as long), and
+    the same counts; one means half of what fits."""
+    grey, depth, r = synth.frames_with_rects(crop, 8, 20, 30, 110, H=240, W=320)
+    g, d, rects = dev_u8(grey), dev_u16(depth), B.rects_tensor(np.concatenate([r] * 25))  # 4000 faces
+
+    def run():
+        best = []
+        for _ in range(12):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            f, _, _ = B.lbp_fused_features(ctx, g, d, rects, crop=crop)
+            e1.record()
+            torch.cuda.synchronize()
+            best.append(e0.elapsed_time(e1))
+        return min(best), f
+
+    t0, f0 = run()
+    times = {}
+    for ctas in (2, 1):
+        ctx.set_tuning(B.TUNE_LBP_CTAS_PER_SM, ctas)
+        try:
+            times[ctas], f = run()
+        finally:
+            ctx.set_tuning(B.TUNE_LBP_CTAS_PER_SM, 0)
+        assert torch.equal(f, f0)
+    assert times[2] < 1.25 * t0, (t0, times)
