@@ -541,7 +541,7 @@ def main():
         peak_t = pk["bf16_tflops"] * NOMINAL_RATIO[dt]
     rl_k1 = {"kernel": f"lbp_fused_kernel<128, {tuning.lbp_shape or 2}>", "bound": "hbm", "achieved": round(k1_gbs, 1),
              "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": round(k1_gbs / pk["hbm_gbs"], 4),
-             "traffic": measured_traffic("k1", f"shape{tuning.lbp_shape or 2}/ctas{tuning.lbp_ctas_per_sm}/{dt}"),
+             "traffic": measured_traffic("k1", f"shape{tuning.lbp_shape or 2}/ctas{tuning.lbp_ctas_per_sm or 2}/{dt}"),
              "algorithmic_bytes": k1_bytes, "ms": round(k1_ms, 4), "peak_source": src,
              "frac_without_normalised_row": round(k1_bytes_u16 / (k1_ms * 1e-3) / 1e9 / pk["hbm_gbs"], 4),
              "algorithmic_bytes_without_normalised_row": k1_bytes_u16}

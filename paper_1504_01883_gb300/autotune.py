@@ -7,7 +7,8 @@ candidate settings of the context's tuning knobs and keeps the fastest:
       128 x 128 crop laid out as 16 x 16 cells of 8 x 8 pixels, with either one thread per
       4 x 8 half cell (512 threads, 64 registers), one thread per cell (256 threads, up to
       128 registers) or one per 4 x 4 quarter cell (1024 threads, one CTA per SM), and one or
-      two such CTAs in flight per SM;
+      two such CTAs in flight per SM; the library's own choice, which also looks at the crop and
+      the number of faces of each call, stays unless another is clearly faster;
   K2  how many SV-tile ranges ("splits") each 128-row block of the tensor-core scoring
       kernel is cut into (the row x SV tiling across SMs), and whether CTA pairs run one
       256-row MMA (tcgen05 cta_group::2) or every CTA runs its own 128-row MMA.
@@ -26,7 +27,7 @@ import torch
 
 from . import binding as B
 
-CACHE_VERSION = 4  # bumped whenever the set of knobs changes
+CACHE_VERSION = 5  # bumped whenever the set of knobs, or a kernel they choose among, changes
 CACHE_PATH = os.environ.get("RGBD_TUNE_CACHE",
                             os.path.join(os.path.expanduser("~"), ".cache", "rgbd_lbp_gb300", "tune.json"))
 
@@ -46,7 +47,10 @@ class Tuning:
 
 
 PAIRING_NAMES = {2: "single", 3: "pair"}
-SHAPE_NAMES = {1: "cell", 2: "halfcell", 3: "quartercell"}
+SHAPE_NAMES = {0: "auto", 1: "cell", 2: "halfcell", 3: "quartercell"}
+# A forced layout holds for every call of the context, whatever its crop and faces, so it has to beat
+# the library's own choice on the workload by more than timings differ.
+CLEARLY = 0.97
 
 
 def _time(fn, stream, reps=3):
@@ -110,16 +114,15 @@ def tune(ctx, key, stage1, stage2, n_rows, n_sv, stream, use_cache=True, tensor_
             return t, dict(cache[full_key], cached=True)
     report = {"k1": {}, "k2": {}}
     best = Tuning()
-    # K1: tile shape x CTAs per SM
+    # K1: the library's choice, then tile shape x CTAs per SM (a 1024-thread CTA fills an SM's registers)
     best_ms = None
-    for shape in (2, 1, 3):
-        for c in ((2, 1) if shape != 3 else (1,)):  # a 1024-thread CTA fills an SM's registers
-            ctx.set_tuning(B.TUNE_LBP_SHAPE, shape)
-            ctx.set_tuning(B.TUNE_LBP_CTAS_PER_SM, c)
-            ms = _time(stage1, stream)
-            report["k1"][f"{SHAPE_NAMES[shape]}/{c}"] = ms
-            if best_ms is None or ms < best_ms:
-                best_ms, best.lbp_shape, best.lbp_ctas_per_sm = ms, shape, c
+    for shape, c in ((0, 0), (2, 2), (2, 1), (1, 2), (1, 1), (3, 1)):
+        ctx.set_tuning(B.TUNE_LBP_SHAPE, shape)
+        ctx.set_tuning(B.TUNE_LBP_CTAS_PER_SM, c)
+        ms = _time(stage1, stream)
+        report["k1"][f"{SHAPE_NAMES[shape]}/{c}" if shape else SHAPE_NAMES[shape]] = ms
+        if best_ms is None or ms < (best_ms if best.lbp_shape else CLEARLY * best_ms):
+            best_ms, best.lbp_shape, best.lbp_ctas_per_sm = ms, shape, c
     ctx.set_tuning(B.TUNE_LBP_SHAPE, best.lbp_shape)
     ctx.set_tuning(B.TUNE_LBP_CTAS_PER_SM, best.lbp_ctas_per_sm)
     # K2: splits x CTA pairing
