@@ -171,7 +171,7 @@ int score_rbf_tc_external_ws(rgbd_ctx* ctx, const rgbd_svm* m, const void* x, co
 // Scores of few rows from partial products G [kz][n][n_pad] of the kernel launched just before on
 // s (which zeroes counters, one per 16 rows, and lets its dependents launch early): adds the K
 // ranges, finishes every SV tile and combines the tiles.  part [tiles][n][C_pad] and ref [tiles][n]
-// are scratch; models of up to 256 SV tiles.
+// are scratch; models of more than 256 SV tiles with up to 8 rows.
 int launch_rows_epilogue(const rgbd_svm* m, const float* gpart, int kz, int n, const float* xsq, float gscale,
                          float d2_min, float* part, float* ref, uint32_t* counters, float* scores, int32_t* labels,
                          cudaStream_t s);

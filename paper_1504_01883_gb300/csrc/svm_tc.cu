@@ -1072,7 +1072,7 @@ __global__ void __launch_bounds__(SK_WARPS * 32, 1)
 // classes, from the end of the kernel before: 17 us with 8 warps, a class at a time and block-wide
 // passes for r and F (5.8 us the classes, 5.3 us the combine), 10 us now.
 // d2_min: least d^2 (0 for the exact fp32 path, -infinity for the tensor-core paths).
-// Any gamma: where the mean lies more than kRefReach / gamma above the tile's least distance, r is that
+// Any gamma: where the mean lies more than reach = 20 / gamma above the tile's least distance, r is that
 // far above it, and the combine's reference r* (tile 0's r) is held as near to the least r.  So neither
 // F nor delta exceeds e^20, their product stays far inside fp32, and exp(-gamma r*) is zero only where
 // every kernel value is below e^-64: a row that is itself a support vector of a widely spread model
@@ -1082,11 +1082,19 @@ constexpr int SKE_ROWS = 16;
 constexpr int SKE_THREADS = 32 * SKE_ROWS;
 size_t ske_smem(int C) { return sizeof(float) * (size_t)((C + 3) / 4 * 4 + SKE_ROWS) * BN; }
 
+// Least value of the warp's lanes (NaNs aside).
+__device__ __forceinline__ float warp_min(float v) {
+    float m;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v));
+    return m;
+}
+// PIECES: more than 256 tiles.
+template <bool PIECES>
 __global__ void __launch_bounds__(SKE_THREADS) rbf_splitk_epilogue_kernel(
     const float* __restrict__ gpart, int kz, int n_pad, int n, const float* __restrict__ xsq,
     const float* __restrict__ svsq, int n_sv, const float* __restrict__ coef, int C, int C_pad, float gamma,
-    float gscale, float d2_min, float* __restrict__ part, float* __restrict__ ref, uint32_t* __restrict__ counters,
-    int nt, const float* __restrict__ asum, const float* __restrict__ asum_tile, const float* __restrict__ bias,
+    float gscale, float d2_min, float reach, float* __restrict__ part, float* __restrict__ ref,
+    uint32_t* __restrict__ counters, int nt, const float* __restrict__ asum, const float* __restrict__ asum_tile, const float* __restrict__ bias,
     float* __restrict__ scores, int32_t* __restrict__ labels) {
     extern __shared__ __align__(16) float ske_smem_raw[];
     float* F = ske_smem_raw;            // [SKE_ROWS][BN]; later the combine's
@@ -1134,15 +1142,16 @@ __global__ void __launch_bounds__(SKE_THREADS) rbf_splitk_epilogue_kernel(
                 least = fminf(least, g[j]);
             }
         }
-        for (int off = 16; off > 0; off >>= 1) {
-            sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
-            least = fminf(least, __shfl_xor_sync(0xFFFFFFFFu, least, off));
-        }
-        const float r = fminf(sum / (float)max(valid, 1), least + kRefReach / gamma);
+        for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
+        least = warp_min(least);
+        const float r = fminf(sum / (float)max(valid, 1), least + reach);
 #pragma unroll
         for (int j = 0; j < PER; ++j)
             F[warp * BN + lane + 32 * j] = lane + 32 * j < valid ? expm1_near0(-gamma * (g[j] - r)) : 0.f;
-        if (lane == 0) ref[(size_t)tile * n + k0 + warp] = r;
+        if (lane == 0) {
+            ref[(size_t)tile * n + k0 + warp] = r;
+            r_star[warp] = r;  // (of a single tile)
+        }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
@@ -1197,51 +1206,70 @@ __global__ void __launch_bounds__(SKE_THREADS) rbf_splitk_epilogue_kernel(
     if (!last) return;
     // Shared memory reused: in F delta_s per row and tile and the scores behind them when they fit, in
     // A the tiles' coefficient sums (read by every row from global memory instead, they were 8 of
-    // the 11 us of this part).
-    float* s_del = F;               // [rows][nt] (nt <= 256)
-    float* s_sc = F + rows * nt;    // [rows][C]
-    const bool sc_fit = rows * nt + rows * C <= SKE_ROWS * BN;
-    float* s_as = A;                // [nt][C]
-#pragma unroll 4
-    for (int i = tid; i < nt * C; i += SKE_THREADS) s_as[i] = __ldcg(asum_tile + (size_t)(i / C) * C_pad + i % C);
-    if (warp < rows) {  // a warp = one row: its r* and every tile's delta
-        float* del = s_del + warp * nt;
-        float least = INFINITY;
-#pragma unroll 4
-        for (int t = lane; t < nt; t += 32) {
-            const float rt = __ldcg(ref + (size_t)t * n + k0 + warp);
-            del[t] = rt;
-            least = fminf(least, rt);
-        }
-        for (int off = 16; off > 0; off >>= 1) least = fminf(least, __shfl_xor_sync(0xFFFFFFFFu, least, off));
-        __syncwarp();
-        const float rs = fminf(del[0], least + kRefReach / gamma);
-        __syncwarp();
-#pragma unroll 1
-        for (int t = lane; t < nt; t += 32) del[t] = del[t] == rs ? 0.f : expm1f(-gamma * (del[t] - rs));
-        if (lane == 0) r_star[warp] = rs;
-    }
-    __syncthreads();
-    // thread = (row, class): the tiles' partial sums 16 at a time, added in tile order
+    // the 11 us of this part).  Models of more than 256 tiles (then of up to 8 rows, whose scores fit) go
+    // in pieces of 256, with the sums so far in the scores' place.
+    constexpr int PIECE = 256;
+    const int tw = PIECES ? PIECE : nt;
+    float* s_del = F;               // [rows][tw]
+    float* s_sc = F + rows * tw;    // [rows][C]
+    const bool sc_fit = rows * tw + rows * C <= SKE_ROWS * BN;
+    float* s_as = A;                // [tw][C]
     const size_t ts = (size_t)n * C_pad;
 #pragma unroll 1
-    for (int i = tid; i < rows * C; i += SKE_THREADS) {
-        const int k = i / C, c = i - k * C;
-        const float* pd = part + (size_t)(k0 + k) * C_pad + c;
-        const float as = __ldg(asum + c), bs = __ldg(bias + c);
-        float acc = 0.f;
+    for (int tb = 0; PIECES ? tb < nt : tb == 0; tb += PIECE) {
+        const int tn = PIECES ? min(PIECE, nt - tb) : nt;
+        if (tb) __syncthreads();  // the piece before has been read
+#pragma unroll 4
+        for (int i = tid; i < tn * C; i += SKE_THREADS)
+            s_as[i] = __ldcg(asum_tile + (size_t)(tb + i / C) * C_pad + i % C);
+        if (nt == 1) {
+            if (tid < rows) s_del[tid] = 0.f;
+        } else if (warp < rows) {  // a warp = one row: its r* (from all tiles) and every tile's delta
+            float* del = s_del + warp * tw;
+            const float* rp = ref + (size_t)tb * n + k0 + warp;
+            float least = INFINITY;
+#pragma unroll 4
+            for (int t = lane; t < tn; t += 32) {
+                const float rt = __ldcg(rp + (size_t)t * n);
+                del[t] = rt;
+                least = fminf(least, rt);
+            }
+            if (tb == 0) {
+                for (int t = PIECE + lane; PIECES && t < nt; t += 32) least = fminf(least, __ldcg(rp + (size_t)t * n));
+                least = warp_min(least);
+            }
+            __syncwarp();
+            const float rs = tb == 0 ? fminf(del[0], least + reach) : r_star[warp];
+            __syncwarp();
 #pragma unroll 1
-        for (int t0 = 0; t0 < nt; t0 += 16) {
-            float d[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) d[j] = t0 + j < nt ? __ldcg(pd + (size_t)(t0 + j) * ts) : 0.f;
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-                if (t0 + j < nt) acc += d[j] + s_del[k * nt + t0 + j] * (s_as[(t0 + j) * C + c] + d[j]);
+            for (int t = lane; t < tn; t += 32) del[t] = del[t] == rs ? 0.f : expm1f(-gamma * (del[t] - rs));
+            if (lane == 0) r_star[warp] = rs;
         }
-        const float sc = expf(-gamma * r_star[k]) * (as + acc) + bs;
-        scores[(size_t)(k0 + k) * C + c] = sc;
-        if (sc_fit) s_sc[i] = sc;
+        __syncthreads();
+        // thread = (row, class): the tiles' partial sums 16 at a time, added in tile order
+#pragma unroll 1
+        for (int i = tid; i < rows * C; i += SKE_THREADS) {
+            const int k = i / C, c = i - k * C;
+            const float* pd = part + (size_t)tb * ts + (size_t)(k0 + k) * C_pad + c;
+            const float as = __ldg(asum + c), bs = __ldg(bias + c);
+            float acc = tb ? s_sc[i] : 0.f;
+#pragma unroll 1
+            for (int t0 = 0; t0 < tn; t0 += 16) {
+                float d[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) d[j] = t0 + j < tn ? __ldcg(pd + (size_t)(t0 + j) * ts) : 0.f;
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    if (t0 + j < tn) acc += d[j] + s_del[k * tw + t0 + j] * (s_as[(t0 + j) * C + c] + d[j]);
+            }
+            if (PIECES && tb + PIECE < nt) {
+                s_sc[i] = acc;
+                continue;
+            }
+            const float sc = expf(-gamma * r_star[k]) * (as + acc) + bs;
+            scores[(size_t)(k0 + k) * C + c] = sc;
+            if (sc_fit) s_sc[i] = sc;
+        }
     }
     if (!labels) return;
     __syncthreads();
@@ -1602,13 +1630,14 @@ int launch_rows_epilogue(const rgbd_svm* m, const float* gpart, int kz, int n, c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaFuncSetAttribute(rbf_splitk_epilogue_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)ske_smem(MAX_CPAD));
+    auto kernel = nt > 256 ? rbf_splitk_epilogue_kernel<true> : rbf_splitk_epilogue_kernel<false>;
+    cudaError_t e =
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ske_smem(MAX_CPAD));
     if (e != cudaSuccess) return cuda_error(e, "svm_score: split-K epilogue smem attribute");
-    e = cudaLaunchKernelEx(
-        &cfg, rbf_splitk_epilogue_kernel, gpart, kz, m->n_pad, n, xsq, (const float*)m->sv_sq, m->n_sv,
-        (const float*)m->coef, m->C, m->C_pad, m->gamma, gscale, d2_min, part, ref, counters, nt,
-        (const float*)m->asum, (const float*)m->asum_tile, (const float*)m->bias, scores, labels);
+    e = cudaLaunchKernelEx(&cfg, kernel, gpart, kz, m->n_pad, n, xsq, (const float*)m->sv_sq, m->n_sv,
+                           (const float*)m->coef, m->C, m->C_pad, m->gamma, gscale, d2_min, kRefReach / m->gamma, part,
+                           ref, counters, nt, (const float*)m->asum, (const float*)m->asum_tile,
+                           (const float*)m->bias, scores, labels);
     if (e != cudaSuccess) return cuda_error(e, "svm_score: split-K epilogue launch");
     return RGBD_OK;
 }

@@ -603,3 +603,26 @@ def test_two_ctas_per_sm_are_those_of_a_128_crop(B, ctx, crop):
             ctx.set_tuning(B.TUNE_LBP_CTAS_PER_SM, 0)
         assert torch.equal(f, f0)
     assert times[2] < 1.25 * t0, (t0, times)
+
+
+@pytest.mark.parametrize("n_sv", [65536, 65537, 132000])
+@pytest.mark.parametrize("n,gamma", [(1, 0.3), (8, 0.3), (3, 20.0)])
+def test_few_rows_against_more_than_256_tiles(B, ctx, orc, n_sv, n, gamma):
+    """Up to eight fp32 rows against models around and beyond 65536 support vectors, which the few-row
+    epilogue combines in pieces of 256 tiles: scores within the path's bound of fp64."""
+    rng = synth.rng_for(n_sv + n)
+    dim, C = 4 * 59, 5
+    X, SV = synth.poisson_counts(rng, n, dim), synth.poisson_counts(rng, n_sv, dim)
+    X[0] = SV[n_sv - 1]
+    a = rng.normal(0, 1, (C, n_sv)).astype(np.float32)
+    b = rng.normal(0, 0.01, C).astype(np.float32)
+    model = B.svm_train_data_pack(ctx, dev_u16(SV), dev_f32(a), dev_f32(b), gamma=gamma, dtype="f32")
+    x, q = B.lbp_normalize_features(ctx, dev_u16(X), "f32")
+    s, lab = B.svm_score(ctx, model, x, q)
+    assert ctx.status() == 0
+    x64, sv64 = orc.normalize_f64(X), orc.normalize_f64(SV)
+    d2 = (x64 ** 2).sum(1)[:, None] + (sv64 ** 2).sum(1)[None, :] - 2.0 * x64 @ sv64.T
+    ref = np.exp(-gamma * np.maximum(d2, 0.0)) @ a.astype(np.float64).T + b
+    # the path's stated bound (1e-5 of the score scale)
+    assert rel_score_error(s.cpu().numpy(), ref, rbf_error_scale(x64, sv64, a, b, gamma)) <= 1e-5
+    assert (lab.cpu().numpy() == s.cpu().numpy().argmax(1)).all()
