@@ -103,6 +103,13 @@ struct DeviceGuard {
 // device: launchers set the largest their kernel takes, whatever the call's own size, so that calls of
 // different sizes from several threads cannot lower it under one another.
 
+// The next larger number of ranges that nt tiles, ceil(nt / sp) in each, make exactly (0: none): of nt
+// numbers only about 2 sqrt(nt) differ in their longest range.
+inline int next_split(int nt, int sp) {
+    const int tps = (nt + sp - 1) / sp;
+    return tps > 1 ? (nt + tps - 2) / (tps - 1) : 0;
+}
+
 // Grows the workspace of ctx to `bytes`.  Refuses while `stream` is capturing.
 int ensure_workspace(rgbd_ctx* ctx, size_t bytes, cudaStream_t stream);
 
@@ -155,9 +162,13 @@ int score_linear(rgbd_ctx* ctx, const rgbd_svm* m, const float* x, int n, float*
                  int32_t* labels, cudaStream_t s);
 int score_rbf_f32(rgbd_ctx* ctx, const rgbd_svm* m, const float* x, const float* xsq, int n,
                   float* scores, int32_t* labels, cudaStream_t s);
-// Workspace bytes a scoring call of n rows takes (0: none, or a model the path rejects).
+// Workspace bytes a scoring call of n rows takes (0: none, or a model the path rejects).  Within 64 rows
+// (of the same 64) more rows take more, but for the steps of score_rbf_tc_bytes behind 32 rows, of
+// score_rbf_f32_bytes behind 8 and behind f32_slice_rows (the most rows whose partial sums are kept per
+// SV tile).
 size_t score_rbf_f32_bytes(rgbd_ctx* ctx, const rgbd_svm* m, int n);
 size_t score_rbf_tc_bytes(rgbd_ctx* ctx, const rgbd_svm* m, int n);
+int f32_slice_rows(const rgbd_svm* m);
 int score_rbf_tc(rgbd_ctx* ctx, const rgbd_svm* m, const void* x, const float* xsq, int n,
                  float x_scale, float* scores, int32_t* labels, cudaStream_t s);
 

@@ -410,9 +410,14 @@ int rgbd_server_create(const rgbd_svm* model, const rgbd_server_config* cfg, rgb
         // some larger batches by tiles), reserved now: growing it during serving would
         // put a cudaFree / cudaMalloc pair, which wait for the device, in a frame's latency
         size_t ws = 0;
-        for (int nq = 1; nq <= c.max_batch_faces; ++nq)
-            ws = std::max(ws, model->dtype == RGBD_DT_F32 ? rgbd::score_rbf_f32_bytes(s->ctx, model, nq)
-                                                           : rgbd::score_rbf_tc_bytes(s->ctx, model, nq));
+        auto ask = [&](int rows) {
+            rows = std::min(rows, c.max_batch_faces);
+            if (rows < 1) return;
+            ws = std::max(ws, model->dtype == RGBD_DT_F32 ? rgbd::score_rbf_f32_bytes(s->ctx, model, rows)
+                                                           : rgbd::score_rbf_tc_bytes(s->ctx, model, rows));
+        };
+        ask(8), ask(32), ask(rgbd::f32_slice_rows(model));
+        for (int rows = 64; rows < c.max_batch_faces + 64; rows += 64) ask(rows);
         rc = ws ? rgbd::ensure_workspace(s->ctx, ws, nullptr) : RGBD_OK;
         if (rc) {
             free_server(s);

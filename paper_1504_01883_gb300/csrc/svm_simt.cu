@@ -333,6 +333,9 @@ __global__ void __launch_bounds__(F32Tile<BM, BM>::NT, 1) rbf_f32_kernel(const F
     }
 }
 
+// Most bytes of partial sums for which every SV tile keeps a slice of its own.
+constexpr size_t kF32SliceBytes = (size_t)256 << 20;
+
 // How a call of n rows is laid out, and the workspace it takes.
 struct F32Plan {
     int bm, mt, nt, slices, tps;
@@ -354,15 +357,15 @@ F32Plan plan_f32(const rgbd_ctx* ctx, const rgbd_svm* m, int n) {
     // while a slice of partial sums per SV tile stays small; smaller tiles on more CTAs otherwise.
     const bool big = tiles(128) >= sms;
     if (!big) tiles(64);
-    p.ordered = big && sizeof(float) * (size_t)p.nt * n * m->C <= ((size_t)256 << 20);
+    p.ordered = big && sizeof(float) * (size_t)p.nt * n * m->C <= kF32SliceBytes;
     p.tps = 1;
     if (!p.ordered) {
         // fewest waves of tiles on the SMs (64 x 64 tiles: four CTAs each), fewest slices on ties
         const long long slots = (long long)sms * (big ? 1 : 4);
         long long best = -1;
-        for (int sp = 1; sp <= p.nt; ++sp) {
+        for (int sp = 1; sp; sp = next_split(p.nt, sp)) {
             const int tps = (p.nt + sp - 1) / sp;
-            const long long cost = (((long long)p.mt * ((p.nt + tps - 1) / tps) + slots - 1) / slots) * tps;
+            const long long cost = (((long long)p.mt * sp + slots - 1) / slots) * tps;
             if (best < 0 || cost < best) best = cost, p.tps = tps;
         }
     }
@@ -700,6 +703,11 @@ static bool takes_rows8(int n) { return n <= 8; }
 size_t score_rbf_f32_bytes(rgbd_ctx* ctx, const rgbd_svm* m, int n) {
     if (takes_rows8(n)) return plan_rows8(ctx, m, n).bytes;
     return plan_f32(ctx, m, n).bytes;
+}
+
+int f32_slice_rows(const rgbd_svm* m) {
+    const size_t nt = ((size_t)m->n_sv + 127) / 128;
+    return (int)std::min<size_t>(kF32SliceBytes / (sizeof(float) * nt * m->C), 1u << 30);
 }
 
 int score_rbf_f32(rgbd_ctx* ctx, const rgbd_svm* m, const float* x, const float* xsq, int n,

@@ -1302,9 +1302,8 @@ __global__ void __launch_bounds__(SKE_THREADS) rbf_splitk_epilogue_kernel(
 int choose_splits(int mt, int nt, int sms) {
     int best = 1;
     long long best_cost = -1;
-    for (int sp = 1; sp <= nt; ++sp) {
+    for (int sp = 1; sp; sp = next_split(nt, sp)) {
         const int tps = (nt + sp - 1) / sp;
-        if ((nt + tps - 1) / tps != sp) continue;
         const long long waves = ((long long)mt * sp + sms - 1) / sms;
         const long long cost = waves * (tps + 1);
         if (best_cost < 0 || cost * 100 < best_cost * 97) {
