@@ -25,19 +25,18 @@ namespace {
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
 // ---------------------------------------------------------------------------------------
-// Linear SVM: a CTA takes R rows and 8 classes at a time, its threads split the columns.  One row
+// Linear SVM: a CTA takes R rows and CG classes at a time, its threads split the columns.  One row
 // is bound by latency (a 64 x 64 crop: 1 row of 3840, 5 classes), so every load of a pass is in
-// flight at once; many rows are bound by reading the weights from L2, which R rows share.
-// 1 row: 19 us with a warp per class and one load in flight per lane, 5.5 us now.  15104 columns, 64
-// classes: 172 us -> 43 us (1 row), 1350 us -> 640 us (4096 rows).
+// flight at once; many rows are bound by reading the weights from L2, which R rows share, and, when
+// rows are short, by the sums over the threads at the end of a pass.
 // ---------------------------------------------------------------------------------------
-template <int R, int T>
+template <int R, int T, int CG>
 __global__ void __launch_bounds__(T) linear_kernel(const float* __restrict__ x, int n, int k_pad,
                                                              const float* __restrict__ w,
                                                              const float* __restrict__ bias, int C,
                                                              float* __restrict__ scores,
                                                              int32_t* __restrict__ labels) {
-    constexpr int CG = 8, NW = T / 32;
+    constexpr int NW = T / 32;
     __shared__ float part[NW][R * CG];
     __shared__ float row_scores[R][256];  // C <= 256
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k4 = k_pad / 4;
@@ -633,20 +632,34 @@ int launch_reduce_scores(const float* part, const float* ref, int splits, int n,
 
 int score_linear(rgbd_ctx* ctx, const rgbd_svm* m, const float* x, int n, float* scores,
                  int32_t* labels, cudaStream_t s) {
-    // Few rows: a CTA of 16 warps each.  Many rows: four per CTA where the weights' traffic counts
-    // (15104 columns, 64 classes: 178 us against 190 us with a warp per class at 700 rows, 640 us
-    // against 1350 us at 4096), else CTAs of 4 warps (3776 columns, 5 classes, 4096 rows: 25 us,
-    // 51 us with 16 warps, 35 us with a warp per class).
-    const bool many = n >= 4 * ctx->props.sm_count;
+    // As many threads per row as let every row be resident at once: 16 warps up to a row per SM, 8 up to
+    // four, 4 up to eight; more rows go four to a CTA.  Classes at a time: no more than there are, and few
+    // where a CTA's registers would cost residents, but for up to 8 classes, which then take one pass.
+    // Against a warp per class and row (columns x classes, rows: before -> now, us): 3840 x 5, 1: 7.2 -> 3.3;
+    // 944 x 2, 20000: 25.5 -> 11; 944 x 64, 500: 19.9 -> 15.6 (30 with 16 warps), 2400: 56 -> 39 (210 with four
+    // rows to 16 warps); 15104 x 64, 1: 156 -> 39, 500: 183 -> 90, 5000: 1529 -> 763.
+    const int per_sm = (n + ctx->props.sm_count - 1) / ctx->props.sm_count, C = m->C;
     auto launch = [&](auto kernel, int rows, int threads) {
-        kernel<<<(n + rows - 1) / rows, threads, 0, s>>>(x, n, m->k_pad, m->coef, m->bias, m->C, scores, labels);
+        kernel<<<(n + rows - 1) / rows, threads, 0, s>>>(x, n, m->k_pad, m->coef, m->bias, C, scores, labels);
     };
-    if (!many)
-        launch(linear_kernel<1, 512>, 1, 512);
-    else if (m->C >= 16)
-        launch(linear_kernel<4, 512>, 4, 512);
-    else
-        launch(linear_kernel<1, 128>, 1, 128);
+    if (per_sm > 8) {
+        if (m->k_pad >= 12000 && C > 4)  // (4 warps, 4 classes at a time: 1.2 x as long)
+            launch(linear_kernel<4, 256, 8>, 4, 256);
+        else
+            C <= 2 ? launch(linear_kernel<4, 128, 2>, 4, 128) : launch(linear_kernel<4, 128, 4>, 4, 128);
+    } else if (per_sm > 4) {
+        C <= 2             ? launch(linear_kernel<1, 128, 2>, 1, 128)
+        : C > 4 && C <= 8 ? launch(linear_kernel<1, 128, 8>, 1, 128)
+                           : launch(linear_kernel<1, 128, 4>, 1, 128);
+    } else if (per_sm > 1) {
+        C <= 2                  ? launch(linear_kernel<1, 256, 2>, 1, 256)
+        : C > 4 && per_sm <= 2 ? launch(linear_kernel<1, 256, 8>, 1, 256)
+                                : launch(linear_kernel<1, 256, 4>, 1, 256);
+    } else {
+        C <= 2   ? launch(linear_kernel<1, 512, 2>, 1, 512)
+        : C <= 4 ? launch(linear_kernel<1, 512, 4>, 1, 512)
+                 : launch(linear_kernel<1, 512, 8>, 1, 512);
+    }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "svm_score: linear launch");
     return RGBD_OK;

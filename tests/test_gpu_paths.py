@@ -645,3 +645,25 @@ def test_server_of_a_large_model_and_batch_is_created_quickly(B, ctx):
 
     create(64)
     assert min(create(65536) for _ in range(3)) < 0.6
+
+
+@pytest.mark.parametrize("per_sm", [1, 2, 4, 8, 9])
+@pytest.mark.parametrize("dim,C", [(59, 1), (944, 2), (59, 3), (944, 4), (944, 5), (59, 8), (944, 9), (59, 33),
+                                   (12036, 5), (12036, 3)])
+def test_linear_scores_by_rows_per_sm(B, ctx, per_sm, dim, C):
+    """Linear scores around the row counts where the threads per row change (a row, two, four and eight per
+    SM), with class counts on both sides of the two, four and eight taken at a time."""
+    rng = synth.rng_for(per_sm + dim + C)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    w, b = synth.linear_model(rng, C, dim)
+    model = B.svm_train_data_pack(ctx, None, dev_f32(w), dev_f32(b), kernel=B.KERNEL_LINEAR, dim=dim)
+    for n in {per_sm * sms, (per_sm - 1) * sms + 1, per_sm * sms - 2}:
+        x = rng.uniform(0, 0.1, (n, B.k_pad_for(dim))).astype(np.float32)
+        x[:, dim:] = 0
+        s, lab = B.svm_score(ctx, model, dev_f32(x))
+        x64 = x[:, :dim].astype(np.float64)
+        ref = x64 @ w.astype(np.float64).T + b
+        scale = np.abs(x64) @ np.abs(w.astype(np.float64)).T + np.abs(b)
+        # fp32 chains of at most 12036 / 128 products and sums over 128 threads, well inside 1e-5
+        assert np.all(np.abs(s.cpu().numpy() - ref) <= 1e-5 * scale)
+        assert (lab.cpu().numpy() == s.cpu().numpy().argmax(1)).all()
