@@ -86,8 +86,7 @@ struct RoiWindow {
 // Only the four extremes are wanted, so the window is scanned from its edges inwards: rows from
 // the top and from the bottom until one holds a pixel, then, between those rows, the columns
 // outside the extremes found so far.  A face fills its box, so this reads the margins (a few rows,
-// and the columns that only a nearer surface could have reached) instead of the area; a window
-// without any pixel is read twice.  What is left is a chain of few L2 or DRAM round trips, so
+// and the columns that only a nearer surface could have reached) instead of the area.  What is left is a chain of few L2 or DRAM round trips, so
 // each step issues all its loads first (two rows of the window per warp, 16 rows of a column).
 // 4096 boxes over 256 frames of 640x480, faces of side 48..256: 640 us when every window pixel was
 // tested with a division, 95 us with the scan from the edges, 86 us since rows that cannot meet the box
@@ -141,6 +140,7 @@ __global__ void __launch_bounds__(kRoiThreads) face_roi_kernel(const uint16_t* _
             // rows, a strip of one per warp from the top and one from the bottom at a time
             bool top = true, bottom = true;
             for (int s0 = 0; s0 <= i1 - i0 && (top || bottom); s0 += NW) {
+                if (top && bottom && 2 * s0 > i1 - i0) break;  // met in the middle: no pixel (600 of side 300..400: 82 -> 43 us)
                 const int it = i0 + s0 + warp, ib = i1 - s0 - warp;
                 // (a row that is above or below the box at both ends of the window cannot hold one)
                 const bool dt = top && it <= i1 && t.row_meets(it, j0, j1);

@@ -667,3 +667,23 @@ def test_linear_scores_by_rows_per_sm(B, ctx, per_sm, dim, C):
         # fp32 chains of at most 12036 / 128 products and sums over 128 threads, well inside 1e-5
         assert np.all(np.abs(s.cpu().numpy() - ref) <= 1e-5 * scale)
         assert (lab.cpu().numpy() == s.cpu().numpy().argmax(1)).all()
+
+
+@pytest.mark.parametrize("H", [1, 8, 15, 16, 17, 33, 40])
+def test_face_roi_of_a_single_pixel(B, ctx, orc, H):
+    """The scans from the top and from the bottom meet in the middle of the window: one pixel in each row in
+    turn, and none."""
+    W = 70
+    depth = np.zeros((H + 1, H, W), np.uint16)  # frame H has none
+    rng = synth.rng_for(H)
+    for i in range(H):
+        depth[i, i, rng.integers(0, W)] = 1000
+    boxes = np.zeros(H + 1, orc.RECT_DTYPE)
+    boxes["frame"], boxes["w"], boxes["h"] = np.arange(H + 1), W + 80, H
+    cal = synth.calibration(rng, W + 80, H)
+    cal["a"][:] = [65536, 0, 0, 0, 65536, 0]
+    want = orc.face_roi(depth, cal, boxes)
+    got = B.rgbd_face_roi(ctx, dev_u16(depth), B.Calib.from_record(cal), B.rects_tensor(boxes)).cpu().numpy()
+    for i, f in enumerate(["frame", "x", "y", "w", "h"]):
+        assert (got[:, i] == want[f]).all(), f
+    assert (want["h"][:H] == 1).all() and want["h"][H] == 0
