@@ -112,12 +112,14 @@ __global__ void __launch_bounds__(kCropThreads) crop_rect_kernel(const CropArgs 
     }
 }
 
-// The same split of the work for a general affine map: source points by 64-bit products per pixel.
+// A general affine map: source points by 64-bit products per pixel, a thread per group of 4 columns; a step
+// of a CTA is 8 rows of 32 groups where a row is whole warps, else 256 groups in a row, and a CTA takes
+// a.rows steps, so that neighbouring rows meet in its L1.  Bound by the products and the gathers.  600 maps
+// to 128x128: 74 us a thread per pixel, 57 us now; to 100x100 (25 groups a row) 48 and 37 us.
 __global__ void __launch_bounds__(kCropThreads) crop_affine_kernel(const CropArgs a) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int v0 = blockIdx.x * a.rows, v1 = min(a.oh, v0 + a.rows);
-    const int lpr = 1 << a.lanes_log2, rpw = 32 >> a.lanes_log2;
-    const int ql = lane & (lpr - 1), vl = v0 + warp * rpw + (lane >> a.lanes_log2);
+    const int per_row = a.ow4 / 32;  // of whole warps: a step is 8 rows of 32 groups
+    const bool tiled = a.ow4 % 32 == 0;
     for (int k = blockIdx.y; k < a.n; k += gridDim.y) {
         const rgbd_rect r = a.rects[k];
         const bool ok = r.frame >= 0 && r.frame < a.n_frames && r.w > 0 && r.h > 0;
@@ -127,21 +129,49 @@ __global__ void __launch_bounds__(kCropThreads) crop_affine_kernel(const CropArg
             for (int i = 0; i < 6; ++i) m[i] = __ldg(a.affine + 6 * (size_t)k + i);
         const uint8_t* gsrc = a.grey + (ok ? (size_t)r.frame * a.H * a.W : 0);
         const uint16_t* dsrc = a.depth + (ok ? (size_t)r.frame * a.H * a.W : 0);
-        for (int v = vl; v < v1; v += (kCropThreads / 32) * rpw)
-            for (int q = ql; q < a.ow4; q += lpr) {
-                uint32_t gw = 0, d[2] = {0, 0};
-                if (ok) {
+        for (int st = blockIdx.x * a.rows; st < (int)(blockIdx.x + 1) * a.rows; ++st) {
+            const int i = st * kCropThreads + threadIdx.x;
+            const int v = tiled ? st / per_row * (kCropThreads / 32) + warp : i / a.ow4;
+            const int q = tiled ? st % per_row * 32 + lane : i - v * a.ow4;
+            if (v >= a.oh) break;
+            uint32_t gw = 0, d[2] = {0, 0};
+            if (ok) {
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int u = 4 * q + e;
-                        const uint2 tx = make_tap(m[0] * u + m[1] * v + m[2], a.W);
-                        const uint2 ty = make_tap(m[3] * u + m[4] * v + m[5], a.H);
-                        gw |= bilerp(gsrc, a.W, tx.x, ty.x) << (8 * e);
-                        d[e >> 1] |= (uint32_t)__ldg(dsrc + (size_t)ty.y * a.W + tx.y) << (16 * (e & 1));
-                    }
+                for (int e = 0; e < 4; ++e) {
+                    const int u = 4 * q + e;
+                    const uint2 tx = make_tap(m[0] * u + m[1] * v + m[2], a.W);
+                    const uint2 ty = make_tap(m[3] * u + m[4] * v + m[5], a.H);
+                    gw |= bilerp(gsrc, a.W, tx.x, ty.x) << (8 * e);
+                    d[e >> 1] |= (uint32_t)__ldg(dsrc + (size_t)ty.y * a.W + tx.y) << (16 * (e & 1));
                 }
-                store_group(a, ((size_t)k * a.oh + v) * a.ow + 4 * q, 4 * q, gw, d[0], d[1]);
             }
+            store_group(a, ((size_t)k * a.oh + v) * a.ow + 4 * q, 4 * q, gw, d[0], d[1]);
+        }
+    }
+}
+
+// A thread per pixel, its coordinates computed for itself: no taps to make and share first.
+template <bool AFFINE>
+__global__ void __launch_bounds__(kCropThreads) crop_pixel_kernel(const CropArgs a) {
+    const int p = blockIdx.x * kCropThreads + threadIdx.x, v = p / a.ow, u = p - v * a.ow;
+    if (v >= a.oh) return;
+    for (int k = blockIdx.y; k < a.n; k += gridDim.y) {
+        const rgbd_rect r = a.rects[k];
+        const size_t o = (size_t)k * a.oh * a.ow + p;
+        uint32_t g = 0, d = 0;
+        if (r.frame >= 0 && r.frame < a.n_frames && r.w > 0 && r.h > 0) {
+            const int32_t* m = a.affine + 6 * (size_t)k;
+            const int64_t x = AFFINE ? (int64_t)m[0] * u + (int64_t)m[1] * v + m[2] : rect_coord_q16(r.x, r.w, a.ow, u);
+            const int64_t y = AFFINE ? (int64_t)m[3] * u + (int64_t)m[4] * v + m[5] : rect_coord_q16(r.y, r.h, a.oh, v);
+            const uint2 tx = make_tap(x, a.W), ty = make_tap(y, a.H);
+            const size_t base = (size_t)r.frame * a.H * a.W;
+            g = bilerp(a.grey + base, a.W, tx.x, ty.x);
+            d = __ldg(a.depth + base + (size_t)ty.y * a.W + tx.y);
+        } else if (p == 0) {
+            atomicOr(a.status, RGBD_STATUS_BAD_RECT);
+        }
+        a.og[o] = (uint8_t)g;
+        a.od[o] = (uint16_t)d;
     }
 }
 
@@ -167,8 +197,29 @@ int launch_crop_affine(rgbd_ctx* ctx, const uint8_t* grey, const uint16_t* depth
     const dim3 grid((unsigned)((out_h + a.rows - 1) / a.rows), (unsigned)std::min(n, 65535));
     const size_t smem = (((sizeof(uint4) + sizeof(uint32_t)) * 2 * (size_t)a.ow4 + 15) & ~size_t(15)) +
                         sizeof(uint4) * (size_t)a.rows;
-    if (affine) {
-        crop_affine_kernel<<<grid, kCropThreads, 0, s>>>(a);
+    // Few pixels are bound by the chain of steps before the first store, which is shorter with a thread per
+    // pixel, while the chip has threads to spare: up to about 1000 pixels per SM (one 100x100 crop: 3.1 us
+    // in strips, 2.4 us; 40 of 32x32: 3.8 and 2.6 us; 40 of 100x100: 3.8 and 5.5 us).  So are crops of a few
+    // pixels, a CTA each in strips (3000 of 8x8: 10.0 and 4.8 us), and rows of little more than a group,
+    // whose last group is mostly padding (600 of 300x5: 16.6 and 10.4 us).  With an affine map there are no taps
+    // to share, and groups gain less: they need more pixels (40 of 100x100: 5.3 and 5.1 us; 600: 37 and 45
+    // us), and 4-byte stores or long rows (3000 of 33x33: 34 and 30 us; of 300x9: 72 and 68 us).
+    const long long sms = ctx->props.sm_count, px = (long long)n * out_h * out_w;
+    const bool pixels = affine ? px <= 4096 * sms || out_w < 12 || (out_w % 4 != 0 && out_w < 64 && px <= 32768 * sms)
+                               : px <= 1024 * sms || out_h * out_w <= 256 || out_w < 4 ||
+                                     (out_w == 5 && px <= 8192 * sms);
+    if (pixels) {
+        const dim3 cells((unsigned)((out_h * out_w + kCropThreads - 1) / kCropThreads), grid.y);
+        if (affine)
+            crop_pixel_kernel<true><<<cells, kCropThreads, 0, s>>>(a);
+        else
+            crop_pixel_kernel<false><<<cells, kCropThreads, 0, s>>>(a);
+    } else if (affine) {
+        const int steps = a.ow4 % 32 == 0 ? (out_h + kCropThreads / 32 - 1) / (kCropThreads / 32) * (a.ow4 / 32)
+                                          : (out_h * a.ow4 + kCropThreads - 1) / kCropThreads;
+        const int parts = (int)std::min((long long)steps, std::max((steps + 63) / 64LL, (16 * sms + n - 1) / n));
+        a.rows = (steps + parts - 1) / parts;
+        crop_affine_kernel<<<dim3((unsigned)((steps + a.rows - 1) / a.rows), grid.y), kCropThreads, 0, s>>>(a);
     } else {
         // crops up to 4096 columns and rows: 41 KB of column taps and 66 KB of row taps at most
         constexpr size_t most = (sizeof(uint4) + sizeof(uint32_t)) * 2 * 1024 + sizeof(uint4) * 4096;

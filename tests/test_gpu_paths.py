@@ -687,3 +687,34 @@ def test_face_roi_of_a_single_pixel(B, ctx, orc, H):
     for i, f in enumerate(["frame", "x", "y", "w", "h"]):
         assert (got[:, i] == want[f]).all(), f
     assert (want["h"][:H] == 1).all() and want["h"][H] == 0
+
+
+@pytest.mark.parametrize("n,out_h,out_w", [(1, 300, 518), (1, 300, 520), (1, 9, 131072 // 32), (2, 1100, 300), (800, 20, 39),
+                                           (3, 1030, 256), (400, 300, 5), (400, 301, 7), (6000, 16, 16), (6000, 16, 17)])
+def test_crops_of_few_and_of_many_pixels(B, ctx, orc, n, out_h, out_w):
+    """Crops around the sizes where a thread makes one pixel or a group of four, by rect and by affine map, rows
+    of whole warps of groups and others: the oracle's pixels, and zeros for a bad rect."""
+    rng = synth.rng_for(n + out_h + out_w)
+    H, W = 60, 80
+    g = rng.integers(0, 256, (2, H, W)).astype(np.uint8)
+    d = rng.integers(0, 65536, (2, H, W)).astype(np.uint16)
+    r = np.zeros(n, orc.RECT_DTYPE)
+    r["frame"] = rng.integers(0, 2, n)
+    r["x"], r["y"] = rng.integers(-20, W, n), rng.integers(-20, H, n)
+    r["w"], r["h"] = rng.integers(1, 90, n), rng.integers(1, 90, n)
+    if n > 1:
+        r["w"][n - 1] = 0
+    aff = rng.integers(-70000, 70000, (n, 6)).astype(np.int32)
+    aff[:, [2, 5]] *= 30
+    gd, dd, rd = dev_u8(g), dev_u16(d), B.rects_tensor(r)
+    for a in (None, aff):
+        og, od = B.rgbd_crop_affine(ctx, gd, dd, rd, out_h, out_w, affine=None if a is None else torch.from_numpy(a).cuda())
+        for k in {0, n // 2, n - 1}:
+            kg, kd = og[k].cpu().numpy(), host_u16(od[k])
+            if r[k]["w"] == 0:
+                assert not kg.any() and not kd.any()
+                continue
+            wg, wd = orc.crop(g[r[k]["frame"]], d[r[k]["frame"]], tuple(r[k][f] for f in ("x", "y", "w", "h")), out_h, out_w,
+                              affine=None if a is None else a[k])
+            assert (kg == wg).all() and (kd == wd).all(), (k, a is None)
+    assert bool(ctx.status(clear=True) & B.STATUS_BAD_RECT) == (n > 1)
