@@ -42,24 +42,34 @@ X_ELEM = {"f32": 4, "tf32": 4, "bf16": 2, "fp8": 1, "bf16x3": 4}
 # DRAM bytes (read + write) per launch from one ncu capture of the batch workload (the
 # profiles/ summaries give the commands), valid only for the kernel source and launch layout
 # they were taken with: (source file, sha256 prefix of its code, layout key) -> bytes.  The
-# digest covers the source with comments and blank space removed, so only a code change (or a
-# changed layout) reports null.
+# digest covers the source and the device headers it includes (.cuh of the same folder, and theirs)
+# with comments and blank space removed, so only a code change (or a changed layout) reports null.
 MEASURED_TRAFFIC = {
-    "k1": ("lbp.cu", "2aac33549a94894c", "shape2/ctas2/bf16", 189_068_032 + 194_797_568),
-    "k2": ("svm_tc.cu", "de114925748423c5", "splits4/pair/bf16", 616_717_312 + 3_664_128),
+    "k1": ("lbp.cu", "147a1377affb3c26", "shape2/ctas2/bf16", 189_067_520 + 194_768_128),
+    "k2": ("svm_tc.cu", "272e72839d4d3a29", "splits4/pair/bf16", 616_664_064 + 326_656),
 }
 
 
 def code_digest(path):
-    """sha256 prefix of a C/CUDA source with its comments and all blank space removed."""
+    """sha256 prefix of a CUDA source and the .cuh files it includes from its own folder, without their
+    comments and blank space."""
     import hashlib
     import re
-    with open(path, encoding="utf-8") as f:
-        text = f.read()
-    # drop string-free comment forms: /* ... */ and // to the end of the line
-    text = re.sub(r"/\*.*?\*/", "", text, flags=re.S)
-    text = re.sub(r"//[^\n]*", "", text)
-    return hashlib.sha256(re.sub(r"\s+", "", text).encode()).hexdigest()[:16]
+    digest, seen, queue = hashlib.sha256(), set(), [path]
+    while queue:
+        path = queue.pop(0)
+        if path in seen or not os.path.exists(path):
+            continue
+        seen.add(path)
+        with open(path, encoding="utf-8") as f:
+            text = f.read()
+        # drop string-free comment forms: /* ... */ and // to the end of the line
+        text = re.sub(r"/\*.*?\*/", "", text, flags=re.S)
+        text = re.sub(r"//[^\n]*", "", text)
+        digest.update(re.sub(r"\s+", "", text).encode())
+        queue += [os.path.join(os.path.dirname(path), h)
+                  for h in re.findall(r'^\s*#\s*include\s*"([^"]+\.cuh)"', text, flags=re.M)]
+    return digest.hexdigest()[:16]
 
 
 def measured_traffic(stage, layout):

@@ -42,3 +42,24 @@ def test_stored_traffic_needs_the_captured_layout():
         path = os.path.join(ROOT, "paper_1504_01883_gb300", "csrc", fname)
         want = nbytes if bench.code_digest(path) == digest else None
         assert bench.measured_traffic(stage, key) == want
+
+
+def test_code_digest_covers_the_device_headers(tmp_path):
+    """A kernel's arithmetic may live in the headers it includes: a change there changes the digest."""
+    src, taps, inner = tmp_path / "k.cu", tmp_path / "taps.cuh", tmp_path / "inner.cuh"
+    src.write_text('#include <stdint.h>\n#include "taps.cuh"\n#include "missing.cuh"\nint f() { return tap(); }\n')
+    taps.write_text('#pragma once\n#include "inner.cuh"\nint tap() { return inner(); }\n')
+    inner.write_text('#pragma once\n#include "taps.cuh"\nint inner() { return 1; }\n')
+    digests = [bench.code_digest(str(src))]
+    inner.write_text('#pragma once\n#include "taps.cuh"\n// one\nint inner() { return 1; }\n')
+    assert bench.code_digest(str(src)) == digests[0]
+    for header, code in ((taps, "int tap() { return 2 * inner(); }"), (inner, "int inner() { return 2; }")):
+        header.write_text('#include "inner.cuh"\n' + code)
+        digests.append(bench.code_digest(str(src)))
+    assert len(set(digests)) == 3
+
+
+def test_stored_traffic_is_of_the_present_kernels():
+    """The stored figures are those of the code as it is."""
+    for fname, digest, key, nbytes in bench.MEASURED_TRAFFIC.values():
+        assert bench.code_digest(os.path.join(ROOT, "paper_1504_01883_gb300", "csrc", fname)) == digest, fname
