@@ -718,3 +718,73 @@ def test_crops_of_few_and_of_many_pixels(B, ctx, orc, n, out_h, out_w):
                               affine=None if a is None else a[k])
             assert (kg == wg).all() and (kd == wd).all(), (k, a is None)
     assert bool(ctx.status(clear=True) & B.STATUS_BAD_RECT) == (n > 1)
+
+
+def _training_rows(n, k_pad, C, spread):
+    rng = synth.rng_for(n + k_pad)
+    lab = rng.integers(0, C, n).astype(np.int32)
+    x = ((rng.normal(0, 1, (C, k_pad))[lab] + rng.normal(0, spread, (n, k_pad))) / np.sqrt(k_pad)).astype(np.float32)
+    q = (x.astype(np.float64) ** 2).sum(1).astype(np.float32)
+    return lab, x, q
+
+
+def _ascent(x, lab, c, a):
+    """-y G of class c's dual at coefficients a, in fp64 (from the rows with a coefficient alone), y, and how far
+    fp32 may be from it after `steps` steps."""
+    x64 = x.astype(np.float64)
+    y = np.where(lab == c, 1.0, -1.0)
+    sv = np.flatnonzero(a)
+    d2 = (x64 ** 2).sum(1)[:, None] + (x64[sv] ** 2).sum(1)[None, :] - 2 * x64 @ x64[sv].T
+    v = y - np.exp(-np.maximum(d2, 0)) @ a[sv]
+    # every step rounds a row's value once; a kernel value is off by the fp32 rounding of its distance (norms and
+    # a chain of k_pad products) and of its exponential
+    off_k = (x.shape[1] + 4) * 2.0 ** -24 * 4 * (x64 ** 2).sum(1).max() + 4 * 2.0 ** -24
+    return v, y, lambda steps: steps * 2.0 ** -24 * 4 + np.abs(a).sum() * off_k
+
+
+@pytest.mark.parametrize("n,k_pad", [(300, 48), (2100, 48), (2300, 50)])
+def test_training_converges_to_the_optimum(B, ctx, n, k_pad):
+    """Trained to the stopping gap, in tiles of a CTA each and in tiles handed from CTA to CTA: the optimality
+    conditions hold in fp64 for every row of every class, which takes the kernel values between all support
+    vectors and all rows; the bias is the mean over the free vectors."""
+    C, eps = 3, 1e-2
+    lab, x, q = _training_rows(n, k_pad, C, 0.9)
+    coef, bias, iters = B.svm_train_rbf(ctx, dev_f32(x), dev_f32(q), torch.from_numpy(lab).cuda(), C, 1.0, 1.0, eps,
+                                        max_iter=200000)
+    assert ctx.status() == 0
+    for c in range(C):
+        a, it = coef[c].cpu().numpy().astype(np.float64), int(iters[c])
+        assert 10 < it < 200000
+        v, y, off = _ascent(x, lab, c, a)
+        alpha, tol = a * y, off(it)
+        assert (alpha >= 0).all() and (alpha <= 1).all() and abs(a.sum()) <= it * 2.0 ** -23
+        up = np.where(y > 0, alpha < 1, alpha > 0)
+        low = np.where(y > 0, alpha > 0, alpha < 1)
+        assert v[up].max() - v[low].min() <= eps + 2 * tol, (c, tol)
+        free = (alpha > 0) & (alpha < 1)
+        assert free.any() and abs(float(bias[c]) - v[free].mean()) <= tol + 1e-6
+
+
+@pytest.mark.parametrize("n", [256, 257, 1024, 1025, 2048, 2049, 4096, 4097, 8192, 8193])
+def test_training_steps_take_the_most_violating_pair(B, ctx, n):
+    """Around the row counts where the threads and the rows per thread change: the pair that step s + 1 moves
+    (the coefficients after s + 1 steps against those after s) is the most violating one after s, in fp64."""
+    C, k_pad = 2, 32
+    lab, x, q = _training_rows(n, k_pad, C, 0.9)
+    lab[-1], lab[0] = 0, 1
+    args = (dev_f32(x), dev_f32(q), torch.from_numpy(lab).cuda(), C, 1.0, 1.0, 1e-6)
+    for s in (0, 1, 2, 7, 40):
+        a0, _, i0 = B.svm_train_rbf(ctx, *args, max_iter=s)
+        a1, _, i1 = B.svm_train_rbf(ctx, *args, max_iter=s + 1)
+        assert (i0 == s).all() and (i1 == s + 1).all()
+        for c in range(C):
+            a, b = a0[c].cpu().numpy().astype(np.float64), a1[c].cpu().numpy().astype(np.float64)
+            v, y, off = _ascent(x, lab, c, a)
+            up = np.where(y > 0, a < 1, a < 0)
+            low = np.where(y > 0, a > 0, a > -1)
+            moved = np.flatnonzero(a != b)
+            assert len(moved) == 2 and (b[moved] - a[moved]).sum() <= 2.0 ** -22
+            i, j = moved if b[moved[0]] > a[moved[0]] else moved[::-1]  # a grows by i's step, falls by j's
+            assert up[i] and low[j]
+            assert v[i] >= v[up].max() - 2 * off(s) and v[j] <= v[low].min() + 2 * off(s)
+    assert ctx.status() == 0
