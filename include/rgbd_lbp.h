@@ -510,7 +510,7 @@ int rgbd_server_destroy(rgbd_server* s);
 
 /* rgbd_debug_expm1 -- evaluates, for a test, the e^z - 1 the tensor-core RBF epilogue uses
  * (Section 2.5's kernel value relative to a reference distance, where |z| is small): a
- * degree-6 Taylor polynomial for |z| < 2^-5, expm1f otherwise.
+ * degree-9 Taylor polynomial for |z| < 1/2, expm1f otherwise.
  *   z, out   device fp32 [n] (caller-owned); out[i] = e^z[i] - 1.
  *   Asynchronous on stream.  Errors: RGBD_ERR_ARG for n < 0 or NULL pointers with n > 0. */
 int rgbd_debug_expm1(const float* z, float* out, int n, void* stream);

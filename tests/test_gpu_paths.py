@@ -788,3 +788,19 @@ def test_training_steps_take_the_most_violating_pair(B, ctx, n):
             assert up[i] and low[j]
             assert v[i] >= v[up].max() - 2 * off(s) and v[j] <= v[low].min() + 2 * off(s)
     assert ctx.status() == 0
+
+
+def test_epilogue_expm1_up_to_its_switch(B):
+    """The series of the epilogue's e^z - 1 reaches to 1/2: within 2 ulp of the exact value (3 of CUDA's expm1f)
+    densely from 1/32 to 1/2 and on both sides of the switch."""
+    rng = np.random.default_rng(6)
+    half = np.float32(0.5)
+    z = np.concatenate([rng.uniform(0.03, 0.5, 300000), np.linspace(0.499, 0.501, 4001),
+                        [half, np.nextafter(half, np.float32(0)), np.nextafter(half, np.float32(1))]]).astype(np.float32)
+    z = np.concatenate([z, -z])
+    zt = torch.from_numpy(z).cuda()
+    ours, cuda = B.rgbd_debug_expm1(zt).cpu().numpy().astype(np.float64), torch.expm1(zt).cpu().numpy().astype(np.float64)
+    exact = np.expm1(z.astype(np.float64))
+    ulp = np.spacing(np.abs(exact).astype(np.float32)).astype(np.float64)
+    assert np.max(np.abs(ours - exact) / ulp) <= 2.0
+    assert np.max(np.abs(ours - cuda) / ulp) <= 3.0
