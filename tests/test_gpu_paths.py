@@ -804,3 +804,27 @@ def test_epilogue_expm1_up_to_its_switch(B):
     ulp = np.spacing(np.abs(exact).astype(np.float32)).astype(np.float64)
     assert np.max(np.abs(ours - exact) / ulp) <= 2.0
     assert np.max(np.abs(ours - cuda) / ulp) <= 3.0
+
+
+@pytest.mark.parametrize("C", [1, 2, 63, 64, 65, 128])
+@pytest.mark.parametrize("n", [129, 130, 131, 132])
+def test_split_combine_of_few_and_many_classes(B, ctx, orc, C, n):
+    """The combine takes up to four rows to a block, fewer for more classes: a last block of one to four rows,
+    against fp64, and the same bits as a warp per row gives (a batch of more than 1024 rows)."""
+    rng = synth.rng_for(C + n)
+    n_sv, dim = 700, 9 * 59
+    X, SV = synth.poisson_counts(rng, 1025, dim), synth.poisson_counts(rng, n_sv, dim)
+    a = rng.normal(0, 1, (C, n_sv)).astype(np.float32)
+    b = rng.normal(0, 0.01, C).astype(np.float32)
+    model = B.svm_train_data_pack(ctx, dev_u16(SV), dev_f32(a), dev_f32(b), gamma=1.0 / dim, dtype="bf16")
+    ctx.set_tuning(B.TUNE_TC_SPLITS, 3)
+    try:
+        x, q = B.lbp_normalize_features(ctx, dev_u16(X), "bf16")
+        big, lbig = B.svm_score(ctx, model, x, q)
+        s, lab = B.svm_score(ctx, model, x[:n].contiguous(), q[:n].contiguous())
+    finally:
+        ctx.set_tuning(B.TUNE_TC_SPLITS, 0)
+    assert ctx.status() == 0 and torch.equal(s, big[:n]) and torch.equal(lab, lbig[:n])
+    x64, sv64 = orc.normalize_f64(X[:n]), orc.normalize_f64(SV)
+    ref = orc.svm_rbf(x64, sv64, a, b, 1.0 / dim)
+    assert rel_score_error(s.cpu().numpy(), ref, rbf_error_scale(x64, sv64, a, b, 1.0 / dim)) <= 5e-5
