@@ -828,3 +828,42 @@ def test_split_combine_of_few_and_many_classes(B, ctx, orc, C, n):
     x64, sv64 = orc.normalize_f64(X[:n]), orc.normalize_f64(SV)
     ref = orc.svm_rbf(x64, sv64, a, b, 1.0 / dim)
     assert rel_score_error(s.cpu().numpy(), ref, rbf_error_scale(x64, sv64, a, b, 1.0 / dim)) <= 5e-5
+
+
+@pytest.mark.parametrize("gamma", [0.02, 0.06, 0.12, 0.3, 1.0])
+@pytest.mark.parametrize("dt", ["bf16", "bf16x3"])
+def test_tile_scores_on_both_sides_of_the_series(B, ctx, orc, gamma, dt):
+    """The tile kernel's e^z - 1 is a polynomial up to |z| = 0.35: gammas for which all, some and few of the
+    arguments lie below, against fp64 of the stored values.  F and the coefficients are rounded to bf16 (to pairs
+    of them), relative to the mean distance of the split."""
+    rng = synth.rng_for(int(100 * gamma))
+    n, n_sv, dim, C = 150, 500, 64 * 59, 9
+    X, SV = rng.poisson(2, (n, dim)).astype(np.uint16), rng.poisson(2, (n_sv, dim)).astype(np.uint16)
+    SV[::3] = (SV[::3] * rng.integers(0, 2, (len(SV[::3]), dim))).astype(np.uint16)  # distances of several kinds
+    a = rng.normal(0, 1, (C, n_sv)).astype(np.float32)
+    b = rng.normal(0, 0.01, C).astype(np.float32)
+    model = B.svm_train_data_pack(ctx, dev_u16(SV), dev_f32(a), dev_f32(b), gamma=gamma, dtype=dt)
+    x, q = B.lbp_normalize_features(ctx, dev_u16(X), dt)
+    s, lab = B.svm_score(ctx, model, x, q)
+    assert ctx.status() == 0
+
+    def held(counts):
+        v = torch.from_numpy(orc.normalize_f32(counts))
+        hi = v.bfloat16()
+        return (hi.double() + ((v - hi.float()).bfloat16().double() if dt == "bf16x3" else 0)).numpy()
+
+    x64, sv64 = held(X), held(SV)
+    xx, ss, g = (x64 ** 2).sum(1)[:, None], (sv64 ** 2).sum(1)[None, :], x64 @ sv64.T
+    d2 = np.maximum(xx + ss - 2 * g, 0)
+    K = np.exp(-gamma * d2)
+    ref = K @ a.astype(np.float64).T + b
+    z = gamma * np.abs(d2 - d2.mean(1, keepdims=True)).max(1, keepdims=True)
+    # F and the coefficient are each rounded to u = 2^-9 (2^-17 as pairs) of themselves, F at most e^z - 1; a
+    # distance is off by the products' fp32 sums (taken as 256 roundings; a pair's lo * lo product, 2^-18 of g, is left
+    # out), the rest by fp32
+    u = 2.0 ** -9 if dt == "bf16" else 2.0 ** -17
+    off = gamma * (256 * 2.0 ** -24 * (xx + ss + 2 * g) + (2.0 ** -16 * g if dt == "bf16x3" else 0))
+    absa = np.abs(a.astype(np.float64)).T
+    tol = np.exp(-gamma * d2.min(1, keepdims=True)) * (2.1 * u * np.expm1(z) + 1e-6) * absa.sum(0) + (K * np.expm1(off)) @ absa
+    assert (np.abs(s.cpu().numpy() - ref) <= tol).all()
+    assert (lab.cpu().numpy() == s.cpu().numpy().argmax(1)).all()
