@@ -112,14 +112,15 @@ __global__ void __launch_bounds__(kCropThreads) crop_rect_kernel(const CropArgs 
     }
 }
 
-// A general affine map: source points by 64-bit products per pixel, a thread per group of 4 columns; a step
-// of a CTA is 8 rows of 32 groups where a row is whole warps, else 256 groups in a row, and a CTA takes
-// a.rows steps, so that neighbouring rows meet in its L1.  Bound by the products and the gathers.  600 maps
-// to 128x128: 74 us a thread per pixel, 57 us now; to 100x100 (25 groups a row) 48 and 37 us.
+// A general affine map: source points by 64-bit products per pixel, a thread per group of 4 columns.  ROWS (where a
+// row is whole warps of groups): a warp per crop row, a strip of a.rows rows per CTA; else a crop's groups in a row,
+// a.rows steps of 256 per CTA.  Either way neighbouring rows meet in a CTA's L1.  Bound by the products and the
+// gathers.  600 maps to 128x128: 74 us a thread per pixel, 62 us now; to 100x100 (25 groups a row) 48 and 37 us (a warp
+// per row there: 47 us; groups in a row at 512x512: 5 % slower).
+template <bool ROWS>
 __global__ void __launch_bounds__(kCropThreads) crop_affine_kernel(const CropArgs a) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int per_row = a.ow4 / 32;  // of whole warps: a step is 8 rows of 32 groups
-    const bool tiled = a.ow4 % 32 == 0;
+    const int lpr = 1 << a.lanes_log2;  // 32 for ROWS (as a constant: 40 maps to 512x512 in 56 us instead of 51)
     for (int k = blockIdx.y; k < a.n; k += gridDim.y) {
         const rgbd_rect r = a.rects[k];
         const bool ok = r.frame >= 0 && r.frame < a.n_frames && r.w > 0 && r.h > 0;
@@ -129,23 +130,30 @@ __global__ void __launch_bounds__(kCropThreads) crop_affine_kernel(const CropArg
             for (int i = 0; i < 6; ++i) m[i] = __ldg(a.affine + 6 * (size_t)k + i);
         const uint8_t* gsrc = a.grey + (ok ? (size_t)r.frame * a.H * a.W : 0);
         const uint16_t* dsrc = a.depth + (ok ? (size_t)r.frame * a.H * a.W : 0);
-        for (int st = blockIdx.x * a.rows; st < (int)(blockIdx.x + 1) * a.rows; ++st) {
-            const int i = st * kCropThreads + threadIdx.x;
-            const int v = tiled ? st / per_row * (kCropThreads / 32) + warp : i / a.ow4;
-            const int q = tiled ? st % per_row * 32 + lane : i - v * a.ow4;
-            if (v >= a.oh) break;
+        auto group = [&](int v, int q, int64_t xv, int64_t yv) {  // xv, yv: the row's share of the source point
             uint32_t gw = 0, d[2] = {0, 0};
             if (ok) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const int u = 4 * q + e;
-                    const uint2 tx = make_tap(m[0] * u + m[1] * v + m[2], a.W);
-                    const uint2 ty = make_tap(m[3] * u + m[4] * v + m[5], a.H);
+                    const uint2 tx = make_tap(m[0] * u + xv, a.W);
+                    const uint2 ty = make_tap(m[3] * u + yv, a.H);
                     gw |= bilerp(gsrc, a.W, tx.x, ty.x) << (8 * e);
                     d[e >> 1] |= (uint32_t)__ldg(dsrc + (size_t)ty.y * a.W + tx.y) << (16 * (e & 1));
                 }
             }
             store_group(a, ((size_t)k * a.oh + v) * a.ow + 4 * q, 4 * q, gw, d[0], d[1]);
+        };
+        if (ROWS) {
+            const int v0 = blockIdx.x * a.rows, v1 = min(a.oh, v0 + a.rows);
+            for (int v = v0 + warp; v < v1; v += kCropThreads / 32)
+                for (int q = lane; q < a.ow4; q += lpr) group(v, q, m[1] * v + m[2], m[4] * v + m[5]);
+        } else {
+            const int i0 = blockIdx.x * a.rows * kCropThreads, i1 = min(a.oh * a.ow4, i0 + a.rows * kCropThreads);
+            for (int i = i0 + threadIdx.x; i < i1; i += kCropThreads) {
+                const int v = i / a.ow4;
+                group(v, i - v * a.ow4, m[1] * v + m[2], m[4] * v + m[5]);
+            }
         }
     }
 }
@@ -205,7 +213,7 @@ int launch_crop_affine(rgbd_ctx* ctx, const uint8_t* grey, const uint16_t* depth
     // to share, and groups gain less: they need more pixels (40 of 100x100: 5.3 and 5.1 us; 600: 37 and 45
     // us), and 4-byte stores or long rows (3000 of 33x33: 34 and 30 us; of 300x9: 72 and 68 us).
     const long long sms = ctx->props.sm_count, px = (long long)n * out_h * out_w;
-    const bool pixels = affine ? px <= 4096 * sms || out_w < 12 || (out_w % 4 != 0 && out_w < 64 && px <= 32768 * sms)
+    const bool pixels = affine ? px <= 3072 * sms || out_w < 12 || (out_w % 4 != 0 && out_w < 64 && px <= 32768 * sms)
                                : px <= 1024 * sms || out_h * out_w <= 256 || out_w < 4 ||
                                      (out_w == 5 && px <= 8192 * sms);
     if (pixels) {
@@ -215,11 +223,14 @@ int launch_crop_affine(rgbd_ctx* ctx, const uint8_t* grey, const uint16_t* depth
         else
             crop_pixel_kernel<false><<<cells, kCropThreads, 0, s>>>(a);
     } else if (affine) {
-        const int steps = a.ow4 % 32 == 0 ? (out_h + kCropThreads / 32 - 1) / (kCropThreads / 32) * (a.ow4 / 32)
-                                          : (out_h * a.ow4 + kCropThreads - 1) / kCropThreads;
-        const int parts = (int)std::min((long long)steps, std::max((steps + 63) / 64LL, (16 * sms + n - 1) / n));
-        a.rows = (steps + parts - 1) / parts;
-        crop_affine_kernel<<<dim3((unsigned)((steps + a.rows - 1) / a.rows), grid.y), kCropThreads, 0, s>>>(a);
+        if (a.ow4 % 32 == 0) {
+            crop_affine_kernel<true><<<grid, kCropThreads, 0, s>>>(a);
+        } else {
+            const int steps = (out_h * a.ow4 + kCropThreads - 1) / kCropThreads;
+            const int parts = (int)std::min((long long)steps, std::max((steps + 63) / 64LL, (16 * sms + n - 1) / n));
+            a.rows = (steps + parts - 1) / parts;
+            crop_affine_kernel<false><<<dim3((unsigned)((steps + a.rows - 1) / a.rows), grid.y), kCropThreads, 0, s>>>(a);
+        }
     } else {
         // crops up to 4096 columns and rows: 41 KB of column taps and 66 KB of row taps at most
         constexpr size_t most = (sizeof(uint4) + sizeof(uint32_t)) * 2 * 1024 + sizeof(uint4) * 4096;
