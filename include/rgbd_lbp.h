@@ -325,7 +325,9 @@ int rgbd_svm_centre(const rgbd_svm* model, const float** centre);
  * score up to 128 rows by splitting the SV tiles' K extent over several CTAs
  * (two launches, the second a programmatic dependent of the first) when the
  * tiles alone would occupy few SMs (RGBD_TUNE_TC_SPLITK); larger batches by SV
- * tiles.  The two paths round differently within the model type's tolerance.
+ * tiles.  The two paths round differently within the model type's tolerance.  Scores by SV
+ * tiles are summed relative to a mean distance, and are NaN for a row where
+ * gamma x (that mean - the squared distance to a support vector) exceeds about 88.
  * Errors: RGBD_ERR_ARG, RGBD_ERR_UNSUPPORTED, RGBD_ERR_NOMEM, RGBD_ERR_CUDA. */
 int svm_score(rgbd_ctx* ctx, const rgbd_svm* model, const void* x, const float* xsq, int n,
               float x_scale, float* scores, int32_t* labels, void* stream);
@@ -508,7 +510,7 @@ int rgbd_server_destroy(rgbd_server* s);
 /* Diagnostics                                                                              */
 /* ======================================================================================= */
 
-/* rgbd_debug_expm1 -- evaluates, for a test, the e^z - 1 the tensor-core RBF epilogue uses
+/* rgbd_debug_expm1 -- evaluates, for a test, the e^z - 1 the few-row RBF epilogue uses
  * (Section 2.5's kernel value relative to a reference distance, where |z| is small): a
  * degree-9 Taylor polynomial for |z| < 1/2, expm1f otherwise.
  *   z, out   device fp32 [n] (caller-owned); out[i] = e^z[i] - 1.
