@@ -21,6 +21,7 @@ struct CropArgs {
     int ow4;        // groups of 4 columns
     int rows;       // crop rows per CTA
     int lanes_log2; // lanes of a warp on one row
+    int narrow;     // the padding of a row's last group is a fifth of it or more
     int wide;       // 4-byte grey and 8-byte depth stores are aligned
     uint8_t* og;
     uint16_t* od;
@@ -103,7 +104,21 @@ __global__ void __launch_bounds__(kCropThreads) crop_rect_kernel(const CropArgs 
                 }
             }
         };
-        if (win == WIN_GROUP)
+        if (win == WIN_NONE && a.narrow) {
+            // without windows a pixel costs its own loads, the padding's too: a thread per pixel on the same taps
+            // (3000 rects of side 48..256 to 300x5: 53 us in groups, 26 us; to 300x9 66 and 35 us)
+            for (int p = tid; p < (v1 - v0) * a.ow; p += kCropThreads) {
+                const int v = p / a.ow, u = p - v * a.ow, at = ((u >> 1) & 1) * a.ow4 + (u >> 2);
+                const uint4 c = cm[at], ry = rm[v];
+                const uint32_t t = u & 1 ? c.z : c.x, near = u & 1 ? nn[at] >> 16 : nn[at] & 0xFFFFu;
+                const uint32_t xa = t & 0xFFFFu, dx = (t >> 16) & 1u, fx = t >> 24, fy = ry.w;
+                const uint32_t h0 = (256u - fx) * __ldg(gsrc + ry.x + xa) + fx * __ldg(gsrc + ry.x + xa + dx);
+                const uint32_t h1 = (256u - fx) * __ldg(gsrc + ry.y + xa) + fx * __ldg(gsrc + ry.y + xa + dx);
+                const size_t o = crop0 + (size_t)v0 * a.ow + p;
+                a.og[o] = (uint8_t)((h0 * (256u - fy) + h1 * fy + 32768u) >> 16);
+                a.od[o] = __ldg(dsrc + ry.z + near);
+            }
+        } else if (win == WIN_GROUP)
             rows(std::integral_constant<int, WIN_GROUP>{});
         else if (win == WIN_PAIR)
             rows(std::integral_constant<int, WIN_PAIR>{});
@@ -192,6 +207,7 @@ int launch_crop_affine(rgbd_ctx* ctx, const uint8_t* grey, const uint16_t* depth
     a.grey = grey, a.depth = depth, a.n_frames = n_frames, a.H = H, a.W = W, a.rects = rects, a.affine = affine;
     a.n = n, a.oh = out_h, a.ow = out_w, a.og = og, a.od = od, a.status = ctx->d_status;
     a.ow4 = (out_w + 3) / 4;
+    a.narrow = 5 * out_w <= 16 * a.ow4;
     a.lanes_log2 = 0;
     while (a.lanes_log2 < 5 && (1 << a.lanes_log2) < a.ow4) ++a.lanes_log2;
     a.wide = out_w % 4 == 0 && (reinterpret_cast<uintptr_t>(og) & 3) == 0 && (reinterpret_cast<uintptr_t>(od) & 7) == 0;
@@ -208,14 +224,12 @@ int launch_crop_affine(rgbd_ctx* ctx, const uint8_t* grey, const uint16_t* depth
     // Few pixels are bound by the chain of steps before the first store, which is shorter with a thread per
     // pixel, while the chip has threads to spare: up to about 1000 pixels per SM (one 100x100 crop: 3.1 us
     // in strips, 2.4 us; 40 of 32x32: 3.8 and 2.6 us; 40 of 100x100: 3.8 and 5.5 us).  So are crops of a few
-    // pixels, a CTA each in strips (3000 of 8x8: 10.0 and 4.8 us), and rows of little more than a group,
-    // whose last group is mostly padding (600 of 300x5: 16.6 and 10.4 us).  With an affine map there are no taps
+    // pixels, a CTA each in strips (3000 of 8x8: 10.1 and 4.9 us).  With an affine map there are no taps
     // to share, and groups gain less: they need more pixels (40 of 100x100: 5.3 and 5.1 us; 600: 37 and 45
     // us), and 4-byte stores or long rows (3000 of 33x33: 34 and 30 us; of 300x9: 72 and 68 us).
     const long long sms = ctx->props.sm_count, px = (long long)n * out_h * out_w;
     const bool pixels = affine ? px <= 3072 * sms || out_w < 12 || (out_w % 4 != 0 && out_w < 64 && px <= 32768 * sms)
-                               : px <= 1024 * sms || out_h * out_w <= 256 || out_w < 4 ||
-                                     (out_w == 5 && px <= 8192 * sms);
+                               : px <= 1024 * sms || out_h * out_w <= 256;
     if (pixels) {
         const dim3 cells((unsigned)((out_h * out_w + kCropThreads - 1) / kCropThreads), grid.y);
         if (affine)
