@@ -867,3 +867,24 @@ def test_tile_scores_on_both_sides_of_the_series(B, ctx, orc, gamma, dt):
     tol = np.exp(-gamma * d2.min(1, keepdims=True)) * (2.1 * u * np.expm1(z) + 1e-6) * absa.sum(0) + (K * np.expm1(off)) @ absa
     assert (np.abs(s.cpu().numpy() - ref) <= tol).all()
     assert (lab.cpu().numpy() == s.cpu().numpy().argmax(1)).all()
+
+
+@pytest.mark.parametrize("w,h", [(1, 90), (90, 1), (13, 17), (59, 60), (60, 60), (61, 59), (60, 61), (90, 91), (30, 129)])
+@pytest.mark.parametrize("density", [0.001, 0.1, 1.0])
+def test_face_roi_of_small_and_large_windows(B, ctx, orc, w, h, density):
+    """Windows around the size up to which every pixel is read (4096, with the margins at the sides), down to
+    single rows and columns, nearly empty to full."""
+    rng = synth.rng_for(100 * w + h + int(1000 * density))
+    H, W, n = 140, 150, 24
+    depth = rng.integers(700, 1300, (3, H, W)).astype(np.uint16)
+    depth[rng.random((3, H, W)) >= density] = 0
+    boxes = np.zeros(n, orc.RECT_DTYPE)
+    boxes["frame"], boxes["w"], boxes["h"] = rng.integers(0, 3, n), w, h
+    boxes["x"], boxes["y"] = rng.integers(0, W - w + 1, n), rng.integers(0, H - h + 1, n)
+    cal = synth.calibration(rng, W, H)
+    cal["a"][:] = [65536, 0, 0, 0, 65536, 0]
+    cal["parallax"] = 0
+    want = orc.face_roi(depth, cal, boxes)
+    got = B.rgbd_face_roi(ctx, dev_u16(depth), B.Calib.from_record(cal), B.rects_tensor(boxes)).cpu().numpy()
+    for i, f in enumerate(["frame", "x", "y", "w", "h"]):
+        assert (got[:, i] == want[f]).all(), f
