@@ -51,7 +51,7 @@ __device__ __forceinline__ void store_group(const CropArgs& a, size_t o, int u, 
 // the crop the whole group does) and each horizontal interpolation is a byte permute and a 4-way
 // byte dot product.  Bound by the gathers through L1,
 // with HBM behind (frames in once, crops out once).  4096 rects of side 48..256 over 256 frames
-// of 640x480 -> 128x128: 570 us with a thread and two divisions per pixel, 104 us now.
+// of 640x480 -> 128x128: 570 us with a thread and two divisions per pixel, 98 us now.
 __global__ void __launch_bounds__(kCropThreads) crop_rect_kernel(const CropArgs a) {
     extern __shared__ __align__(16) unsigned char crop_smem[];
     uint4* cm = reinterpret_cast<uint4*>(crop_smem);                  // [2][ow4]: taps of a column pair
@@ -89,8 +89,8 @@ __global__ void __launch_bounds__(kCropThreads) crop_rect_kernel(const CropArgs 
             }
         }
         __syncthreads();
-        // a loop per kind of window, rolled: 104 us, against 107 us unrolled twice (113 us with the kind
-        // tested inside), 114 us four times
+        // a loop per kind of window, rolled: 104 us when it was made so, against 107 us unrolled twice (113 us
+        // with the kind tested inside), 114 us four times
         auto rows = [&](auto mode) {
             constexpr int M = decltype(mode)::value;
 #pragma unroll 1

@@ -94,8 +94,8 @@ struct RoiWindow {
 // and the columns that only a nearer surface could have reached) instead of the area.  What is left is a chain of few L2 or DRAM round trips, so
 // each step issues all its loads first (two rows of the window per warp, 16 rows of a column).
 // 4096 boxes over 256 frames of 640x480, faces of side 48..256: 640 us when every window pixel was
-// tested with a division, 95 us with the scan from the edges, 86 us since rows that cannot meet the box
-// are passed over and what all faces share comes from the host.
+// tested with a division, 95 us with the scan from the edges, 84 us since rows that cannot meet the box
+// are passed over, what all faces share comes from the host, and small windows are read in full.
 template <typename T>
 __global__ void __launch_bounds__(kRoiThreads) face_roi_kernel(const uint16_t* __restrict__ depth, int n_frames, int H,
                                                                int W, rgbd_calib c, RoiWindow wd,
